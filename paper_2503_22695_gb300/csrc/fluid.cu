@@ -31,6 +31,7 @@
 #include <cstring>
 
 #include "ib_device.cuh"
+#include "spectral.cuh"
 
 struct ib_fluid {
   int precision;
@@ -56,12 +57,16 @@ struct ib_fluid {
   cudaGraphExec_t gexec;
   const void* gkey[4];
   int gcyc[2];
+  // the direct solve (spectral.cu), where the lattice has one
+  bool direct;
+  ibfe::Spectral spec;
 };
 
 namespace ibfe {
 namespace {
 
 constexpr int kFluidRedCTAs = 1024;  // first-level reduction CTAs
+constexpr int kCycH32 = 2, kCycP32 = 6;  // default V-cycles, FP32
 constexpr int kCoarseMax = 8;        // coarsest level: every dimension <= 8 (or odd)
 constexpr int kCoarseCells = 8192;   // shared-memory limit of the coarsest solve
 
@@ -532,7 +537,42 @@ ib_status step_direct(ib_fluid* fl, const void* u, const void* f, void* un, void
 }
 }  // namespace
 
-// Advance the fluid one step (internal entry shared with ib_step).  Without
+// The direct solve (spectral.cu) replaces the V-cycles wherever the lattice
+// has one and the cycle counts are the defaults: it gives the discrete
+// solution that the cycles approach, to FP32 rounding, in five launches.  A
+// caller who sets other counts asks for that many V-cycles and gets them.
+namespace {
+bool use_direct(const ib_fluid* fl) {
+  return fl->direct && fl->cyc_h == kCycH32 && fl->cyc_p == kCycP32;
+}
+
+// With residuals, u is kept aside (u_next may alias it) and the increment is
+// left in the solver's workspace for the residual pass (synchronises s).
+ib_status step_spectral(ib_fluid* fl, const float* u, const float* f, float* un, float* p,
+                        double* residuals, cudaStream_t s) {
+  float* u0 = static_cast<float*>(fl->rhs0);
+  const size_t bytes = 3 * sizeof(float) * (size_t)fl->n[0] * fl->n[1] * fl->n[2];
+  if (residuals && !ok(cudaMemcpyAsync(u0, u, bytes, cudaMemcpyDeviceToDevice, s)))
+    return IB_ERR_CUDA;
+  const ib_status st = spectral_step(&fl->spec, u, f, un, p, residuals != nullptr, s);
+  if (st != IB_OK || !residuals) return st;
+  constexpr int kCtas = kFluidRedCTAs / 4;
+  double* out = fl->red + 4 * kCtas;
+  launch_spectral_resid(&fl->spec, u0, f, p, fl->rho / fl->dt, fl->mu / (fl->h * fl->h),
+                        fl->dt / fl->h, fl->red, kCtas, s);
+  k_sums_l2<<<1, 256, 0, s>>>(fl->red, kCtas, 4, out, 1.0);
+  double r[4] = {0.0, 0.0, 0.0, 0.0};
+  if (!ok(cudaMemcpyAsync(r, out, sizeof(r), cudaMemcpyDeviceToHost, s)) ||
+      !ok(cudaStreamSynchronize(s)))
+    return IB_ERR_CUDA;
+  for (int k = 0; k < 2; ++k)
+    residuals[k] = r[2 * k + 1] > 0.0 ? std::sqrt(r[2 * k] / r[2 * k + 1]) : std::sqrt(r[2 * k]);
+  return IB_OK;
+}
+}  // namespace
+
+// Advance the fluid one step (internal entry shared with ib_step).  V-cycles
+// without
 // residuals (which need host round trips) the step's ~300 launches run as
 // one CUDA graph, captured on the solver's own stream the first time a set
 // of field pointers is seen; a caller's stream that is itself being
@@ -540,6 +580,9 @@ ib_status step_direct(ib_fluid* fl, const void* u, const void* f, void* un, void
 ib_status fluid_step_async(ib_fluid* fl, const void* u, const void* f, void* u_next, void* p,
                            double* residuals, cudaStream_t s) {
   void* pp = p ? p : fl->ptmp;
+  if (use_direct(fl))
+    return step_spectral(fl, (const float*)u, (const float*)f, (float*)u_next, (float*)pp,
+                         residuals, s);
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (residuals || !ok(cudaStreamIsCapturing(s, &cs)) || cs != cudaStreamCaptureStatusNone)
     return step_direct(fl, u, f, u_next, pp, residuals, s);
@@ -612,8 +655,8 @@ ib_status ib_fluid_create(const ib_grid* grid, int32_t precision, double rho, do
   fl->dt = dt;
   // V-cycles that reach the rounding floor of each precision on the
   // workloads of the tests (FP32: relative residuals ~1e-7 and ~1e-6)
-  fl->cyc_h = precision == IB_FP64 ? 3 : 2;
-  fl->cyc_p = precision == IB_FP64 ? 12 : 6;
+  fl->cyc_h = precision == IB_FP64 ? 3 : ibfe::kCycH32;
+  fl->cyc_p = precision == IB_FP64 ? 12 : ibfe::kCycP32;
   fl->pre = 2;
   fl->post = 2;
   fl->coarse_sweeps = 20;
@@ -673,6 +716,14 @@ ib_status ib_fluid_create(const ib_grid* grid, int32_t precision, double rho, do
     ib_fluid_destroy(fl);
     return IB_ERR_CUDA;
   }
+  // without room for its workspace the V-cycles serve every step
+  if (precision != IB_FP64 && spectral_supports(fl->n)) {
+    fl->direct = spectral_create(&fl->spec, fl->n, fl->h, rho, mu, dt) == IB_OK;
+    if (!fl->direct) {
+      spectral_destroy(&fl->spec);
+      cudaGetLastError();
+    }
+  }
   (void)stream;
   *out = fl;
   return IB_OK;
@@ -682,6 +733,7 @@ ib_status ib_fluid_destroy(ib_fluid* fl) {
   if (!fl) return IB_ERR_INVALID_ARG;
   if (fl->gexec) cudaGraphExecDestroy(fl->gexec);
   if (fl->cap) cudaStreamDestroy(fl->cap);
+  spectral_destroy(&fl->spec);
   cudaFree(fl->rhs0);
   cudaFree(fl->div);
   cudaFree(fl->ptmp);

@@ -1,0 +1,880 @@
+// Direct solve of the fluid step (Section 4.2) on the periodic MAC grid, FP32.
+//
+// On a periodic lattice the Helmholtz and Poisson operators of Chorin's
+// projection are circulant, so one discrete Fourier transform diagonalises
+// the whole step.  It is solved for the increment w = u^{n+1} - u^n:
+//   (a - mu Lap_h) d = f + mu Lap_h u^n                 (a = rho / dt, u* = u^n + d)
+//   Lap_h p = (div_h u^n + div_h d) / dt
+//   w = d - dt grad_h p
+// The four right-hand fields r_c = f_c + mu Lap_h u_c (c = 0..2) and
+// r_3 = h div_h u^n are formed from the stencils in FP32 before the transform:
+// div_h u is a difference of neighbours (no cancellation against transformed
+// velocities, whose rounding would enter p multiplied by |u| / dt), and the
+// transform's rounding is relative to the increment, not to u.
+// With the forward-difference symbols D_d = exp(2 pi i k_d / n_d) - 1 and
+// S = sum_d |D_d|^2, per mode
+//   d_c = r_c / (a + mu S / h^2),   q = (r_3 + sum_d D_d d_d) / S   (0 at k = 0),
+//   w_c = d_c - conj(D_c) q,        p = -(h / dt) q.
+//
+// Five kernels, all bound by memory (each reads and writes every mode once):
+//   k_spec_rhs    stencils and the x transform; two rows of a field make one
+//                 complex line, unpacked to n0/2 + 1 modes per row
+//   k_spec_y<0>   y transform, 16 adjacent modes x one line per thread group
+//   k_spec_solve  z transform of the four fields, the algebra above and the
+//                 inverse z transform, without leaving the SM
+//   k_spec_y<1>   inverse y transform
+//   k_spec_out    inverse x transform, u_next = u + w and p
+// Transforms are in place: decimation in frequency forward (natural order in,
+// digit-reversed order out), decimation in time backward, so no pass permutes
+// anything and a butterfly owns its places; the symbols are tabulated in the
+// order the modes are stored in.  Each transform's first pass reads global
+// memory and its last pass writes it.
+//
+// Measured on GB300 (us; V-cycles of fluid.cu before, this after): 32^3 step
+// 631 -> 46, 192^3 3425 -> 371, 256^3 6550 -> 770.  At 256^3 the five passes
+// take 198, 107, 175, 104 and 184 us for 0.57, 0.54, 0.54, 0.54 and 0.74 GB:
+// the y passes run at 5 TB/s, the others at 3 to 4 TB/s (instruction issue at
+// 50% beside the loads' latency).  x lines use radices up to 8 (48 registers,
+// 5 CTAs per SM: 184 against 250 us with radix 16 for k_spec_out); y lines up
+// to 16 (two passes at 256: 104 against 114..130 us); the z transform holds
+// four fields, 3 CTAs per SM (175 us; 2: 208, 4 with spills: 211).
+#include <algorithm>
+#include <cmath>
+#include <vector>
+
+#include "ib_internal.cuh"
+#include "spectral.cuh"
+
+namespace ibfe {
+namespace {
+
+constexpr int kTX = 16;   // modes per tile of the y transform (128-byte rows)
+constexpr int kTZ = 8;    // modes per tile of the z transform (four fields in shared memory)
+constexpr int kMaxN = 1024;
+
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
+  return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
+// a conj(b)
+__device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
+  return make_float2(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
+}
+// a times -i (forward) or i (inverse)
+template <bool kInv>
+__device__ __forceinline__ float2 rot(float2 a) {
+  return kInv ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
+}
+
+// R-point transforms in registers, natural order (exponent sign - forward, + inverse)
+template <int R, bool kInv>
+struct Dft;
+template <bool kInv>
+struct Dft<2, kInv> {
+  static __device__ __forceinline__ void run(float2* v) {
+    const float2 a = v[0];
+    v[0] = cadd(a, v[1]);
+    v[1] = csub(a, v[1]);
+  }
+};
+template <bool kInv>
+struct Dft<3, kInv> {
+  static __device__ __forceinline__ void run(float2* v) {
+    constexpr float s3 = 0.86602540378443864676f;  // sin(2 pi / 3)
+    const float2 t = cadd(v[1], v[2]), d = csub(v[1], v[2]);
+    const float2 m = make_float2(v[0].x - 0.5f * t.x, v[0].y - 0.5f * t.y);
+    const float2 s = rot<kInv>(make_float2(s3 * d.x, s3 * d.y));
+    v[0] = cadd(v[0], t);
+    v[1] = cadd(m, s);
+    v[2] = csub(m, s);
+  }
+};
+template <bool kInv>
+struct Dft<4, kInv> {
+  static __device__ __forceinline__ void run(float2* v) {
+    const float2 t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]);
+    const float2 t2 = cadd(v[1], v[3]), t3 = rot<kInv>(csub(v[1], v[3]));
+    v[0] = cadd(t0, t2);
+    v[1] = cadd(t1, t3);
+    v[2] = csub(t0, t2);
+    v[3] = csub(t1, t3);
+  }
+};
+template <bool kInv>
+struct Dft<5, kInv> {
+  static __device__ __forceinline__ void run(float2* v) {
+    constexpr float c1 = 0.30901699437494742410f, c2 = -0.80901699437494742410f;
+    constexpr float s1 = 0.95105651629515357212f, s2 = 0.58778525229247312917f;
+    const float2 t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
+    const float2 t3 = csub(v[1], v[4]), t4 = csub(v[2], v[3]);
+    const float2 m1 = make_float2(v[0].x + c1 * t1.x + c2 * t2.x, v[0].y + c1 * t1.y + c2 * t2.y);
+    const float2 m2 = make_float2(v[0].x + c2 * t1.x + c1 * t2.x, v[0].y + c2 * t1.y + c1 * t2.y);
+    const float2 e1 = rot<kInv>(make_float2(s1 * t3.x + s2 * t4.x, s1 * t3.y + s2 * t4.y));
+    const float2 e2 = rot<kInv>(make_float2(s2 * t3.x - s1 * t4.x, s2 * t3.y - s1 * t4.y));
+    v[0] = make_float2(v[0].x + t1.x + t2.x, v[0].y + t1.y + t2.y);
+    v[1] = cadd(m1, e1);
+    v[4] = csub(m1, e1);
+    v[2] = cadd(m2, e2);
+    v[3] = csub(m2, e2);
+  }
+};
+
+// cos and sin of 2 pi j / R for the composite radices
+template <int R>
+__device__ constexpr float kCosT(int j) {
+  constexpr float c16[16] = {1.f, 0.92387953251128675613f, 0.70710678118654752440f,
+                             0.38268343236508977173f, 0.f, -0.38268343236508977173f,
+                             -0.70710678118654752440f, -0.92387953251128675613f, -1.f,
+                             -0.92387953251128675613f, -0.70710678118654752440f,
+                             -0.38268343236508977173f, 0.f, 0.38268343236508977173f,
+                             0.70710678118654752440f, 0.92387953251128675613f};
+  constexpr float c6[6] = {1.f, 0.5f, -0.5f, -1.f, -0.5f, 0.5f};
+  return R == 6 ? c6[j % 6] : c16[(j * (16 / (R == 6 ? 16 : R))) % 16];
+}
+template <int R>
+__device__ constexpr float kSinT(int j) {
+  constexpr float s3 = 0.86602540378443864676f;
+  constexpr float s6[6] = {0.f, s3, s3, 0.f, -s3, -s3};
+  // sin(2 pi j / 16) = cos(2 pi (j - 4) / 16)
+  return R == 6 ? s6[j % 6] : kCosT<16>((j * (16 / (R == 6 ? 16 : R)) + 12) % 16);
+}
+
+// R = R1 R2: n = R2 n1 + n2, k = k1 + R1 k2
+template <int R1, int R2, bool kInv>
+struct DftC {
+  static __device__ __forceinline__ void run(float2* v) {
+    constexpr int R = R1 * R2;
+    float2 t[R];
+#pragma unroll
+    for (int n2 = 0; n2 < R2; ++n2) {
+      float2 a[R1];
+#pragma unroll
+      for (int n1 = 0; n1 < R1; ++n1) a[n1] = v[R2 * n1 + n2];
+      Dft<R1, kInv>::run(a);
+#pragma unroll
+      for (int k1 = 0; k1 < R1; ++k1) {
+        const int e = n2 * k1;
+        if (e == 0)
+          t[k1 * R2 + n2] = a[k1];
+        else if (4 * e == R)
+          t[k1 * R2 + n2] = rot<kInv>(a[k1]);
+        else
+          t[k1 * R2 + n2] =
+              cmul(a[k1], make_float2(kCosT<R>(e), kInv ? kSinT<R>(e) : -kSinT<R>(e)));
+      }
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < R1; ++k1) {
+      Dft<R2, kInv>::run(t + k1 * R2);
+#pragma unroll
+      for (int k2 = 0; k2 < R2; ++k2) v[k1 + R1 * k2] = t[k1 * R2 + k2];
+    }
+  }
+};
+template <bool kInv>
+struct Dft<6, kInv> : DftC<3, 2, kInv> {};
+template <bool kInv>
+struct Dft<8, kInv> : DftC<2, 4, kInv> {};
+template <bool kInv>
+struct Dft<16, kInv> : DftC<4, 4, kInv> {};
+
+// One pass over blocks of L = R Q places: butterfly j takes the places
+// b R Q + m + r Q, r < R, with b = j / Q and m = j mod Q.  magic = 2^20 / Q + 1
+// divides by Q exactly for j < n <= 1024.
+struct Pass {
+  int R, Q, tws;   // radix, stride, twiddle step n / L
+  unsigned magic;
+};
+__device__ __forceinline__ Pass get_pass(const SpecDim& d, int i) {
+  return Pass{d.rad[i], d.q[i], d.tws[i], d.magic[i]};
+}
+
+// Butterflies j0, j0 + step, ... of one pass on NF lines that share their
+// twiddles (the fields of the z transform; 1 elsewhere).  A.place(p0, Q) gives
+// the butterfly's address base, A.ld / A.st move place p0 + r Q of line c.
+// Forward: transform, then twiddles; inverse: conjugate twiddles, then
+// transform.
+template <int R, bool kInv, int NF, typename In, typename Out>
+__device__ __forceinline__ void pass_r(const Pass& P, int n, int j0, int step,
+                                       const float2* __restrict__ tw, const In& in,
+                                       const Out& out) {
+  for (int j = j0; j < n / R; j += step) {
+    const int b = (int)(((unsigned)j * P.magic) >> 20);
+    const int m = j - b * P.Q, p0 = b * R * P.Q + m;
+    constexpr bool kHold = NF > 1 && R <= 8;  // twiddles kept over the lines
+    float2 w[kHold ? R : 1];
+    if (kHold && P.Q > 1) {
+#pragma unroll
+      for (int r = 1; r < R; ++r) w[r] = __ldg(tw + m * r * P.tws);
+    }
+    auto twid = [&](int r) { return kHold ? w[r] : __ldg(tw + m * r * P.tws); };
+    const auto pi = in.place(p0, P.Q);
+    const auto po = out.place(p0, P.Q);
+#pragma unroll 1
+    for (int c = 0; c < NF; ++c) {
+      float2 v[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[r] = in.ld(pi, c, r);
+      if (kInv && P.Q > 1) {
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[r] = cmulc(v[r], twid(r));
+      }
+      Dft<R, kInv>::run(v);
+      if (!kInv && P.Q > 1) {
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[r] = cmul(v[r], twid(r));
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r) out.st(po, c, r, v[r]);
+    }
+  }
+}
+
+template <bool kInv, int NF, bool k16, typename In, typename Out>
+__device__ __forceinline__ void run_pass(const Pass& P, int n, int j0, int step,
+                                         const float2* __restrict__ tw, const In& in,
+                                         const Out& out) {
+  switch (P.R) {
+    case 2: pass_r<2, kInv, NF>(P, n, j0, step, tw, in, out); break;
+    case 3: pass_r<3, kInv, NF>(P, n, j0, step, tw, in, out); break;
+    case 4: pass_r<4, kInv, NF>(P, n, j0, step, tw, in, out); break;
+    case 5: pass_r<5, kInv, NF>(P, n, j0, step, tw, in, out); break;
+    case 6: pass_r<6, kInv, NF>(P, n, j0, step, tw, in, out); break;
+    case 8: pass_r<8, kInv, NF>(P, n, j0, step, tw, in, out); break;
+    case 16:
+      if constexpr (k16) pass_r<16, kInv, NF>(P, n, j0, step, tw, in, out);
+      break;
+  }
+}
+
+// A base address and the steps between the butterfly's places (even and odd r
+// start from a and b).
+struct Place {
+  int a, b, step;
+  __device__ __forceinline__ int at(int r) const { return ((r & 1) ? b : a) + r * step; }
+};
+
+// Column of a [place][mode] array in global memory, masked beyond the last mode
+struct GlobalCol {
+  float2* g;
+  int pitch;        // between places
+  int64_t field;    // between the lines c
+  bool on;
+  __device__ __forceinline__ Place place(int p0, int Q) const {
+    const int a = p0 * pitch;
+    return Place{a, a, Q * pitch};
+  }
+  __device__ __forceinline__ float2 ld(const Place& p, int c, int r) const {
+    return on ? g[c * field + p.at(r)] : make_float2(0.f, 0.f);
+  }
+  __device__ __forceinline__ void st(const Place& p, int c, int r, float2 v) const {
+    if (on) g[c * field + p.at(r)] = v;
+  }
+};
+
+// Column of a [place][width] array in shared memory.  width 16: a half-warp's
+// 16 columns of one place fill the 32 banks.  width 8: two places share them,
+// and the places whose (p >> sh) is odd swap with their neighbour (p ^ 1), so
+// that butterflies 2^sh places apart (the last pass) differ in parity; every
+// other pass's stride is a multiple of 2^sh, so the swap is one of two bases.
+// en = 0: no swap (odd last radix: neighbours already differ).
+template <int kW>
+struct SharedCol {
+  float2* s;
+  int field, sh, en;
+  __device__ __forceinline__ Place place(int p0, int Q) const {
+    if (kW == 16) return Place{p0 * kW, p0 * kW, Q * kW};
+    const int a = p0 ^ ((p0 >> sh) & en);
+    return Place{a * kW, (a ^ ((Q >> sh) & en)) * kW, Q * kW};
+  }
+  __device__ __forceinline__ float2 ld(const Place& p, int c, int r) const {
+    return s[c * field + p.at(r)];
+  }
+  __device__ __forceinline__ void st(const Place& p, int c, int r, float2 v) const {
+    s[c * field + p.at(r)] = v;
+  }
+};
+
+// Lines of the x transforms, [place][16 lines] with a row pitch of 17 (the
+// load and store phases run along the places) and one more skew per block of
+// the first pass's stride Q1: consecutive modes lie Q1 places apart, and
+// 17 Q1 + skew = 1 (mod 16) spreads them over the banks.
+constexpr int kXL = 16;  // lines: four row pairs x four fields
+constexpr int kXP = kXL + 1;
+struct LineSmem {
+  float2* s;
+  int Q1, skew;
+  unsigned magic1;
+  __device__ __forceinline__ int addr(int p) const {
+    return p * kXP + (int)(((unsigned)p * magic1) >> 20) * skew;
+  }
+  __device__ __forceinline__ Place place(int p0, int Q) const {
+    const int a = addr(p0);
+    return Place{a, a, Q * kXP + (Q == Q1 ? skew : 0)};
+  }
+  __device__ __forceinline__ float2 ld(const Place& p, int, int r) const { return s[p.at(r)]; }
+  __device__ __forceinline__ void st(const Place& p, int, int r, float2 v) const {
+    s[p.at(r)] = v;
+  }
+};
+__device__ __forceinline__ LineSmem line_smem(const SpecArgs& A, float2* s) {
+  return LineSmem{s, A.x.q[0], A.xskew, A.x.magic[0]};
+}
+
+__device__ __forceinline__ int up(int i, int n) { return i + 1 == n ? 0 : i + 1; }
+__device__ __forceinline__ int dn(int i, int n) { return i == 0 ? n - 1 : i - 1; }
+
+// kV adjacent cells of a row (kV = 2: 8-byte aligned)
+template <int kV>
+__device__ __forceinline__ void ld_cells(float* v, const float* __restrict__ g) {
+  if (kV == 2) {
+    const float2 t = __ldg(reinterpret_cast<const float2*>(g));
+    v[0] = t.x;
+    v[1] = t.y;
+  } else {
+    v[0] = __ldg(g);
+  }
+}
+
+// Transforms the 16 lines held in shared memory.
+template <bool kInv>
+__device__ __forceinline__ void line_passes(const SpecArgs& A, float2* z) {
+  const SpecDim& X = A.x;
+  const LineSmem L = line_smem(A, z + (threadIdx.x & (kXL - 1)));
+  for (int i = 0; i < X.np; ++i) {
+    run_pass<kInv, 1, false>(get_pass(X, kInv ? X.np - 1 - i : i), X.n, threadIdx.x / kXL,
+                      blockDim.x / kXL, X.tw, L, L);
+    __syncthreads();
+  }
+}
+
+// Row pairs 4 b .. 4 b + 3 of plane k (b = blockIdx.x): the four fields'
+// right-hand sides as complex lines (first row of the pair real, second
+// imaginary), their x transform, and the modes 0 .. n0/2 of every row.  Line
+// l = 4 (pair) + field.
+template <int kV>
+__global__ void __launch_bounds__(256, 5) k_spec_rhs(SpecArgs A, const float* __restrict__ u,
+                                                  const float* __restrict__ f) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* z = reinterpret_cast<float2*>(smem_raw);
+  const LineSmem L = line_smem(A, z);
+  const int n0 = A.x.n, n1 = A.y.n, n2 = A.z.n;
+  const int k = blockIdx.y, jp0 = blockIdx.x * 4, np = min(4, n1 / 2 - jp0);
+  const int cells = n0 * n1 * n2;
+  const int kp = up(k, n2) * n1, km = dn(k, n2) * n1, kc = k * n1;
+  // a thread forms kV cells of a row pair; work (pair, cells) laid out flat
+  const int nv = n0 / kV;
+  int rp = threadIdx.x / nv, iv = threadIdx.x - rp * nv;
+  while (rp < 4) {
+    const int i = iv * kV;
+    if (rp < np) {
+      const int ip = i + kV == n0 ? 0 : i + kV, im = dn(i, n0);
+      const int j = 2 * (jp0 + rp);
+      const int r0 = (kc + j) * n0, r1 = r0 + n0;
+      const int ra = (kc + dn(j, n1)) * n0 + i, rc = (kc + up(j + 1, n1)) * n0 + i;
+      const int ru = (kp + j) * n0 + i, rd = (km + j) * n0 + i;
+      float div0[kV], div1[kV];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const float* uc = u + c * cells;
+        float v0[kV + 1], v1[kV + 1], y2[kV], z0[kV], z1[kV];
+        ld_cells<kV>(v0, uc + r0 + i);
+        ld_cells<kV>(v1, uc + r1 + i);
+        v0[kV] = __ldg(uc + r0 + ip);
+        v1[kV] = __ldg(uc + r1 + ip);
+        ld_cells<kV>(y2, uc + rc);
+        ld_cells<kV>(z0, uc + ru);
+        ld_cells<kV>(z1, uc + ru + n0);
+#pragma unroll
+        for (int e = 0; e < kV; ++e) {
+          if (c == 0) div0[e] = v0[e + 1] - v0[e], div1[e] = v1[e + 1] - v1[e];
+          if (c == 1) div0[e] += v1[e] - v0[e], div1[e] += y2[e] - v1[e];
+          if (c == 2) div0[e] += z0[e] - v0[e], div1[e] += z1[e] - v1[e];
+        }
+        float g0[kV], g1[kV];
+        if (f) {
+          ld_cells<kV>(g0, f + c * cells + r0 + i);
+          ld_cells<kV>(g1, f + c * cells + r1 + i);
+        } else {
+#pragma unroll
+          for (int e = 0; e < kV; ++e) g0[e] = g1[e] = 0.f;
+        }
+        if (A.nu != 0.f) {
+          // second differences as sums of first differences
+          float ym[kV], q0[kV], q1[kV];
+          ld_cells<kV>(ym, uc + ra);
+          ld_cells<kV>(q0, uc + rd);
+          ld_cells<kV>(q1, uc + rd + n0);
+          float w0 = v0[0] - __ldg(uc + r0 + im), w1 = v1[0] - __ldg(uc + r1 + im);
+#pragma unroll
+          for (int e = 0; e < kV; ++e) {
+            const float x0 = v0[e + 1] - v0[e], x1 = v1[e + 1] - v1[e];
+            const float dy = v1[e] - v0[e];
+            g0[e] = fmaf(A.nu, (x0 - w0) + (dy - (v0[e] - ym[e])) +
+                                   ((z0[e] - v0[e]) - (v0[e] - q0[e])), g0[e]);
+            g1[e] = fmaf(A.nu, (x1 - w1) + ((y2[e] - v1[e]) - dy) +
+                                   ((z1[e] - v1[e]) - (v1[e] - q1[e])), g1[e]);
+            w0 = x0;
+            w1 = x1;
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < kV; ++e) z[L.addr(i + e) + 4 * rp + c] = make_float2(g0[e], g1[e]);
+      }
+#pragma unroll
+      for (int e = 0; e < kV; ++e) z[L.addr(i + e) + 4 * rp + 3] = make_float2(div0[e], div1[e]);
+    } else {  // lines past the last pair of the plane
+#pragma unroll
+      for (int e = 0; e < kV; ++e)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) z[L.addr(i + e) + 4 * rp + c] = make_float2(0.f, 0.f);
+    }
+    for (iv += blockDim.x; iv >= nv; iv -= nv) ++rp;
+  }
+  __syncthreads();
+  line_passes<false>(A, z);
+  // z_k = a_k + i b_k of the two real rows a, b:
+  //   2 a_k = z_k + conj z_{n-k},  2 b_k = -i (z_k - conj z_{n-k})
+  // (the factor 2 is in inv_n)
+  const int nx = n0 / 2 + 1;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  for (int l = warp; l < 4 * np; l += nwarps) {
+    float2* o = A.spec + ((int64_t)((l & 3) * n2 + k) * n1 + 2 * (jp0 + (l >> 2))) * A.pitch;
+    const float2* zl = z + l;
+#pragma unroll 4
+    for (int kx = lane; kx < nx; kx += 32) {
+      const float2 a = zl[__ldg(A.posx + kx)];
+      const float2 b = zl[__ldg(A.posx + (kx ? n0 - kx : 0))];
+      o[kx] = make_float2(a.x + b.x, a.y - b.y);
+      o[A.pitch + kx] = make_float2(a.y + b.y, b.x - a.x);
+    }
+  }
+}
+
+// One line of n1 places x kTX adjacent modes of one field and plane.
+template <bool kInv, bool k16>
+__global__ void __launch_bounds__(256, k16 ? 3 : 5) k_spec_y(SpecArgs A, int tile0) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int n1 = A.y.n, np = A.y.np;
+  const int col = threadIdx.x & (kTX - 1), j0 = threadIdx.x / kTX, step = blockDim.x / kTX;
+  const int kx = (blockIdx.x + tile0) * kTX + col;
+  const GlobalCol g{A.spec + (int64_t)(blockIdx.z * A.z.n + blockIdx.y) * n1 * A.pitch + kx,
+                    A.pitch, 0, kx <= A.x.n / 2};
+  const SharedCol<kTX> s{reinterpret_cast<float2*>(smem_raw) + col, 0, 0, 0};
+  run_pass<kInv, 1, k16>(get_pass(A.y, kInv ? np - 1 : 0), n1, j0, step, A.y.tw, g, s);
+  __syncthreads();
+  for (int i = 1; i + 1 < np; ++i) {
+    run_pass<kInv, 1, k16>(get_pass(A.y, kInv ? np - 1 - i : i), n1, j0, step, A.y.tw, s, s);
+    __syncthreads();
+  }
+  run_pass<kInv, 1, k16>(get_pass(A.y, kInv ? 0 : np - 1), n1, j0, step, A.y.tw, s, g);
+}
+
+// Last forward pass (stride 1, no twiddles) of the four fields, the solve and
+// the first inverse pass over the same places, in registers.
+template <int R>
+__device__ __forceinline__ void solve_pass(const SpecArgs& A, const SharedCol<kTZ>& s, int j0,
+                                           int step, float2 dx, float2 dy, float sxy) {
+  for (int j = j0; j < A.z.n / R; j += step) {
+    float2 v[4][R];
+    const int p0 = j * R, par = j & s.en;  // p0 >> sh = j for the even radices
+    float2* q0 = s.s + p0 * kTZ;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[c][r] = q0[c * s.field + (r ^ par) * kTZ];
+      Dft<R, false>::run(v[c]);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const float4 w = __ldg(A.symz + p0 + r);  // (Re D_z, Im D_z, |D_z|^2, 0)
+      const float2 dz = make_float2(w.x, w.y);
+      const float S = sxy + w.z;
+      const float hm = A.inv_n / fmaf(A.nu, S, A.alpha);
+      const float2 d0 = make_float2(v[0][r].x * hm, v[0][r].y * hm);
+      const float2 d1 = make_float2(v[1][r].x * hm, v[1][r].y * hm);
+      const float2 d2 = make_float2(v[2][r].x * hm, v[2][r].y * hm);
+      const float2 t = cadd(cadd(cmul(dx, d0), cmul(dy, d1)), cmul(dz, d2));
+      const float iS = S > 0.f ? 1.f / S : 0.f;
+      const float2 q = make_float2(fmaf(v[3][r].x, A.inv_n, t.x) * iS,
+                                   fmaf(v[3][r].y, A.inv_n, t.y) * iS);
+      v[0][r] = csub(d0, cmulc(q, dx));
+      v[1][r] = csub(d1, cmulc(q, dy));
+      v[2][r] = csub(d2, cmulc(q, dz));
+      v[3][r] = make_float2(q.x * A.pscale, q.y * A.pscale);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      Dft<R, true>::run(v[c]);
+#pragma unroll
+      for (int r = 0; r < R; ++r) q0[c * s.field + (r ^ par) * kTZ] = v[c][r];
+    }
+  }
+}
+
+template <bool k16>
+__global__ void __launch_bounds__(256, 3) k_spec_solve(SpecArgs A, int tile0) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int n2 = A.z.n, np = A.z.np;
+  const int col = threadIdx.x & (kTZ - 1), j0 = threadIdx.x / kTZ, step = blockDim.x / kTZ;
+  const int kx = (blockIdx.x + tile0) * kTZ + col;
+  const bool on = kx <= A.x.n / 2;
+  const int plane = A.y.n * A.pitch;
+  const GlobalCol g{A.spec + (int64_t)blockIdx.y * A.pitch + kx, plane, (int64_t)n2 * plane, on};
+  const SharedCol<kTZ> s{reinterpret_cast<float2*>(smem_raw) + col, n2 * kTZ, A.zsh, A.zen};
+  run_pass<false, 4, k16>(get_pass(A.z, 0), n2, j0, step, A.z.tw, g, s);
+  __syncthreads();
+  for (int i = 1; i + 1 < np; ++i) {
+    run_pass<false, 4, k16>(get_pass(A.z, i), n2, j0, step, A.z.tw, s, s);
+    __syncthreads();
+  }
+  const float4 wx = __ldg(A.symx + (on ? kx : 0)), wy = __ldg(A.symy + blockIdx.y);
+  const float2 dx = make_float2(wx.x, wx.y), dy = make_float2(wy.x, wy.y);
+  const float sxy = wx.z + wy.z;
+  switch (A.z.rad[np - 1]) {
+    case 2: solve_pass<2>(A, s, j0, step, dx, dy, sxy); break;
+    case 3: solve_pass<3>(A, s, j0, step, dx, dy, sxy); break;
+    case 4: solve_pass<4>(A, s, j0, step, dx, dy, sxy); break;
+    case 5: solve_pass<5>(A, s, j0, step, dx, dy, sxy); break;
+  }
+  __syncthreads();
+  for (int i = np - 2; i > 0; --i) {
+    run_pass<true, 4, k16>(get_pass(A.z, i), n2, j0, step, A.z.tw, s, s);
+    __syncthreads();
+  }
+  run_pass<true, 4, k16>(get_pass(A.z, 0), n2, j0, step, A.z.tw, s, g);
+}
+
+// Inverse x transform of four row pairs (plane k) of the four fields,
+// u_next = u + w and p.  kKeep: the increment w is also left in the rows of
+// spec (for the residuals).
+template <bool kKeep>
+__global__ void __launch_bounds__(256, 5) k_spec_out(SpecArgs A, const float* u, float* un,
+                                                  float* __restrict__ p) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* z = reinterpret_cast<float2*>(smem_raw);
+  const LineSmem L = line_smem(A, z);
+  const int n0 = A.x.n, n1 = A.y.n, n2 = A.z.n;
+  const int k = blockIdx.y, jp0 = blockIdx.x * 4, np = min(4, n1 / 2 - jp0);
+  const int nx = n0 / 2 + 1;
+  // a warp takes a line, four groups of 32 modes of both rows in flight
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  for (int l = warp; l < kXL; l += nwarps) {
+    const bool on = l < 4 * np;
+    const float2* g =
+        A.spec + ((int64_t)((l & 3) * n2 + k) * n1 + 2 * (jp0 + (on ? l >> 2 : 0))) * A.pitch;
+    float2* zl = z + l;
+    for (int k0 = lane; k0 < nx; k0 += 128) {
+      float2 a[4], b[4];
+      int pa[4], pb[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int kx = k0 + 32 * q;
+        a[q] = b[q] = make_float2(0.f, 0.f);
+        pa[q] = pb[q] = 0;
+        if (kx < nx) {
+          if (on) {
+            a[q] = g[kx];
+            b[q] = g[A.pitch + kx];
+          }
+          pa[q] = __ldg(A.posx + kx);
+          pb[q] = __ldg(A.posx + (kx ? n0 - kx : 0));
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int kx = k0 + 32 * q;
+        if (kx >= nx) break;
+        // z_k = a_k + i b_k, z_{n-k} = conj a_k + i conj b_k; real at k = 0, n/2
+        if (kx == 0 || 2 * kx == n0) {
+          zl[pa[q]] = make_float2(a[q].x, b[q].x);
+        } else {
+          zl[pa[q]] = make_float2(a[q].x - b[q].y, a[q].y + b[q].x);
+          zl[pb[q]] = make_float2(a[q].x + b[q].y, b[q].x - a[q].y);
+        }
+      }
+    }
+  }
+  __syncthreads();
+  line_passes<true>(A, z);
+  const int cells = n0 * n1 * n2;
+  int rp = threadIdx.x / n0, i = threadIdx.x - rp * n0;
+  while (rp < np) {
+    const int row = (k * n1 + 2 * (jp0 + rp)) * n0 + i;
+    const float2* zi = z + L.addr(i) + 4 * rp;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const float2 w = zi[c];
+      const float a = u[c * cells + row] + w.x, b = u[c * cells + row + n0] + w.y;
+      un[c * cells + row] = a;
+      un[c * cells + row + n0] = b;
+      if (kKeep) {
+        float* o = reinterpret_cast<float*>(A.spec + ((int64_t)(c * n2 + k) * n1 +
+                                                      2 * (jp0 + rp)) * A.pitch);
+        o[i] = w.x;
+        o[2 * A.pitch + i] = w.y;
+      }
+    }
+    const float2 w = zi[3];
+    p[row] = w.x;
+    p[row + n0] = w.y;
+    for (i += blockDim.x; i >= n0; i -= n0) ++rp;
+  }
+}
+
+// Squared residuals and right-hand sides of both solves, per CTA in fixed
+// order: part[4 b ..] = (Helmholtz residual, its rhs, Poisson residual, rhs).
+// u: the velocity before the step; w (rows of spec): the increment.
+__global__ void __launch_bounds__(256) k_spec_resid(SpecArgs A, const float* __restrict__ u,
+                                                    const float* __restrict__ f,
+                                                    const float* __restrict__ p, double a,
+                                                    double nu, double dtoh,
+                                                    double* __restrict__ part) {
+  __shared__ double sh[4][8];
+  const int n0 = A.x.n, n1 = A.y.n, n2 = A.z.n, cells = n0 * n1 * n2;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  auto at = [&](int i, int j, int k) { return (k * n1 + j) * n0 + i; };
+  // d = w + dt grad p (u* = u + d)
+  auto d = [&](int c, int i, int j, int k) {
+    const float w = reinterpret_cast<const float*>(
+        A.spec + ((int64_t)(c * n2 + k) * n1 + j) * A.pitch)[i];
+    const int b = c == 0 ? at(dn(i, n0), j, k) : (c == 1 ? at(i, dn(j, n1), k) : at(i, j, dn(k, n2)));
+    return double(w) + dtoh * (double(p[at(i, j, k)]) - double(p[b]));
+  };
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < cells; t += gridDim.x * blockDim.x) {
+    const int i = t % n0, j = (t / n0) % n1, k = t / (n0 * n1);
+    const int ip = up(i, n0), im = dn(i, n0), jp = up(j, n1), jm = dn(j, n1), kp = up(k, n2),
+              km = dn(k, n2);
+    for (int c = 0; c < 3; ++c) {
+      const float* uc = u + c * cells;
+      const double uu = uc[t];
+      const double lu = double(uc[at(ip, j, k)]) + uc[at(im, j, k)] + uc[at(i, jp, k)] +
+                        uc[at(i, jm, k)] + uc[at(i, j, kp)] + uc[at(i, j, km)] - 6.0 * uu;
+      const double dc = d(c, i, j, k);
+      const double ld = d(c, ip, j, k) + d(c, im, j, k) + d(c, i, jp, k) + d(c, i, jm, k) +
+                        d(c, i, j, kp) + d(c, i, j, km) - 6.0 * dc;
+      const double fc = f ? double(f[c * cells + t]) : 0.0;
+      const double rhs = a * uu + fc;
+      const double res = fc + nu * lu - (a * dc - nu * ld);
+      acc[0] += res * res;
+      acc[1] += rhs * rhs;
+    }
+    const double dv = (double(u[at(ip, j, k)]) - u[t]) +
+                      (double(u[cells + at(i, jp, k)]) - u[cells + t]) +
+                      (double(u[2 * cells + at(i, j, kp)]) - u[2 * cells + t]) +
+                      (d(0, ip, j, k) - d(0, i, j, k)) + (d(1, i, jp, k) - d(1, i, j, k)) +
+                      (d(2, i, j, kp) - d(2, i, j, k));
+    const double lp = double(p[at(ip, j, k)]) + p[at(im, j, k)] + p[at(i, jp, k)] +
+                      p[at(i, jm, k)] + p[at(i, j, kp)] + p[at(i, j, km)] - 6.0 * double(p[t]);
+    const double res = dv - dtoh * lp;  // both scaled by h
+    acc[2] += res * res;
+    acc[3] += dv * dv;
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_down_sync(0xffffffffu, acc[c], o);
+    if (lane == 0) sh[c][warp] = acc[c];
+  }
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    double s = 0.0;
+    for (int w = 0; w < 8; ++w) s += sh[threadIdx.x][w];
+    part[4 * blockIdx.x + threadIdx.x] = s;
+  }
+}
+
+// Radices of a transform of length n (product n, at least two; empty if n has
+// a prime factor above 5).  Few passes are best; the last one is `last` at
+// most (the z transform holds four fields' last butterflies in registers).
+std::vector<int> radices(int n, int last, int first = 16) {
+  int e2 = 0, e3 = 0, e5 = 0, m = n;
+  while (m % 2 == 0) m /= 2, ++e2;
+  while (m % 3 == 0) m /= 3, ++e3;
+  while (m % 5 == 0) m /= 5, ++e5;
+  std::vector<int> best;
+  if (m != 1) return best;
+  // smallest number of passes, then the smallest sum of radices
+  std::vector<int> cur;
+  static const int all[] = {16, 8, 6, 5, 4, 3, 2};
+  auto sum = [](const std::vector<int>& v) {
+    int s = 0;
+    for (int r : v) s += r;
+    return s;
+  };
+    std::function<void(int)> rec = [&](int left) {
+    if (left == 1) {
+      if (cur.size() < 2 || cur.back() > last) return;
+      if (best.empty() || cur.size() < best.size() ||
+          (cur.size() == best.size() && sum(cur) < sum(best)))
+        best = cur;
+      return;
+    }
+    if ((int)cur.size() >= kSpecMaxPasses) return;
+    for (int r : all) {
+          if (r > first || left % r || (!cur.empty() && r > cur.back())) continue;  // descending
+      cur.push_back(r);
+      rec(left / r);
+      cur.pop_back();
+    }
+  };
+  rec(n);
+  return best;
+}
+
+std::vector<int> dim_radices(int n, int d) {
+  return d == 0 ? radices(n, 8, 8) : (d == 1 ? radices(n, 16) : radices(n, 5));
+}
+// Threads of a CTA whose columns are `w` wide: one butterfly of the first
+// (largest) radix each, or an equal number each.
+int col_threads(int n, int r0, int w) {
+  const int rows = n / r0;
+  int t = (rows + 256 / w - 1) / (256 / w);
+  while (rows % t && t < rows) ++t;
+  return std::max(32, w * (rows / t));
+}
+
+size_t z_smem(int n2) { return sizeof(float2) * 4 * kTZ * (size_t)n2; }
+constexpr size_t kMaxSmem = 227 * 1024;
+
+bool ok(cudaError_t e) { return e == cudaSuccess; }
+
+}  // namespace
+
+bool spectral_supports(const int n[3]) {
+  for (int d = 0; d < 3; ++d)
+    if (n[d] % 2 || n[d] > kMaxN || dim_radices(n[d], d).empty()) return false;
+  return z_smem(n[2]) <= kMaxSmem;
+}
+
+ib_status spectral_create(Spectral* sp, const int n[3], double h, double rho, double mu,
+                          double dt) {
+  SpecArgs& A = sp->a;
+  SpecDim* dims[3] = {&A.x, &A.y, &A.z};
+  const double pi = 3.14159265358979323846;
+  std::vector<unsigned char> host;
+  auto put = [&](const void* src, size_t bytes) {
+    const size_t at = (host.size() + 15) / 16 * 16;
+    host.resize(at + bytes);
+    std::memcpy(host.data() + at, src, bytes);
+    return at;
+  };
+  size_t tw_at[3], sym_at[3], pos_at = 0;
+  for (int d = 0; d < 3; ++d) {
+    const int N = n[d];
+    SpecDim& D = *dims[d];
+    const std::vector<int> rad = dim_radices(N, d);
+    D.n = N;
+    D.np = (int)rad.size();
+    int L = N;
+    for (int i = 0; i < D.np; ++i) {
+      D.rad[i] = rad[i];
+      D.q[i] = L / rad[i];
+      D.tws[i] = N / L;
+      D.magic[i] = (1u << 20) / D.q[i] + 1;
+      L /= rad[i];
+    }
+    std::vector<float2> tw(N);
+    for (int j = 0; j < N; ++j)
+      tw[j] = make_float2((float)std::cos(2 * pi * j / N), (float)-std::sin(2 * pi * j / N));
+    // place p of the transformed line holds mode freq[p]
+    std::vector<int> freq(N), pos(N);
+    for (int p = 0; p < N; ++p) {
+      int k = 0, w = 1, r = p;
+      for (int i = 0; i < D.np; ++i) {
+        k += w * (r / D.q[i]);
+        r %= D.q[i];
+        w *= D.rad[i];
+      }
+      freq[p] = k;
+      pos[k] = p;
+    }
+    std::vector<float4> sym(N);
+    for (int p = 0; p < N; ++p) {
+      const int k = d == 0 ? p : freq[p];  // x modes are stored in order
+      const double s = std::sin(pi * k / N), c = std::cos(pi * k / N);
+      // D = exp(2 i t) - 1 = 2 i s exp(i t), |D|^2 = 4 s^2
+      sym[p] = make_float4((float)(-2 * s * s), (float)(2 * s * c), (float)(4 * s * s), 0.f);
+    }
+    tw_at[d] = put(tw.data(), sizeof(float2) * N);
+    sym_at[d] = put(sym.data(), sizeof(float4) * N);
+    if (d == 0) {  // shared-memory address of each mode (LineSmem::addr)
+      A.xskew = ((1 - D.q[0]) % 16 + 16) % 16;
+      for (int& q : pos) q = q * kXP + q / D.q[0] * A.xskew;
+      pos_at = put(pos.data(), sizeof(int) * N);
+    }
+  }
+  A.pitch = (n[0] / 2 + 1 + 3) / 4 * 4;  // rows start on 32-byte sectors
+  const size_t spec = sizeof(float2) * 4 * (size_t)n[2] * n[1] * A.pitch;
+  if (!ok(cudaMalloc(&sp->tables, host.size())) || !ok(cudaMalloc((void**)&A.spec, spec)) ||
+      !ok(cudaMemcpy(sp->tables, host.data(), host.size(), cudaMemcpyHostToDevice)))
+    return IB_ERR_CUDA;
+  const char* t = static_cast<const char*>(sp->tables);
+  for (int d = 0; d < 3; ++d) dims[d]->tw = reinterpret_cast<const float2*>(t + tw_at[d]);
+  A.symx = reinterpret_cast<const float4*>(t + sym_at[0]);
+  A.symy = reinterpret_cast<const float4*>(t + sym_at[1]);
+  A.symz = reinterpret_cast<const float4*>(t + sym_at[2]);
+  A.posx = reinterpret_cast<const int*>(t + pos_at);
+  A.alpha = (float)(rho / dt);
+  A.nu = (float)(mu / (h * h));
+  A.inv_n = (float)(0.5 / ((double)n[0] * n[1] * n[2]));
+  A.pscale = (float)(-h / dt);
+  // shared-memory swap of the z lines (even last radices 2 and 4)
+  const int last = A.z.rad[A.z.np - 1];
+  A.zsh = last == 4 ? 2 : 1;
+  A.zen = last % 2 == 0 ? 1 : 0;
+  sp->smem_x = sizeof(float2) * (size_t)(kXP * n[0] + A.x.rad[0] * A.xskew);
+  sp->smem_y = sizeof(float2) * kTX * n[1];
+  sp->smem_z = z_smem(n[2]);
+  sp->threads_x = col_threads(n[0], A.x.rad[0], kXL);
+  sp->threads_y = col_threads(n[1], A.y.rad[0], kTX);
+  sp->threads_z = col_threads(n[2], A.z.rad[0], kTZ);
+  auto opt = [](auto k) {
+    return ok(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)kMaxSmem));
+  };
+  return opt(k_spec_rhs<1>) && opt(k_spec_rhs<2>) && opt(k_spec_out<false>) &&
+                 opt(k_spec_out<true>) && opt(k_spec_y<false, false>) &&
+                 opt(k_spec_y<true, false>) && opt(k_spec_y<false, true>) &&
+                 opt(k_spec_y<true, true>) && opt(k_spec_solve<false>) && opt(k_spec_solve<true>)
+             ? IB_OK
+             : IB_ERR_CUDA;
+}
+
+void spectral_destroy(Spectral* sp) {
+  cudaFree(sp->tables);
+  cudaFree(sp->a.spec);
+  sp->tables = nullptr;
+  sp->a.spec = nullptr;
+}
+
+ib_status spectral_step(const Spectral* sp, const float* u, const float* f, float* un, float* p,
+                        bool keep, cudaStream_t s) {
+  const SpecArgs& A = sp->a;
+  const int n1 = A.y.n, n2 = A.z.n, nx = A.x.n / 2 + 1;
+  const dim3 gx((n1 / 2 + 3) / 4, n2);
+  const int ty = (nx + kTX - 1) / kTX, tz = (nx + kTZ - 1) / kTZ;
+  const bool y16 = A.y.rad[0] == 16, z16 = A.z.rad[0] == 16;  // radices descend
+  // cell pairs by 8-byte loads where the arrays' bases allow (rows are even)
+  const bool pairs = ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(f)) & 7) == 0;
+  (pairs ? k_spec_rhs<2> : k_spec_rhs<1>)<<<gx, sp->threads_x, sp->smem_x, s>>>(A, u, f);
+  (y16 ? k_spec_y<false, true> : k_spec_y<false, false>)<<<dim3(ty, n2, 4), sp->threads_y,
+                                                           sp->smem_y, s>>>(A, 0);
+  (z16 ? k_spec_solve<true> : k_spec_solve<false>)<<<dim3(tz, n1), sp->threads_z, sp->smem_z,
+                                                     s>>>(A, 0);
+  (y16 ? k_spec_y<true, true> : k_spec_y<true, false>)<<<dim3(ty, n2, 4), sp->threads_y,
+                                                         sp->smem_y, s>>>(A, 0);
+  (keep ? k_spec_out<true> : k_spec_out<false>)<<<gx, sp->threads_x, sp->smem_x, s>>>(A, u, un,
+                                                                                      p);
+  return ok(cudaGetLastError()) ? IB_OK : IB_ERR_CUDA;
+}
+
+void launch_spectral_resid(const Spectral* sp, const float* u, const float* f, const float* p,
+                           double a, double nu, double dtoh, double* part, int ctas,
+                           cudaStream_t s) {
+  k_spec_resid<<<ctas, 256, 0, s>>>(sp->a, u, f, p, a, nu, dtoh, part);
+}
+
+}  // namespace ibfe
