@@ -37,7 +37,7 @@ void free_plan(ib_plan* p) {
                   p->elem_scratch2, p->keys[0], p->keys[1], p->vals[0], p->vals[1], p->hist,
                   p->tile_start, p->tile_end, p->tile_slot, p->tile_nonempty, p->tile_near,
                   p->tile_list, p->tile_list_near, p->tile_vmax, p->tile_done, p->tile_sk, p->tile_bcount, p->tile_counters,
-                  p->digit_tot, p->rpart, p->spread_scratch, p->q_cell, p->q_off, p->q_val, p->p_cell,
+                  p->digit_tot, p->rpart, p->red_count, p->spread_scratch, p->q_cell, p->q_off, p->q_val, p->p_cell,
                   p->p_off, p->p_val, p->p_idx, p->vol_jm1, p->gq_a, p->gq_b, p->epart, p->ered,
                   p->dstatus, p->node_tmp, p->pen_part, p->mat_range, p->inst, p->tile_inst,
                   p->elem_inst, p->mat_dev};
@@ -224,9 +224,10 @@ ib_status do_spread(ib_plan* p, double scale, void* f, cudaStream_t s, bool zero
   return launch_spread(p, scale, f, s, zero_fill, calls, vals);
 }
 
-ib_status do_reduce(ib_plan* p, int nvals, int n_mats, cudaStream_t s, bool real_parts) {
-  Stage sc(p, IB_STAGE_REDUCE, s, 2);
-  return launch_reduce_parts(p, nvals, n_mats, s, real_parts);
+ib_status do_reduce(ib_plan* p, int nvals, int n_mats, cudaStream_t s, bool real_parts,
+                    double* out = nullptr) {
+  Stage sc(p, IB_STAGE_REDUCE, s, 1);
+  return launch_reduce_parts(p, nvals, n_mats, s, real_parts, out);
 }
 
 ib_status do_interp_tail(ib_plan* p, const void* u, void* U, cudaStream_t s,
@@ -400,6 +401,7 @@ ib_status plan_build(const ib_mesh* mesh, const GridDev& grid, int ntiles, int32
               dalloc(&p->tile_bcount, 12 * (size_t)classify_blocks(p->ntiles)) &&
               dalloc(&p->tile_counters, 32) && dalloc(&p->digit_tot, 4 * 256) &&
               dalloc(&p->rpart, 8 * kParamRow * (size_t)mat_cap * kReduceCTAs) &&
+              dalloc(&p->red_count, sizeof(int) * (size_t)mat_cap) &&
               dalloc(&p->mat_range, sizeof(int2) * (size_t)mat_cap) &&
               dalloc(&p->spread_scratch,
                      spread_scratch_bytes(precision, Q < p->ntiles ? (Q > 0 ? Q : 1)
@@ -440,6 +442,7 @@ ib_status plan_build(const ib_mesh* mesh, const GridDev& grid, int ntiles, int32
                             cudaMemcpyHostToDevice, s)) &&
          (E == 0 || ok(cudaMemcpyAsync(p->inc_idx, inc_idx.data(), 4 * nc * E,
                                        cudaMemcpyHostToDevice, s))) &&
+         ok(cudaMemsetAsync(p->red_count, 0, sizeof(int) * (size_t)mat_cap, s)) &&
          ok(cudaMemsetAsync(p->dstatus, 0, 16, s));
   int least = 0, greatest = 0;  // stream priorities (greatest: numerically lowest)
   if (good)
@@ -720,7 +723,15 @@ ib_status backward_body(ib_plan* p, const MatTable& mt, int n_mats, const ib_pos
     Stage sc(p, IB_STAGE_FORCE, s, 1);
     st = launch_fe_force_adj(p, mt, pos_a(p, x), x->off, gGt, p->elem_scratch, params, s);
   }
-  if (st == IB_OK && force && params) st = do_reduce(p, kParamRow, n_mats, s, true);
+  // the parameter gradients' sums, needed by nothing else: on the plan's
+  // high-priority stream beside the rest (one structure)
+  const bool reduce = force && params;
+  cudaStream_t r = pc ? s : p->hi;
+  if (reduce && st == IB_OK && r != s &&
+      (!ok(cudaEventRecord(p->ev_fsorted, s)) || !ok(cudaStreamWaitEvent(r, p->ev_fsorted, 0))))
+    st = IB_ERR_CUDA;
+  if (st == IB_OK && reduce) st = do_reduce(p, kParamRow, n_mats, r, true, gparams);
+  if (reduce && st == IB_OK && r != s && !ok(cudaEventRecord(p->ev_hjoin, r))) st = IB_ERR_CUDA;
   if (!pc && st == IB_OK && gf) st = to_nodes(p, p->gq_b, p->elem_scratch2, nullptr, gx, s);
   // join: gx = (spreading adjoint's term + interpolation adjoint's term) +
   // the force adjoint's gather, in that order
@@ -731,13 +742,12 @@ ib_status backward_body(ib_plan* p, const MatTable& mt, int n_mats, const ib_pos
   }
   if (st == IB_OK && force) st = do_gather(p, p->elem_scratch, nullptr, gx, s, gx, gxu);
   if (st == IB_OK && force) st = launch_penalty_adj(p, gGt, gx, s, gxu);
-  if (st == IB_OK && params) {
-    const size_t pb = sizeof(double) * kParamRow * (size_t)n_mats;
-    if (!force && !ok(cudaMemsetAsync(p->ered, 0, pb, s))) st = IB_ERR_CUDA;
-    if (st == IB_OK && gparams &&
-        !ok(cudaMemcpyAsync(gparams, p->ered, pb, cudaMemcpyDeviceToDevice, s)))
-      st = IB_ERR_CUDA;
-  }
+  if (st == IB_OK && reduce && r != s && !ok(cudaStreamWaitEvent(s, p->ev_hjoin, 0)))
+    st = IB_ERR_CUDA;
+  if (st == IB_OK && params && !force &&
+      !ok(cudaMemsetAsync(gparams ? gparams : p->ered, 0,
+                          sizeof(double) * kParamRow * (size_t)n_mats, s)))
+    st = IB_ERR_CUDA;
   return check_launch(st);
 }
 

@@ -10,15 +10,22 @@
 namespace ibfe {
 namespace {
 
-// Deterministic per-material sums of per-element partials in two levels.
-// Material m's elements lie in the range mrange[m] (the whole mesh for a
-// plan of one structure; its instance's elements in a packed plan): CTA b
-// reduces chunk b of that range, all values of the material in one pass, each
-// value with its own fixed-shape tree (warp shuffles, then the warp sums; one
-// barrier pair per material); then one warp per (material, value) pair sums
-// the per-CTA partials with the same tree.  The partition and the trees
-// depend only on the range, so an instance of a packed plan gets the bits of
-// a plan of its own.
+// Deterministic per-material sums of per-element partials, one launch.
+// Material m's elements lie in the range mrange[m] (the whole mesh for a plan
+// of one structure; its instance's elements in a packed plan), cut into at
+// most kReduceCTAs chunks of at least kRedMin elements; CTA (b, m) sums chunk
+// b: each thread its elements in order, then one warp per value the threads'
+// sums (eight per lane, then a shuffle tree).  The CTA that completes its
+// material's count adds the chunks' sums, again one warp per value in a fixed
+// order.  The partition and the trees depend only on the range, so an
+// instance of a packed plan gets the bits of a plan of its own.
+//
+// FP64 adds run at 1/64 of the FP32 rate on GB300, and this kernel runs
+// beside the spreading: a value takes 12 warp-wide adds per CTA (every warp's
+// own tree for each value took 50), and materials have their own CTAs instead
+// of being visited in turn by all of them.  Packed sweep of 16 shells, beside
+// the spreading: 346 + 20 us before (two levels, every CTA through every
+// material); 256^3 backward 125 + 6 us.
 __device__ __forceinline__ double warp_tree(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -26,76 +33,66 @@ __device__ __forceinline__ double warp_tree(double v) {
 }
 
 constexpr int kRedThreads = 256;
-
-// The block_sum tree for every value k < nvals of a thread at once (one
-// barrier pair for all of them); value k's sum is bitwise the one block_sum
-// forms for it alone.
-__device__ __forceinline__ void block_sum_row(double (&v)[kParamRow], int nvals,
-                                              double (*sh)[kParamRow]) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < kParamRow; ++k)
-    if (k < nvals) {
-      v[k] = warp_tree(v[k]);
-      if (lane == 0) sh[warp][k] = v[k];
-    }
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int k = 0; k < kParamRow; ++k)
-      if (k < nvals) v[k] = warp_tree(lane < (int)(blockDim.x >> 5) ? sh[lane][k] : 0.0);
-  }
-  __syncthreads();
-}
+constexpr int kRedMin = 1024;
 
 template <typename T>
-__global__ void __launch_bounds__(kRedThreads) k_reduce_l1(const T* __restrict__ part,
-                                                           const int32_t* __restrict__ mat_id,
-                                                           const int2* __restrict__ mrange,
-                                                           int E, int nvals, int n_mats,
-                                                           double* __restrict__ rpart) {
-  __shared__ double sh[32][kParamRow];
-  for (int m = 0; m < n_mats; ++m) {
-    const int2 r = mrange[m];
-    const int chunk = (r.y - r.x + gridDim.x - 1) / gridDim.x;
-    const int e0 = r.x + blockIdx.x * chunk, e1 = min(r.y, e0 + chunk);
-    double s[kParamRow];
+__global__ void __launch_bounds__(kRedThreads) k_reduce(const T* __restrict__ part,
+                                                        const int32_t* __restrict__ mat_id,
+                                                        const int2* __restrict__ mrange, int E,
+                                                        int nvals, double* rpart, int* count,
+                                                        double* __restrict__ out) {
+  __shared__ double sh[kParamRow][kRedThreads];
+  __shared__ bool last;
+  const int m = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int2 r = mrange[m];
+  const int len = r.y - r.x;
+  const int chunk = max(kRedMin, (len + kReduceCTAs - 1) / kReduceCTAs);
+  const int nblk = max(1, (len + chunk - 1) / chunk);
+  if ((int)blockIdx.x >= nblk) return;
+  const int e0 = r.x + blockIdx.x * chunk, e1 = min(r.y, e0 + chunk);
+  double s[kParamRow];
 #pragma unroll
-    for (int k = 0; k < kParamRow; ++k) s[k] = 0.0;
-    for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x)
-      if ((mat_id ? __ldg(mat_id + e) : 0) == m) {
-#pragma unroll
-        for (int k = 0; k < kParamRow; ++k)
-          if (k < nvals) s[k] += double(__ldg(part + (int64_t)k * E + e));
-      }
-    block_sum_row(s, nvals, sh);
-    if (threadIdx.x == 0) {
+  for (int k = 0; k < kParamRow; ++k) s[k] = 0.0;
+#pragma unroll 2
+  for (int e = e0 + threadIdx.x; e < e1; e += kRedThreads)
+    if ((mat_id ? __ldg(mat_id + e) : 0) == m) {
 #pragma unroll
       for (int k = 0; k < kParamRow; ++k)
-        if (k < nvals) rpart[((int64_t)blockIdx.x * n_mats + m) * kParamRow + k] = s[k];
+        if (k < nvals) s[k] += double(__ldg(part + (int64_t)k * E + e));
+    }
+#pragma unroll
+  for (int k = 0; k < kParamRow; ++k)
+    if (k < nvals) sh[k][threadIdx.x] = s[k];
+  __syncthreads();
+  double* mine = rpart + (int64_t)m * kReduceCTAs * kParamRow;
+  for (int k = warp; k < nvals; k += kRedThreads / 32) {
+    double v = 0.0;
+#pragma unroll
+    for (int t = 0; t < kRedThreads / 32; ++t) v += sh[k][32 * t + lane];
+    v = warp_tree(v);
+    if (lane == 0) {
+      if (nblk == 1)
+        out[m * kParamRow + k] = v;
+      else
+        mine[blockIdx.x * kParamRow + k] = v;
     }
   }
-}
-
-// One warp per (material, value): the block_sum tree of a kRedThreads-thread
-// CTA whose thread t holds partial t (nblk <= kRedThreads), evaluated warp
-// by warp.
-__global__ void __launch_bounds__(kRedThreads) k_reduce_l2(const double* __restrict__ rpart,
-                                                           int nblk, int nvals, int n_mats,
-                                                           double* __restrict__ out) {
-  const int pair = blockIdx.x * (kRedThreads / 32) + (threadIdx.x >> 5);
-  if (pair >= n_mats * nvals) return;
-  const int m = pair / nvals, k = pair % nvals, lane = threadIdx.x & 31;
-  double ws = 0.0;  // lane w: the tree sum of the partials of thread block w
-  for (int w = 0; w < kRedThreads / 32; ++w) {
-    const int b = 32 * w + lane;
-    double v = 0.0;
-    if (b < nblk) v += rpart[((int64_t)b * n_mats + m) * kParamRow + k];
-    v = __shfl_sync(0xffffffffu, warp_tree(v), 0);
-    if (lane == w) ws = v;
+  if (nblk == 1) return;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(count + m, 1) + 1 == nblk;
+    if (last) count[m] = 0;  // for the next call
   }
-  const double t = warp_tree(ws);
-  if (lane == 0) out[m * kParamRow + k] = t;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int k = warp; k < nvals; k += kRedThreads / 32) {
+    double v = 0.0;
+    for (int b = lane; b < nblk; b += 32) v += __ldcg(mine + b * kParamRow + k);
+    v = warp_tree(v);
+    if (lane == 0) out[m * kParamRow + k] = v;
+  }
 }
 
 // The smallest instantiated law set covering the material table (every
@@ -220,24 +217,24 @@ ib_status launch_fe_force_adj(ib_plan* p, const MatTable& mt, const void* xa, co
 #undef IBFE_FE_ARGS
 
 ib_status launch_reduce_parts(ib_plan* p, int nvals, int n_mats, cudaStream_t s,
-                              bool real_parts) {
+                              bool real_parts, double* out) {
   if (n_mats > p->mat_cap) return IB_ERR_INVALID_ARG;
+  if (!out) out = p->ered;
   if (p->E == 0) {
-    cudaMemsetAsync(p->ered, 0, sizeof(double) * kParamRow * p->mat_cap, s);
+    cudaMemsetAsync(out, 0, sizeof(double) * kParamRow * n_mats, s);
     return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
   }
-  static_assert(kReduceCTAs <= kRedThreads, "one partial per thread of the second level");
+  // chunks any material can have: the whole mesh's
+  const int nblk = std::min(kReduceCTAs, (p->E + kRedMin - 1) / kRedMin);
+  const dim3 grid(nblk, n_mats);
   // FP32 partials are widened exactly: the sums are those of their doubles
   if (real_parts && p->precision != IB_FP64)
-    k_reduce_l1<float><<<kReduceCTAs, kRedThreads, 0, s>>>(
-        reinterpret_cast<const float*>(p->epart), p->mat_id, p->mat_range, p->E, nvals, n_mats,
-        p->rpart);
+    k_reduce<float><<<grid, kRedThreads, 0, s>>>(reinterpret_cast<const float*>(p->epart),
+                                                 p->mat_id, p->mat_range, p->E, nvals, p->rpart,
+                                                 p->red_count, out);
   else
-    k_reduce_l1<double><<<kReduceCTAs, kRedThreads, 0, s>>>(p->epart, p->mat_id, p->mat_range,
-                                                            p->E, nvals, n_mats, p->rpart);
-  const int pairs = n_mats * nvals, per = kRedThreads / 32;
-  k_reduce_l2<<<(pairs + per - 1) / per, kRedThreads, 0, s>>>(p->rpart, kReduceCTAs, nvals,
-                                                             n_mats, p->ered);
+    k_reduce<double><<<grid, kRedThreads, 0, s>>>(p->epart, p->mat_id, p->mat_range, p->E, nvals,
+                                                  p->rpart, p->red_count, out);
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 

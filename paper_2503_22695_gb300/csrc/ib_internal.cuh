@@ -190,7 +190,8 @@ struct ib_plan {
                          //     [3] near count, [4] second interpolation's counter,
                          //     [6] FE force block counter
   int32_t* digit_tot;    // [256] radix digit totals
-  double* rpart;         // [reduce CTAs][IB_MAX_MATERIALS*kParamRow] reduction partials
+  double* rpart;         // [mat_cap][reduce CTAs][kParamRow] reduction partials
+  int* red_count;        // [mat_cap] chunks reduced (zero between calls)
   cudaStream_t side;     // interpolation branch of ib_forward
   cudaStream_t hi;       // ib_forward's critical branch (force -> spread), high priority
   cudaStream_t zside;    // far-tile zero-fill of the spread
@@ -267,9 +268,10 @@ ib_status launch_fe_force_adj(ib_plan* p, const MatTable& mt, const void* x_cell
                               const float* off, const void* v, void* elem_out, bool params,
                               cudaStream_t s);
 // real_parts: the partials are in the plan's Real (parameter gradients),
-// else in double (energy); the sums are in double either way
+// else in double (energy); the sums are in double either way, written to out
+// ([n_mats][kParamRow], default the plan's ered)
 ib_status launch_reduce_parts(ib_plan* p, int nvals, int n_mats, cudaStream_t s,
-                              bool real_parts);
+                              bool real_parts, double* out = nullptr);
 // one instantiation of the force kernel's launcher (fe_kernel.cuh; explicit
 // instantiations in fe_force_f32.cu, fe_force_adj.cu, fe_force_var.cu)
 template <typename Real, typename S, bool kEnergy, bool kAdj, bool kParams, int kLaws, int kEl>
@@ -387,7 +389,7 @@ struct PackedCalls {
 // The sequences of ib_forward and ib_backward (pc null: one structure, the
 // fields and scalars are the arguments; pc set: a packed plan, the fields and
 // h-dependent scalars are pc's).  params: compute the parameter gradients
-// into p->ered (copied to gparams when it is not null).
+// into gparams (p->ered when it is null).
 ib_status forward_body(ib_plan* p, const MatTable& mt, const ib_pos* x, const void* u, void* G,
                        void* f, void* U, cudaStream_t s, const PackedCalls* pc);
 ib_status backward_body(ib_plan* p, const MatTable& mt, int n_mats, const ib_pos* x,
