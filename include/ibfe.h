@@ -266,7 +266,8 @@ ib_status ib_backward(ib_plan* plan, const ib_material* mats, int32_t n_mats, co
 
 /* Launch tuning of a plan, four entries:
  *   [0] points per work item of spreading and interpolation, 512..1024
- *       (a tile's points are cut into items of at most this many);
+ *       (a tile's points are cut into items of at most this many; a plan with
+ *       too few points to give every SM an item cuts them smaller);
  *   [1] FE-force CTAs per SM in ib_forward, 1..5 (its persistent grid leaves
  *       the rest of each SM to the binning and interpolation beside it);
  *   [2] cap on the spreading CTAs per SM, 1..8;

@@ -36,7 +36,7 @@ void free_plan(ib_plan* p) {
   void* ptrs[] = {p->inc_off, p->inc_idx, p->mass, p->inv_mass, p->wj0, p->elem_scratch,
                   p->elem_scratch2, p->keys[0], p->keys[1], p->vals[0], p->vals[1], p->hist,
                   p->tile_start, p->tile_end, p->tile_slot, p->tile_nonempty, p->tile_near,
-                  p->tile_list, p->tile_list_near, p->tile_vmax, p->tile_done, p->tile_sk, p->tile_bcount, p->tile_counters,
+                  p->items, p->tile_list_near, p->tile_vmax, p->tile_done, p->tile_sk, p->tile_bcount, p->tile_counters,
                   p->digit_tot, p->rpart, p->red_count, p->spread_scratch, p->q_cell, p->q_off, p->q_val, p->p_cell,
                   p->p_off, p->p_val, p->p_idx, p->vol_jm1, p->gq_a, p->gq_b, p->epart, p->ered,
                   p->dstatus, p->node_tmp, p->pen_part, p->mat_range, p->inst, p->tile_inst,
@@ -363,6 +363,15 @@ ib_status plan_build(const ib_mesh* mesh, const GridDev& grid, int ntiles, int32
   p->nc = nc;
   p->nq = nq;
   p->chunk = kChunk;
+  {
+    int dev = 0, sms = 0;
+    if (!ok(cudaGetDevice(&dev)) ||
+        !ok(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) {
+      delete p;
+      return IB_ERR_CUDA;
+    }
+    p->item = item_size(precision, Q, sms);
+  }
   // the fastest tuning of the 256^3 shell forward in A/B runs
   p->fe_ctas = 4;
   p->push_per_sm = 8;
@@ -393,7 +402,7 @@ ib_status plan_build(const ib_mesh* mesh, const GridDev& grid, int ntiles, int32
               dalloc(&p->tile_slot, 4 * (size_t)p->ntiles) &&
               dalloc(&p->tile_nonempty, 4 * (size_t)p->ntiles) &&
               dalloc(&p->tile_near, 4 * (size_t)p->ntiles) &&
-              dalloc(&p->tile_list, 4 * (size_t)max_work_items(p->ntiles, Q)) &&
+              dalloc(&p->items, 16 * (size_t)max_work_items(p->ntiles, Q, p->item)) &&
               dalloc(&p->tile_list_near, 4 * (size_t)p->ntiles) &&
               dalloc(&p->tile_vmax, 4 * (size_t)p->ntiles) &&
               dalloc(&p->tile_done, 4 * (size_t)p->ntiles) &&
@@ -404,8 +413,7 @@ ib_status plan_build(const ib_mesh* mesh, const GridDev& grid, int ntiles, int32
               dalloc(&p->red_count, sizeof(int) * (size_t)mat_cap) &&
               dalloc(&p->mat_range, sizeof(int2) * (size_t)mat_cap) &&
               dalloc(&p->spread_scratch,
-                     spread_scratch_bytes(precision, Q < p->ntiles ? (Q > 0 ? Q : 1)
-                                                                   : max_work_items(p->ntiles, Q))) &&
+                     spread_scratch_bytes(precision, max_work_items(p->ntiles, Q, p->item))) &&
               dalloc(&p->q_cell, 4 * Q) &&
               dalloc(&p->q_off, rs * 3 * Q) && dalloc(&p->q_val, rs * 3 * Q) &&
               dalloc(&p->p_cell, 4 * Q) && dalloc(&p->p_off, rs * 3 * Q) &&

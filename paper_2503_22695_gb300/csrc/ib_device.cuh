@@ -216,6 +216,28 @@ __device__ __forceinline__ TileGeo tile_geo(const GridDev& g, const InstDev* ins
   }
   return t;
 }
+// Points per work item of a tile holding n points: the plan's item size
+// `item` where that gives at most eight items, else an eighth of the tile's
+// points (in whole `gran`s; one CTA sums a tile's items in the spreading), at
+// most `chunk`.
+__device__ __forceinline__ int item_points(int n, const ItemRule& r) {
+  const int eighth = ((n + 7) / 8 + r.gran - 1) / r.gran * r.gran;
+  return min(r.chunk, max(r.item, eighth));
+}
+
+// Work item of the transfer kernels: its points [begin, begin + n), its tile,
+// its scratch block and the tile's number of items, in one 16-byte record.
+struct Item {
+  int begin, n, tile, slot, nit;
+};
+__device__ __forceinline__ int4 make_item(int begin, int n, int tile, int slot, int nit) {
+  return make_int4(begin, tile, slot, n | nit << 11);  // n <= kChunk = 1024
+}
+__device__ __forceinline__ Item load_item(const int4* items, int k) {
+  const int4 v = __ldg(items + k);
+  return Item{v.x, v.w & 2047, v.y, v.z, v.w >> 11};
+}
+
 // tile coordinates of a tile within its structure's grid
 __device__ __forceinline__ void tile_coords(const TileGeo& t, int tile, int& tx, int& ty,
                                             int& tz) {

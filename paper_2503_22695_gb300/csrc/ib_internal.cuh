@@ -29,6 +29,13 @@ constexpr int kPackBits = 10;       // packed wrapped cell: x | y << 10 | z << 2
 constexpr int kChunk = 1024;        // maximum points per spread / interp work item
 constexpr int kMinChunk = 512;      // smallest work item the tuning may choose
 
+// How the points of a tile are cut into work items (item_points in
+// ib_device.cuh): `chunk` is the tuning's size; `item` <= chunk the size for
+// plans with few points, in steps of `gran`.
+struct ItemRule {
+  int chunk, item, gran;
+};
+
 // Device-side status bits latched by kernels (read by ib_plan_sync_status).
 constexpr int kStatNonfinite = 1;
 constexpr int kStatInverted = 2;
@@ -180,12 +187,12 @@ struct ib_plan {
   int32_t* tile_slot;    // [ntiles] first work item of each tile holding points (-1: none)
   int32_t* tile_nonempty;// [ntiles] number of work items of the tile
   int32_t* tile_near;    // [ntiles] 1 if a tile of its 3x3x3 neighbourhood holds points
-  int32_t* tile_list;    // [max work items] tile of each work item
+  int4* items;           // [max work items] work items (ib_device.cuh)
   int32_t* tile_list_near;// [ntiles] near tiles, ascending
   uint32_t* tile_vmax;   // [ntiles] FP32: bits of the largest |carried value| of each tile
   int32_t* tile_done;    // [ntiles] work items of the tile written (FP32 spreading, per call)
   int32_t* tile_sk;      // [4 ntiles] FP32: first block slot, exponent, item bound, items
-  int32_t* tile_bcount;  // [2 * classify CTAs] per-CTA counts
+  int32_t* tile_bcount;  // [3 * classify CTAs] per-CTA counts
   int32_t* tile_counters;// [8] [0] work items, [1] push counter, [2] interpolation counter,
                          //     [3] near count, [4] second interpolation's counter,
                          //     [6] FE force block counter
@@ -203,6 +210,7 @@ struct ib_plan {
   // item, FE-force CTAs per SM in the forward, caps on the spreading and
   // interpolation CTAs per SM (the occupancy maxima above are per-SM * sm_count)
   int chunk, fe_ctas, push_per_sm, interp_per_sm;
+  int item;              // work item size for plans with few points (<= kChunk)
   void* spread_scratch;  // Real [slots][3][12^3] halo'd per-tile blocks
   int32_t* q_cell;       // packed wrapped cell per Gauss point (unsorted, gq order)
   void* q_off;           // Real [3][Q]
@@ -425,7 +433,12 @@ ib_status launch_advance_positions(ib_plan* p, const ib_pos* x, const void* U, d
 // tiles.cu
 ib_status launch_classify_tiles(ib_plan* p, cudaStream_t s);
 int classify_blocks(int ntiles);
-int64_t max_work_items(int ntiles, int64_t Q);
+int item_size(int precision, int64_t Q, int sms);
+int64_t max_work_items(int ntiles, int64_t Q, int item);
+inline ItemRule item_rule(const ib_plan* p) {
+  const int gran = p->precision == IB_FP64 ? 32 : 128;
+  return ItemRule{p->chunk, p->item < p->chunk ? p->item : p->chunk, gran};
+}
 int sort_key_bits(int ntiles);
 constexpr int kReduceCTAs = 128;
 

@@ -11,8 +11,8 @@
 //
 // FP32 plans stage the block with the Tensor Memory Accelerator: one thread
 // issues a 4-D tiled bulk copy (x 16 from face -4 so that the start is
-// 16-byte aligned, y 12, z 12, all 3 components) of the next item into a
-// dense buffer while the CTA evaluates the current item; the dense box is
+// 16-byte aligned, y 12, z 12, all 3 components) of the item's box into a
+// dense buffer while the CTA stages the item's points; the dense box is
 // then rewritten into the padded block layout (z stride 145, odd in banks)
 // that keeps the per-thread stencil gathers spread over the banks.  Tiles
 // whose halo crosses the periodic boundary are staged with cp.async and
@@ -49,17 +49,13 @@ struct InterpArgs {
   const GridCall* calls;     // packed plans: each instance's u, vscale, gscale, else null
   const CUtensorMap* tmaps;  // packed plans: each instance's tensor map of u (FP32)
   int64_t Q;
-  const int32_t* tile_start;
-  const int32_t* tile_end;
-  const int32_t* tile_slot;  // first work item of each tile
-  const int32_t* tile_list;  // tile of each work item
+  const int4* items;         // work items
   int32_t* counters;      // [0] work items, [2] the values-only mode's work counter
   int32_t* work;          // the gradient modes' work counter (zero at launch)
   const int32_t* p_cell;
   const Real* p_off;
   const Real* p_val;
   const int32_t* p_idx;
-  int chunk;               // points per work item
   const Real* u;
   Real vscale, gscale;
   Real* out_a;
@@ -97,13 +93,11 @@ __device__ __forceinline__ void cp_async_wait_group() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
-// Copy the halo'd 12^3 block of each velocity component around the tile of
-// work item `slot` (faces local -2..9, periodically wrapped) into `ub`,
+// Copy the halo'd 12^3 block of each velocity component around a tile (faces local -2..9, periodically wrapped) into `ub`,
 // asynchronously: 16 lanes per 12-face x-row, 16 rows per pass.
 template <bool kPacked, typename Real>
-__device__ __forceinline__ void stage_block(const InterpArgs<Real>& A, int slot, Real* ub, int tid) {
-  const int tile = A.tile_list[slot];
-  const TileGeo geo = tile_geo<kPacked>(A.g, A.inst, A.tile_inst, tile);
+__device__ __forceinline__ void stage_block(const InterpArgs<Real>& A, const TileGeo& geo, int tile,
+                                            Real* ub, int tid) {
   int tx, ty, tz;
   tile_coords(geo, tile, tx, ty, tz);
   const int n0 = geo.n[0], n1 = geo.n[1], n2 = geo.n[2];
@@ -155,7 +149,11 @@ __global__ void __launch_bounds__(kThreads) k_interp_tile(InterpArgs<Real> A) {
   if (tid == 0) next = atomicAdd(work_counter<MODE>(A), 1);
   __syncthreads();
   int cur = next;
-  if (cur < count) stage_block<kPacked>(A, cur, buf0, tid);
+  auto stage = [&](int k, Real* ub) {
+    const int tile = load_item(A.items, k).tile;
+    stage_block<kPacked>(A, tile_geo<kPacked>(A.g, A.inst, A.tile_inst, tile), tile, ub, tid);
+  };
+  if (cur < count) stage(cur, buf0);
   cp_async_commit();
   int b = 0;
   while (cur < count) {
@@ -163,7 +161,7 @@ __global__ void __launch_bounds__(kThreads) k_interp_tile(InterpArgs<Real> A) {
     if (tid == 0) next = atomicAdd(work_counter<MODE>(A), 1);
     __syncthreads();
     const int nxt = next;
-    if (nxt < count) stage_block<kPacked>(A, nxt, buf0 + (b ^ 1) * 3 * kComp, tid);
+    if (nxt < count) stage(nxt, buf0 + (b ^ 1) * 3 * kComp);
     cp_async_commit();
     cp_async_wait_group<1>();  // the current item's block has landed
     __syncthreads();
@@ -270,13 +268,12 @@ struct PtStage {
 };
 
 template <int MODE, bool kPacked>
-__device__ __forceinline__ int local_cell_stage(const InterpArgs<float>& A, int slot, int* cnt,
-                                                PtStage<MODE>& P, int* tmp, int tid) {
-  const int tile = A.tile_list[slot];
-  const int s = A.tile_start[tile] + (slot - A.tile_slot[tile]) * A.chunk;
-  const int e = min(A.tile_end[tile], s + A.chunk);
+__device__ __forceinline__ void local_cell_stage(const InterpArgs<float>& A, const Item& item,
+                                                 const TileGeo& g, int* cnt, PtStage<MODE>& P,
+                                                 int* tmp, int tid) {
+  const int s = item.begin, e = s + item.n;
   int tx, ty, tz;
-  tile_coords(tile_geo<kPacked>(A.g, A.inst, A.tile_inst, tile), tile, tx, ty, tz);
+  tile_coords(g, item.tile, tx, ty, tz);
   const int x0 = tx * kTile, y0 = ty * kTile, z0 = tz * kTile;
   cnt[tid] = 0;
   cnt[tid + kThreads] = 0;
@@ -326,11 +323,10 @@ __device__ __forceinline__ int local_cell_stage(const InterpArgs<float>& A, int 
       P.lc[q] = (short)cell[k];
     }
   }
-  return e - s;
 }
 
-// Per item: wait for its box (or stage it with cp.async), rewrite it into the
-// padded block, issue the next item's box, evaluate the points
+// Per item: issue its box, stage its points, wait for the box (or stage it
+// with cp.async), rewrite it into the padded block, evaluate the points
 // (shared memory holds 3 CTAs per SM in mode 0 and 2 in the gradient modes;
 // the register bounds follow)
 template <int MODE, bool kPacked>
@@ -352,59 +348,44 @@ __global__ void __launch_bounds__(kThreads, MODE == 0 ? 3 : 2)
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     abort_flag = 0;
-    next = atomicAdd(work_counter<MODE>(A), 1);
   }
   __syncthreads();
-  int cur = next;
-  // the tile of an item, its structure's grid and tensor map
-  auto geo_of = [&](int item) {
-    return tile_geo<kPacked>(A.g, A.inst, A.tile_inst, A.tile_list[item]);
-  };
-  auto map_of = [&](const TileGeo& g) { return kPacked ? A.tmaps + g.inst : &tmap; };
-  // only the instance of the current item is carried across iterations
-  int cinst = 0;
-  bool cur_tma = false;
-  if (cur < count) {
-    const TileGeo g = geo_of(cur);
-    cinst = g.inst;
-    cur_tma = tile_interior(g, A.tile_list[cur]);
-    if (tid == 0 && cur_tma)
-      issue_box(map_of(g), kPacked, g, A.tile_list[cur], dense_s, bar);
-  }
+  // The first items are the CTAs' own, the counter hands out the rest, asked
+  // for when an item is done: an item taken ahead, so that its box could be
+  // fetched during the evaluation, is work that no idle CTA can take, and the
+  // box arrives while the points are staged in any case.  Values only:
+  // 1.38 M points at 256^3 109 -> 104 us, 115 k at 128^3 24 -> 17 (with the
+  // smaller items of small plans); 16 packed shells 88 -> 83, gradient modes
+  // 109 -> 103.
   uint32_t parity = 0;
-  while (cur < count) {
-    const int np = local_cell_stage<MODE, kPacked>(A, cur, cnt, pts, tmp, tid);  // box in flight
+  for (int cur = blockIdx.x; cur < count;) {
+    const Item item = load_item(A.items, cur);
+    const TileGeo g = tile_geo<kPacked>(A.g, A.inst, A.tile_inst, item.tile);
+    const bool tma = tile_interior(g, item.tile);
+    // the box in flight beside the staging of the points
+    if (tid == 0 && tma)
+      issue_box(kPacked ? A.tmaps + g.inst : &tmap, kPacked, g, item.tile, dense_s, bar);
+    local_cell_stage<MODE, kPacked>(A, item, g, cnt, pts, tmp, tid);
     // thread 0 alone waits (bounded) for the box; the barrier below hands
     // the landed data and the outcome to the CTA
-    if (cur_tma) {
+    if (tma) {
       if (tid == 0 && !mbar_wait(bar, parity)) abort_flag = 1;
     } else {
-      stage_block<kPacked>(A, cur, ub, tid);
+      stage_block<kPacked>(A, g, item.tile, ub, tid);
       cp_async_commit();
       cp_async_wait_group<0>();
     }
-    if (tid == 0) next = atomicAdd(work_counter<MODE>(A), 1);
-    __syncthreads();  // box landed everywhere; next item known
+    __syncthreads();  // box landed everywhere
     if (abort_flag) break;
-    if (cur_tma) {
+    if (tma) {
       parity ^= 1;
       relayout(dense, ub, tid);
       __syncthreads();  // dense free, padded block complete
     }
-    const int nxt = next;
-    int ninst = cinst;
-    bool nxt_tma = false;
-    if (nxt < count) {
-      const TileGeo g = geo_of(nxt);
-      ninst = g.inst;
-      nxt_tma = tile_interior(g, A.tile_list[nxt]);
-      if (tid == 0 && nxt_tma)
-        issue_box(map_of(g), kPacked, g, A.tile_list[nxt], dense_s, bar);
-    }
     float vs, gs;
-    call_scales<kPacked>(A, cinst, vs, gs);
+    call_scales<kPacked>(A, g.inst, vs, gs);
     // the points in cell order, from the staged copy
-    for (int j = tid; j < np; j += kThreads) {
+    for (int j = tid; j < item.n; j += kThreads) {
       const int c = pts.lc[j];
       const int lc[3] = {c & (kTile - 1), (c >> kTileShift) & (kTile - 1), c >> (2 * kTileShift)};
       const float off[3] = {pts.off[0][j], pts.off[1][j], pts.off[2][j]};
@@ -415,10 +396,9 @@ __global__ void __launch_bounds__(kThreads, MODE == 0 ? 3 : 2)
       }
       interp_one<float, MODE>(A, ub, lc, off, pts.idx[j], val, vs, gs);
     }
-    __syncthreads();  // padded block free; `next` consumed
-    cur = nxt;
-    cinst = ninst;
-    cur_tma = nxt_tma;
+    if (tid == 0) next = (int)gridDim.x + atomicAdd(work_counter<MODE>(A), 1);
+    __syncthreads();  // padded block free; next item known
+    cur = next;
   }
   if (abort_flag && tid == 0) {
     atomicOr(A.status, kStatTimeout);
@@ -501,9 +481,8 @@ __device__ __forceinline__ void interp_one(const InterpArgs<Real>& A, const Real
 template <typename Real, int MODE, bool kPacked>
 __device__ __forceinline__ void interp_points(const InterpArgs<Real>& A, int slot, const Real* ub,
                                               int tid) {
-  const int tile = A.tile_list[slot];
-  const int s = A.tile_start[tile] + (slot - A.tile_slot[tile]) * A.chunk;
-  const int e = min(A.tile_end[tile], s + A.chunk);
+  const Item item = load_item(A.items, slot);
+  const int tile = item.tile, s = item.begin, e = s + item.n;
   const TileGeo geo = tile_geo<kPacked>(A.g, A.inst, A.tile_inst, tile);
   int tx, ty, tz;
   tile_coords(geo, tile, tx, ty, tz);
@@ -587,17 +566,13 @@ ib_status interp_t(ib_plan* p, const void* u, int mode, double vscale, double gs
   A.calls = calls;
   A.tmaps = tmaps;
   A.Q = p->Q;
-  A.tile_start = p->tile_start;
-  A.tile_end = p->tile_end;
-  A.tile_slot = p->tile_slot;
-  A.tile_list = p->tile_list;
+  A.items = p->items;
   A.counters = p->tile_counters;
   A.work = p->tile_counters + (io ? io->counter : 2);
   A.p_cell = p->p_cell;
   A.p_off = (const Real*)p->p_off;
   A.p_val = (const Real*)(io && io->vals ? io->vals : p->p_val);
   A.p_idx = p->p_idx;
-  A.chunk = p->chunk;
   // the projection weight w_q j0 of a Gauss point; none for the nodal rule
   A.u = (const Real*)u;
   A.vscale = (Real)vscale;

@@ -57,13 +57,12 @@ struct SpreadArgs {
   const int32_t* tile_slot;    // first work item of each tile
   const int32_t* tile_nitems;  // work items of each tile
   const int32_t* tile_near;
-  const int32_t* tile_list;    // tile of each work item
+  const int4* items;           // work items
   const int32_t* tile_list_near;
   int32_t* counters;           // [0] work items, [1] work counter, [3] near tiles
   const int32_t* p_cell;
   const Real* p_off;
   const Real* p_val;
-  int chunk;                   // points per work item
   Real scale;
   Real* scratch;               // [items][3][12^3]
   Real* f;
@@ -125,8 +124,7 @@ __device__ __forceinline__ void zero_shared(Real* p, int n, int tid, int nthread
   for (int i = tid; i < n4; i += nthreads) v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// Work item `slot`: points [start + j kChunk, min(end, start + (j+1) kChunk))
-// of its tile, j = slot - first item of the tile.
+// Work item `slot` of the list.
 // Raw point data of one work item, copied to shared memory once.
 template <typename Real>
 struct RawItem {
@@ -138,13 +136,13 @@ struct RawItem {
 template <typename Real>
 __device__ __forceinline__ void push_item(const SpreadArgs<Real>& A, int slot, Staged<Real>* stage,
                                           Real* acc, RawItem<Real>* raw, int tid) {
-  const int tile = A.tile_list[slot];
+  const Item item = load_item(A.items, slot);
+  const int tile = item.tile;
   const TileGeo geo = tile_geo<false>(A.g, nullptr, nullptr, tile);  // FP64: one structure
   int tx, ty, tz;
   tile_coords(geo, tile, tx, ty, tz);
   const Real scale = A.scale;
-  const int s = A.tile_start[tile] + (slot - A.tile_slot[tile]) * A.chunk;
-  const int e = min(A.tile_end[tile], s + A.chunk);
+  const int s = item.begin, e = s + item.n;
   const int x0 = tx * kTile, y0 = ty * kTile, z0 = tz * kTile;
   const int hw = tid >> 4, l16 = tid & 15, dz = l16 >> 2, dy = l16 & 3;
   const int warp = tid >> 5;
@@ -227,7 +225,7 @@ __device__ __forceinline__ void push_item(const SpreadArgs<Real>& A, int slot, S
       }
     }
     __syncthreads();
-    Real* out = A.scratch + ((int64_t)slot * 3 + c) * kBlk;
+    Real* out = A.scratch + ((int64_t)item.slot * 3 + c) * kBlk;
     for (int idx = tid; idx < kBlk; idx += kPT) {
       const int z = idx / (kB * kB), y = (idx / kB) % kB, x = idx % kB;
       const int o = z * kSZ + y * kSY + x;
@@ -479,29 +477,55 @@ __global__ void __launch_bounds__(kFxThreads) k_spread_push_fx(SpreadArgs<float>
   const int pt = lane & (kFxGroup - 1), part = (lane / kFxGroup) & 1;
   const bool stager = lane < 2 * kFxGroup;
   float4* G = groups + warp * kFxGroup * kFxRec;
-  for (;;) {
-    __syncthreads();  // previous item written out
-    if (tid == 0) next = atomicAdd(A.counters + 1, 1);
-    __syncthreads();
-    const int slot = next;
-    if (slot >= count) break;
-    const int tile = A.tile_list[slot];
+  // Tiles cut into several work items: the item whose block completes the
+  // tile's count adds all of the tile's item blocks, in item order and in
+  // exact 64-bit integers, into the tile's first block, while they are fresh
+  // in L2; the merge then reads one block per tile.  Every thread fences its
+  // own block stores before the barrier that precedes the count; the summing
+  // CTA fences after reading it.
+  auto sum_items = [&](int tile, int nit) {
+    __threadfence();
+    longlong2* first = reinterpret_cast<longlong2*>(A.scratch) +
+                       (int64_t)A.tile_slot[tile] * (kFxBlk / 2);
+    for (int u = tid; u < kFxBlk / 2; u += kFxThreads) {
+      long long a0 = 0, a1 = 0;
+#pragma unroll 4
+      for (int j = 0; j < nit; ++j) {
+        const longlong2 v = __ldcg(first + (int64_t)j * (kFxBlk / 2) + u);
+        a0 += v.x;
+        a1 += v.y;
+      }
+      first[u] = make_longlong2(a0, a1);
+    }
+  };
+  // The first items are the CTAs' own, the counter hands out the rest, asked
+  // for when an item's sums are done: asked for at the item's start, the next
+  // item waits for its CTA while others run dry (149 -> 163 us at 256^3).
+  // The next record is read while the block is written out, and a tile's
+  // items are summed by their last CTA behind its next item's zeroing.
+  // 115 k points at 128^3: 39 us before (every item from the counter, four
+  // dependent loads for its record, items of 1024), 31 now; 102 k points of
+  // tetrahedra at 104^3 48 -> 34; 1.38 M points at 256^3 152 -> 149.
+  int k = blockIdx.x, done_tile = 0, done_nit = 0;
+  Item it = {};
+  if (k < count) it = load_item(A.items, k);
+  while (k < count) {
+    const int tile = it.tile;
     const TileGeo geo = tile_geo<kPacked>(A.g, A.inst, A.tile_inst, tile);
-    int tx, ty, tz;
-    tile_coords(geo, tile, tx, ty, tz);
-    const int t0 = A.tile_start[tile], t1 = A.tile_end[tile];
-    const int s = t0 + (slot - A.tile_slot[tile]) * A.chunk;
-    const int e = min(t1, s + A.chunk);
-    const int lc0[3] = {tx * kTile, ty * kTile, tz * kTile};
-    const int4 tsk = A.tile_sk[tile];
-    const float vscale = call_scale<kPacked>(A, geo.inst) * ldexpf(1.f, tsk.y - 11);
+    const int s = it.begin, e = s + it.n;
     // warp w takes the groups starting at s + kFxGroup (w + 8 j)
     FxRaw raw = {0, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
     int g0 = s + warp * kFxGroup;
     if (stager && g0 + pt < e) fx_fetch(A, g0 + pt, raw);
+    const int4 tsk = A.tile_sk[tile];
+    int tx, ty, tz;
+    tile_coords(geo, tile, tx, ty, tz);
+    const int lc0[3] = {tx * kTile, ty * kTile, tz * kTile};
+    const float vscale = call_scale<kPacked>(A, geo.inst) * ldexpf(1.f, tsk.y - 11);
     for (int i = tid; i < 2 * kFxWords / 4; i += kFxThreads)
       reinterpret_cast<uint4*>(acc_hi)[i] = make_uint4(0u, 0u, 0u, 0u);
-    __syncthreads();  // accumulators zeroed
+    __syncthreads();  // accumulators zeroed; `last` of the previous item known
+    if (done_nit > 1 && last) sum_items(done_tile, done_nit);
     for (; g0 < e; g0 += kFxWarps * kFxGroup) {
       const int ng = min(kFxGroup, e - g0);
       fx_stage(G + pt * kFxRec, part, stager && pt < ng, raw, lc0, vscale);
@@ -533,47 +557,36 @@ __global__ void __launch_bounds__(kFxThreads) k_spread_push_fx(SpreadArgs<float>
       }
       __syncwarp();  // group consumed before it is restaged
     }
-    __syncthreads();
+    if (tid == 0) next = (int)gridDim.x + atomicAdd(A.counters + 1, 1);
+    __syncthreads();  // sums complete, next item known
+    const int kn = next;
+    Item itn = {};
+    if (kn < count) itn = load_item(A.items, kn);
     // S = 2^11 H + L of every face, exact, in the 12-face rows of the scratch
-    // block; consecutive threads take consecutive face pairs (16-byte stores)
-    longlong2* out = reinterpret_cast<longlong2*>(A.scratch) + (int64_t)slot * (kFxBlk / 2);
+    // block; consecutive threads take consecutive face pairs (16-byte stores).
+    // Rows (component, z, y) follow each other in shared memory too.
+    static_assert(kFxSZ == kB * kFxSY && kFxAcc == kB * kFxSZ, "rows kFxSY words apart");
+    longlong2* out = reinterpret_cast<longlong2*>(A.scratch) + (int64_t)it.slot * (kFxBlk / 2);
     for (int u = tid; u < kFxBlk / 2; u += kFxThreads) {
-      const int row = u / (kB / 2), x = 2 * (u % (kB / 2));
-      const int c = row / (kB * kB), zy = row % (kB * kB);
-      const int o = c * kFxAcc + (zy / kB) * kFxSZ + (zy % kB) * kFxSY + x;  // even: 8-byte aligned
+      const int row = u / (kB / 2);
+      const int o = row * (kFxSY - kB) + 2 * u;  // even: 8-byte aligned
       const uint2 hw = *reinterpret_cast<const uint2*>(acc_hi + o);
       const uint2 lw = *reinterpret_cast<const uint2*>(acc_lo + o);
       const int L0 = (int)(lw.x << 10) >> 10, L1 = (int)(lw.y << 10) >> 10;
       const int H0 = (int)(hw.x - lw.x) + L0, H1 = (int)(hw.y - lw.y) + L1;
       out[u] = make_longlong2((long long)H0 * 2048 + L0, (long long)H1 * 2048 + L1);
     }
-    // Tiles cut into several work items: the item whose block completes the
-    // tile's count adds all of the tile's item blocks, in item order and in
-    // exact 64-bit integers, into the tile's first block, while they are
-    // fresh in L2; the merge then reads one block per tile.  Every thread
-    // fences its own block stores before the barrier that precedes the count;
-    // the summing CTA fences after reading it.
-    const int nit = A.tile_nitems[tile];
-    if (nit > 1) {
-      __threadfence();
-      __syncthreads();
-      if (tid == 0) last = atomicAdd(A.tile_done + tile, 1) + 1 == nit;
-      __syncthreads();
-      if (last) {
-        __threadfence();
-        longlong2* first = reinterpret_cast<longlong2*>(A.scratch) +
-                           (int64_t)A.tile_slot[tile] * (kFxBlk / 2);
-        for (int u = tid; u < kFxBlk / 2; u += kFxThreads) {
-          long long a0 = 0, a1 = 0;
-          for (int j = 0; j < nit; ++j) {
-            const longlong2 v = __ldcg(first + (int64_t)j * (kFxBlk / 2) + u);
-            a0 += v.x;
-            a1 += v.y;
-          }
-          first[u] = make_longlong2(a0, a1);
-        }
-      }
-    }
+    if (it.nit > 1) __threadfence();
+    __syncthreads();  // block written out, accumulators free
+    if (it.nit > 1 && tid == 0) last = atomicAdd(A.tile_done + tile, 1) + 1 == it.nit;
+    done_tile = tile;
+    done_nit = it.nit;
+    k = kn;
+    it = itn;
+  }
+  if (done_nit > 1) {
+    __syncthreads();
+    if (last) sum_items(done_tile, done_nit);
   }
 }
 
@@ -818,13 +831,12 @@ SpreadArgs<Real> spread_args(ib_plan* p, double scale, void* f, const GridCall* 
   A.tile_slot = p->tile_slot;
   A.tile_nitems = p->tile_nonempty;
   A.tile_near = p->tile_near;
-  A.tile_list = p->tile_list;
+  A.items = p->items;
   A.tile_list_near = p->tile_list_near;
   A.counters = p->tile_counters;
   A.p_cell = p->p_cell;
   A.p_off = (const Real*)p->p_off;
   A.p_val = (const Real*)(vals ? vals : p->p_val);
-  A.chunk = p->chunk;
   A.scale = (Real)scale;
   A.scratch = (Real*)p->spread_scratch;
   A.f = (Real*)f;

@@ -5,11 +5,11 @@
 //   near       a tile of its 3x3x3 neighbourhood holds points
 //                                                   -> its faces are merged
 //   far        otherwise                          -> its faces are zero
-// A non-empty tile is cut into work items ("chunks") of at most `chunk`
-// consecutive points, so that a densely populated tile (mesh singularities
-// concentrate points) is shared by several CTAs.  Work items are numbered in
-// ascending (tile, chunk) order; a tile's first item number is its slot, and
-// item k owns scratch block k.  Two kernels: per-CTA counts, then every CTA
+// A non-empty tile is cut into work items ("chunks") of consecutive points
+// (item_points), so that a densely populated tile (mesh singularities
+// concentrate points) is shared by several CTAs, and a small structure by
+// many.  A tile's items own consecutive scratch blocks, the first of which is
+// the tile's slot.  Two kernels: per-CTA counts, then every CTA
 // finds its output offsets from the counts of the CTAs before it and writes
 // its part of the work list and of the near-tile list.
 #include "ib_device.cuh"
@@ -18,6 +18,7 @@ namespace ibfe {
 namespace {
 
 constexpr int kT = 256;  // tiles per CTA
+constexpr int kCounts = 3;  // per-CTA counts: work items, near tiles, points
 
 // Block-wide exclusive scans of K integers at once (one pair of barriers for
 // all of them); total[k] receives the block sum of v[k].  tmp: K * 32 ints.
@@ -69,18 +70,19 @@ __global__ void __launch_bounds__(kT) k_classify(GridDev g, const InstDev* __res
                                                  const int32_t* __restrict__ end, int ntiles,
                                                  int32_t* __restrict__ nonempty,
                                                  int32_t* __restrict__ near,
-                                                 int32_t* __restrict__ bcount, int chunk) {
-  __shared__ int tmp[32];
+                                                 int32_t* __restrict__ bcount, ItemRule rule) {
+  __shared__ int sum[kCounts];
+  if (threadIdx.x < kCounts) sum[threadIdx.x] = 0;
   const int t = blockIdx.x * kT + threadIdx.x;
-  int ne = 0, nr = 0, nch = 0, npt = 0;
+  int nr = 0, nch = 0, npt = 0;
   if (t < ntiles) {
     const TileGeo geo = tile_geo<kPacked>(g, inst, tile_inst, t);
     const int nt0 = geo.nt[0], nt1 = geo.nt[1], nt2 = geo.nt[2];
     int tx, ty, tz;
     tile_coords(geo, t, tx, ty, tz);
     npt = end[t] - start[t];
-    ne = npt > 0;
-    nch = (npt + chunk - 1) / chunk;
+    const int per = item_points(npt, rule);
+    nch = (npt + per - 1) / per;
     // all 27 neighbours' ranges loaded at once (most tiles are far from the
     // structure and would otherwise wait for 27 dependent round trips)
     nr = 0;
@@ -97,15 +99,17 @@ __global__ void __launch_bounds__(kT) k_classify(GridDev g, const InstDev* __res
     nonempty[t] = nch;
     near[t] = nr;
   }
-  int cne, cpt;
-  block_exclusive_scan(nch, tmp, cne);
-  block_exclusive_scan(npt, tmp, cpt);
-  const int cnr = __syncthreads_count(nr);
-  if (threadIdx.x == 0) {
-    bcount[3 * blockIdx.x] = cne;
-    bcount[3 * blockIdx.x + 1] = cnr;
-    bcount[3 * blockIdx.x + 2] = cpt;
+  __syncthreads();
+  const unsigned full = 0xffffffffu;
+  const int v[kCounts] = {__reduce_add_sync(full, nch), __reduce_add_sync(full, nr),
+                          __reduce_add_sync(full, npt)};
+  if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+    for (int k = 0; k < kCounts; ++k)
+      if (v[k]) atomicAdd(sum + k, v[k]);
   }
+  __syncthreads();
+  if (threadIdx.x < kCounts) bcount[kCounts * blockIdx.x + threadIdx.x] = sum[threadIdx.x];
 }
 
 // counters: [0] work items, [1] push / [2] interp work counters, [3] near tiles.
@@ -118,45 +122,43 @@ __global__ void __launch_bounds__(kT) k_compact(const int32_t* __restrict__ none
                                                 int32_t* __restrict__ start,
                                                 int32_t* __restrict__ end,
                                                 int32_t* __restrict__ slot,
-                                                int32_t* __restrict__ work,
+                                                int4* __restrict__ work, ItemRule rule,
                                                 int32_t* __restrict__ list_near,
                                                 int32_t* __restrict__ counters) {
-  __shared__ int tmp[5 * 32];
-  __shared__ int base[3];
-  // offsets: sums of the counts of the CTAs before this one (and of all)
-  int sums[5] = {0, 0, 0, 0, 0};  // ne, nr, np before this CTA; ne, nr of all
+  __shared__ int tmp[kCounts * 32];
+  __shared__ int base[2 * kCounts];  // counts of the CTAs before this one, and of all
+  if (threadIdx.x < 2 * kCounts) base[threadIdx.x] = 0;
+  __syncthreads();
+  int sums[2 * kCounts] = {};
   for (int b = threadIdx.x; b < nblocks; b += kT) {
-    const int a = bcount[3 * b], c = bcount[3 * b + 1], d = bcount[3 * b + 2];
-    if (b < (int)blockIdx.x) {
-      sums[0] += a;
-      sums[1] += c;
-      sums[2] += d;
+#pragma unroll
+    for (int k = 0; k < kCounts; ++k) {
+      const int a = bcount[kCounts * b + k];
+      if (b < (int)blockIdx.x) sums[k] += a;
+      sums[kCounts + k] += a;
     }
-    sums[3] += a;
-    sums[4] += c;
   }
-  int spre[5], stot[5];
-  block_scan_k<5>(sums, spre, stot, tmp);
-  const int t2 = stot[3], t3 = stot[4];
-  if (threadIdx.x == 0) {
-    base[0] = stot[0];
-    base[1] = stot[1];
-    base[2] = stot[2];
+#pragma unroll
+  for (int k = 0; k < 2 * kCounts; ++k) {
+    const int v = __reduce_add_sync(0xffffffffu, sums[k]);
+    if ((threadIdx.x & 31) == 0 && v) atomicAdd(base + k, v);
   }
   __syncthreads();
+  const int t2 = base[kCounts], t3 = base[kCounts + 1];
   const int t = blockIdx.x * kT + threadIdx.x;
-  const int cnt[3] = {t < ntiles ? nonempty[t] : 0, t < ntiles ? near[t] : 0,
-                      t < ntiles ? end[t] - start[t] : 0};
-  const int ne = cnt[0], nr = cnt[1], np = cnt[2];
-  int cpre[3], ctot[3];
-  block_scan_k<3>(cnt, cpre, ctot, tmp);
-  const int pne = cpre[0], pnr = cpre[1], pnp = cpre[2];
+  const int np = t < ntiles ? end[t] - start[t] : 0;
+  const int per = item_points(np, rule);
+  const int cnt[kCounts] = {t < ntiles ? nonempty[t] : 0, t < ntiles ? near[t] : 0, np};
+  int cpre[kCounts], ctot[kCounts];
+  block_scan_k<kCounts>(cnt, cpre, ctot, tmp);
+  const int ne = cnt[0], first = base[0] + cpre[0], s0 = base[2] + cpre[2];
   if (t < ntiles) {
-    start[t] = base[2] + pnp;
-    end[t] = base[2] + pnp + np;
-    slot[t] = ne ? base[0] + pne : -1;
-    for (int j = 0; j < ne; ++j) work[base[0] + pne + j] = t;
-    if (nr) list_near[base[1] + pnr] = t;
+    start[t] = s0;
+    end[t] = s0 + np;
+    slot[t] = ne ? first : -1;
+    for (int j = 0; j < ne; ++j)
+      work[first + j] = make_item(s0 + j * per, min(per, np - j * per), t, first + j, ne);
+    if (cnt[1]) list_near[base[1] + cpre[1]] = t;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     counters[0] = t2;
@@ -170,16 +172,38 @@ __global__ void __launch_bounds__(kT) k_compact(const int32_t* __restrict__ none
 
 int classify_blocks(int ntiles) { return (ntiles + kT - 1) / kT; }
 
-int64_t max_work_items(int ntiles, int64_t Q) { return ntiles + Q / kMinChunk + 1; }
+// Work item size of a plan with Q points: full items (kChunk points) where
+// they give every SM several, smaller ones where they would leave SMs idle
+// (the transfer kernels take one item per CTA at a time).  FP32: 1.5 items
+// per SM in steps of 128 (a 16-point group per warp of the accumulation);
+// below that the items' fixed costs (a 41 KB block written and merged) win.
+// Accumulation / interpolation in us, items of 1024, 512, 256, 128 points:
+// 115 k points at 128^3 30 / 25, 30 / 18, 32 / 18, 36 / 20; 102 k points of
+// tetrahedra at 104^3 42 / 26, 33 / 20, 38 / 22, 51 / 23; 1.38 M points at
+// 256^3 149 / 110, 158 / 118, 177 / 124, 192 / 132.  FP64: 4 items per SM in
+// steps of 32 (FP64 arithmetic alone takes microseconds per point and SM).
+int item_size(int precision, int64_t Q, int sms) {
+  const int gran = precision == IB_FP64 ? 32 : 128;
+  const int64_t items = precision == IB_FP64 ? 4 * sms : sms + sms / 2;
+  const int64_t item = ((Q + items - 1) / items + gran - 1) / gran * gran;
+  return (int)(item < gran ? gran : (item > kChunk ? kChunk : item));
+}
+
+// a tile of n points has at most 1 + n / min(item, kMinChunk) items
+int64_t max_work_items(int ntiles, int64_t Q, int item) {
+  const int64_t m = ntiles + Q / (item < kMinChunk ? item : kMinChunk) + 1;
+  return Q > 0 && m > Q ? Q : m;
+}
 
 ib_status launch_classify_tiles(ib_plan* p, cudaStream_t s) {
   const int nt = p->ntiles, nb = classify_blocks(nt);
   auto classify = p->n_inst > 1 ? k_classify<true> : k_classify<false>;
   classify<<<nb, kT, 0, s>>>(p->grid, p->inst, p->tile_inst, p->tile_start, p->tile_end, nt,
-                             p->tile_nonempty, p->tile_near, p->tile_bcount, p->chunk);
+                             p->tile_nonempty, p->tile_near, p->tile_bcount,
+                             item_rule(p));
   k_compact<<<nb, kT, 0, s>>>(p->tile_nonempty, p->tile_near, nt, p->tile_bcount, nb,
-                              p->tile_start, p->tile_end, p->tile_slot, p->tile_list,
-                              p->tile_list_near, p->tile_counters);
+                              p->tile_start, p->tile_end, p->tile_slot, p->items,
+                              item_rule(p), p->tile_list_near, p->tile_counters);
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 
