@@ -20,6 +20,8 @@ __global__ void __launch_bounds__(256) k_node_gather(const int32_t* __restrict__
                                                      const Real* __restrict__ scale,
                                                      const Real* add, int N, int E, Real* out,
                                                      Real mul) {
+  chain_wait();
+  chain_next();
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
   Real acc[NC];
@@ -47,6 +49,8 @@ template <typename Real, int NC, int kEl>
 __global__ void __launch_bounds__(256) k_elem_project(const Real* __restrict__ vals,
                                                       const Real* __restrict__ w, int E,
                                                       Real* __restrict__ out) {
+  chain_wait();
+  chain_next();
   using EL = El<kEl>;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= E) return;
@@ -72,6 +76,8 @@ __global__ void __launch_bounds__(256) k_elem_project(const Real* __restrict__ v
 // out[i] = add[i] + src[i] (add optional, may alias out)
 template <typename Real>
 __global__ void k_node_copy(const Real* __restrict__ src, const Real* add, int64_t n, Real* out) {
+  chain_wait();
+  chain_next();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = add ? add[i] + src[i] : src[i];
 }
@@ -167,13 +173,9 @@ ib_status gather_t(ib_plan* p, const void* elem, const void* scale, const void* 
   if (p->N == 0) return IB_OK;
   const int blocks = (p->N + 255) / 256;
   if (nc == 3)
-    k_node_gather<Real, 3><<<blocks, 256, 0, s>>>(p->inc_off, p->inc_idx, (const Real*)elem,
-                                                  (const Real*)scale, (const Real*)add, p->N,
-                                                  p->E, (Real*)out, (Real)mul);
+    chain_launch(k_node_gather<Real, 3>, blocks, 256, 0, s, p->inc_off, p->inc_idx, (const Real*)elem, (const Real*)scale, (const Real*)add, p->N, p->E, (Real*)out, (Real)mul);
   else
-    k_node_gather<Real, 1><<<blocks, 256, 0, s>>>(p->inc_off, p->inc_idx, (const Real*)elem,
-                                                  (const Real*)scale, (const Real*)add, p->N,
-                                                  p->E, (Real*)out, (Real)mul);
+    chain_launch(k_node_gather<Real, 1>, blocks, 256, 0, s, p->inc_off, p->inc_idx, (const Real*)elem, (const Real*)scale, (const Real*)add, p->N, p->E, (Real*)out, (Real)mul);
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 
@@ -185,11 +187,9 @@ ib_status project_t(ib_plan* p, const void* vals, const void* w, void* out, int 
   with_elem(p->elem, [&](auto el) {
     constexpr int kE = decltype(el)::value;
     if (nc == 3)
-      k_elem_project<Real, 3, kE><<<blocks, 256, 0, s>>>((const Real*)vals, (const Real*)w,
-                                                         p->E, (Real*)out);
+      chain_launch(k_elem_project<Real, 3, kE>, blocks, 256, 0, s, (const Real*)vals, (const Real*)w, p->E, (Real*)out);
     else
-      k_elem_project<Real, 1, kE><<<blocks, 256, 0, s>>>((const Real*)vals, (const Real*)w,
-                                                         p->E, (Real*)out);
+      chain_launch(k_elem_project<Real, 1, kE>, blocks, 256, 0, s, (const Real*)vals, (const Real*)w, p->E, (Real*)out);
   });
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
@@ -218,8 +218,7 @@ ib_status static_t(ib_plan* p, cudaStream_t s) {
         k_mass_corner_d<Real, kE><<<(p->E + 255) / 256, 256, 0, s>>>((const Real*)p->wj0, p->E,
                                                                      ed);
       });
-    k_node_gather<double, 1><<<(p->N + 255) / 256, 256, 0, s>>>(
-        p->inc_off, p->inc_idx, ed, nullptr, nullptr, p->N, p->E, md, 1.0);
+    chain_launch(k_node_gather<double, 1>, (p->N + 255) / 256, 256, 0, s, p->inc_off, p->inc_idx, ed, nullptr, nullptr, p->N, p->E, md, 1.0);
     if (sizeof(Real) == 4)
       k_mass_round<<<(p->N + 255) / 256, 256, 0, s>>>(md, (float*)p->mass, (float*)p->inv_mass,
                                                       p->N);
@@ -256,11 +255,9 @@ ib_status launch_node_copy(ib_plan* p, const void* src, void* out, const void* a
   if (n == 0) return IB_OK;
   const unsigned blocks = (unsigned)((n + 255) / 256);
   if (p->precision == IB_FP64)
-    k_node_copy<double><<<blocks, 256, 0, s>>>((const double*)src, (const double*)add, n,
-                                               (double*)out);
+    chain_launch(k_node_copy<double>, blocks, 256, 0, s, (const double*)src, (const double*)add, n, (double*)out);
   else
-    k_node_copy<float><<<blocks, 256, 0, s>>>((const float*)src, (const float*)add, n,
-                                              (float*)out);
+    chain_launch(k_node_copy<float>, blocks, 256, 0, s, (const float*)src, (const float*)add, n, (float*)out);
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 

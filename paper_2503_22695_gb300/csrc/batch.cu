@@ -56,6 +56,8 @@ template <int kMode>
 __global__ void __launch_bounds__(256) k_nodes(const NodeSeg* __restrict__ segs, int64_t N,
                                                int32_t* __restrict__ cell, float* __restrict__ a,
                                                float* __restrict__ b, float* __restrict__ c) {
+  chain_wait();
+  chain_next();
   const NodeSeg sg = segs[blockIdx.y];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= sg.count) return;
@@ -82,6 +84,8 @@ __global__ void __launch_bounds__(256) k_nodes(const NodeSeg* __restrict__ segs,
 // rows per instance (zero past an instance's materials).
 __global__ void k_gparams(const double* __restrict__ ered, const int2* __restrict__ mats,
                           double* __restrict__ out) {
+  chain_wait();
+  chain_next();
   const int i = blockIdx.x;
   const int2 m = mats[i];  // (first packed row, rows)
   for (int k = threadIdx.x; k < IB_MAX_MATERIALS * kParamRow; k += blockDim.x) {
@@ -162,10 +166,10 @@ ib_status run_forward(ib_batch* b, cudaStream_t s) {
   const ib_pos x = packed_pos(b);
   MatTable none;
   std::memset(&none, 0, sizeof(none));
-  k_nodes<kPackPos><<<node_grid(b), 256, 0, s>>>(b->segs, b->N, b->cell, b->off, nullptr, nullptr);
+  chain_launch(k_nodes<kPackPos>, node_grid(b), 256, 0, s, b->segs, b->N, b->cell, b->off, nullptr, nullptr);
   ib_status st = forward_body(b->P, none, &x, b->inst[0].u, b->G, b->inst[0].f, b->U, s, &b->pc);
   if (st == IB_OK)
-    k_nodes<kUnpackFwd><<<node_grid(b), 256, 0, s>>>(b->segs, b->N, nullptr, b->G, b->U, nullptr);
+    chain_launch(k_nodes<kUnpackFwd>, node_grid(b), 256, 0, s, b->segs, b->N, nullptr, b->G, b->U, nullptr);
   return st == IB_OK && ok(cudaGetLastError()) ? IB_OK : (st == IB_OK ? IB_ERR_CUDA : st);
 }
 
@@ -173,9 +177,8 @@ ib_status run_adjoint(ib_batch* b, cudaStream_t s) {
   const ib_pos x = packed_pos(b);
   MatTable none;
   std::memset(&none, 0, sizeof(none));
-  k_nodes<kPackPos><<<node_grid(b), 256, 0, s>>>(b->segs, b->N, b->cell, b->off, nullptr, nullptr);
-  k_nodes<kPackAdj><<<node_grid(b), 256, 0, s>>>(b->segs, b->N, nullptr, b->Gin, b->gU,
-                                                 b->any_gG ? b->gG : nullptr);
+  chain_launch(k_nodes<kPackPos>, node_grid(b), 256, 0, s, b->segs, b->N, b->cell, b->off, nullptr, nullptr);
+  chain_launch(k_nodes<kPackAdj>, node_grid(b), 256, 0, s, b->segs, b->N, nullptr, b->Gin, b->gU, b->any_gG ? b->gG : nullptr);
   // the instances' own fields come from the call tables; the pointers passed
   // here only mark which adjoint terms are wanted
   const ib_instance& i0 = b->inst[0];
@@ -183,9 +186,8 @@ ib_status run_adjoint(ib_batch* b, cudaStream_t s) {
                                b->any_gG ? b->gG : nullptr, i0.gf, b->gU, b->gx, i0.gu,
                                /*params=*/true, nullptr, s, &b->pc);
   if (st == IB_OK) {
-    k_gparams<<<b->n, 128, 0, s>>>(b->P->ered, b->gp_rows, b->gparams);
-    k_nodes<kUnpackAdj><<<node_grid(b), 256, 0, s>>>(b->segs, b->N, nullptr, b->gx, nullptr,
-                                                     nullptr);
+    chain_launch(k_gparams, b->n, 128, 0, s, b->P->ered, b->gp_rows, b->gparams);
+    chain_launch(k_nodes<kUnpackAdj>, node_grid(b), 256, 0, s, b->segs, b->N, nullptr, b->gx, nullptr, nullptr);
   }
   return st == IB_OK && ok(cudaGetLastError()) ? IB_OK : (st == IB_OK ? IB_ERR_CUDA : st);
 }

@@ -36,7 +36,7 @@ void free_plan(ib_plan* p) {
   void* ptrs[] = {p->inc_off, p->inc_idx, p->mass, p->inv_mass, p->wj0, p->elem_scratch,
                   p->elem_scratch2, p->keys[0], p->keys[1], p->vals[0], p->vals[1], p->hist,
                   p->tile_start, p->tile_end, p->tile_slot, p->tile_nonempty, p->tile_near,
-                  p->items, p->tile_list_near, p->tile_vmax, p->tile_done, p->tile_sk, p->tile_bcount, p->tile_counters,
+                  p->items, p->tile_list_near, p->tile_vmax, p->tile_done, p->tile_cnt, p->tile_bcount, p->tile_counters,
                   p->digit_tot, p->rpart, p->red_count, p->spread_scratch, p->q_cell, p->q_off, p->q_val, p->p_cell,
                   p->p_off, p->p_val, p->p_idx, p->vol_jm1, p->gq_a, p->gq_b, p->epart, p->ered,
                   p->dstatus, p->node_tmp, p->pen_part, p->mat_range, p->inst, p->tile_inst,
@@ -166,10 +166,10 @@ struct Stage {
 };
 
 int sort_launches(const ib_plan* p) {
-  // FP32 binning: classify, compact (ranges), scatter.  FP64: radix passes
-  // (hist, digit scan, scatter), bounds, classify, compact, reorder
+  // FP32 binning: classify, compact (ranges), scatter.  FP64: classify,
+  // compact, radix passes (hist, digit scan, scatter), reorder
   if (p->precision != IB_FP64) return 3;
-  return 3 * ((sort_key_bits(p->ntiles) + 7) / 8) + 4;
+  return 3 * ((sort_key_bits(p->ntiles) + 7) / 8) + 3;
 }
 
 // forward pieces shared by the entry points
@@ -406,9 +406,9 @@ ib_status plan_build(const ib_mesh* mesh, const GridDev& grid, int ntiles, int32
               dalloc(&p->tile_list_near, 4 * (size_t)p->ntiles) &&
               dalloc(&p->tile_vmax, 4 * (size_t)p->ntiles) &&
               dalloc(&p->tile_done, 4 * (size_t)p->ntiles) &&
-              dalloc(&p->tile_sk, 16 * (size_t)p->ntiles) &&
+              dalloc(&p->tile_cnt, 4 * (size_t)p->ntiles) &&
               dalloc(&p->tile_bcount, 12 * (size_t)classify_blocks(p->ntiles)) &&
-              dalloc(&p->tile_counters, 32) && dalloc(&p->digit_tot, 4 * 256) &&
+              dalloc(&p->tile_counters, 64) && dalloc(&p->digit_tot, 4 * 256) &&
               dalloc(&p->rpart, 8 * kParamRow * (size_t)mat_cap * kReduceCTAs) &&
               dalloc(&p->red_count, sizeof(int) * (size_t)mat_cap) &&
               dalloc(&p->mat_range, sizeof(int2) * (size_t)mat_cap) &&
@@ -451,6 +451,8 @@ ib_status plan_build(const ib_mesh* mesh, const GridDev& grid, int ntiles, int32
          (E == 0 || ok(cudaMemcpyAsync(p->inc_idx, inc_idx.data(), 4 * nc * E,
                                        cudaMemcpyHostToDevice, s))) &&
          ok(cudaMemsetAsync(p->red_count, 0, sizeof(int) * (size_t)mat_cap, s)) &&
+         ok(cudaMemsetAsync(p->tile_cnt, 0, 4 * (size_t)p->ntiles, s)) &&
+         ok(cudaMemsetAsync(p->tile_counters, 0, 64, s)) &&
          ok(cudaMemsetAsync(p->dstatus, 0, 16, s));
   int least = 0, greatest = 0;  // stream priorities (greatest: numerically lowest)
   if (good)
@@ -561,6 +563,7 @@ ib_status ib_interp(ib_plan* p, const ib_pos* x, const void* u, void* U, void* s
 
 namespace ibfe {
 
+// (U null: without the interpolation)
 ib_status forward_body(ib_plan* p, const MatTable& mt, const ib_pos* x, const void* u, void* G,
                        void* f, void* U, cudaStream_t s, const PackedCalls* pc) {
   // Two branches forked from the caller's stream s.  The critical one -- the
@@ -577,11 +580,6 @@ ib_status forward_body(ib_plan* p, const MatTable& mt, const ib_pos* x, const vo
       (m != s && !ok(cudaStreamWaitEvent(m, p->ev_ffork, 0))))
     return IB_ERR_CUDA;
   ib_status st = do_points_sorted(p, x, nullptr, b);
-  // the spreading's per-tile maxima zeroed here, off the critical stream,
-  // which takes them after waiting for the binning
-  if (st == IB_OK && p->precision != IB_FP64 &&
-      !ok(cudaMemsetAsync(p->tile_vmax, 0, sizeof(uint32_t) * p->ntiles, b)))
-    st = IB_ERR_CUDA;
   if (st == IB_OK && !ok(cudaEventRecord(p->ev_fsorted, b))) st = IB_ERR_CUDA;
   // the far-tile zeros of f (HBM writes) on the side branch, beside the
   // force kernel and ahead of the interpolation
@@ -589,7 +587,7 @@ ib_status forward_body(ib_plan* p, const MatTable& mt, const ib_pos* x, const vo
     p->prof_launches[IB_STAGE_SPREAD] += 1;  // overlapped: not in the spread stage's time
     st = launch_spread_zero(p, f, b, pc ? pc->spread_f : nullptr);
   }
-  if (st == IB_OK) st = do_interp_tail(p, u, U, b, p->elem_scratch2, pc);
+  if (st == IB_OK && U) st = do_interp_tail(p, u, U, b, p->elem_scratch2, pc);
   if (st == IB_OK && !ok(cudaEventRecord(p->ev_fjoin, b))) st = IB_ERR_CUDA;
   if (st == IB_OK) {
     Stage sc(p, IB_STAGE_FORCE, m, 1);
@@ -605,7 +603,7 @@ ib_status forward_body(ib_plan* p, const MatTable& mt, const ib_pos* x, const vo
     Stage sc(p, IB_STAGE_POINTS, m, 2);
     st = launch_point_values(p, G, m);
     if (st == IB_OK && !ok(cudaStreamWaitEvent(m, p->ev_fsorted, 0))) st = IB_ERR_CUDA;
-    if (st == IB_OK) st = launch_permute_values(p, m, true, nullptr, nullptr, false);
+    if (st == IB_OK) st = launch_permute_values(p, m, true);
   }
   if (st == IB_OK)
     st = do_spread(p, 1.0 / (p->grid.h * p->grid.h * p->grid.h), f, m, /*zero_fill=*/false,
@@ -643,16 +641,9 @@ ib_status ib_step(ib_plan* p, ib_fluid* fl, const ib_material* mats, int32_t n_m
   MatTable mt;
   if ((st = make_table(p, mats, n_mats, mt)) != IB_OK) return st;
   cudaStream_t s = S(stream);
-  const double h = p->grid.h;
-  // nodal force of x^n, spread at x^n
-  {
-    Stage sc(p, IB_STAGE_FORCE, s, 1);
-    st = launch_fe_force(p, mt, pos_a(p, x), x->off, p->elem_scratch, false, s);
-  }
-  if (st == IB_OK) st = do_gather(p, p->elem_scratch, nullptr, G, s);
-  if (st == IB_OK) st = launch_penalty(p, x, G, false, s);
-  if (st == IB_OK) st = do_points_sorted(p, x, G, s);
-  if (st == IB_OK) st = do_spread(p, 1.0 / (h * h * h), f, s);
+  // nodal force of x^n, spread at x^n: ib_forward's two branches without the
+  // interpolation
+  st = forward_body(p, mt, x, nullptr, G, f, nullptr, s, nullptr);
   // u^n -> u^{n+1} in place
   if (st == IB_OK) st = fluid_step_async(fl, u, f, u, pr, nullptr, s);
   // U = interpolation of u^{n+1} at the same (binned) points, then x += dt U

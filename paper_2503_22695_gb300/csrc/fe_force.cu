@@ -41,6 +41,7 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce(const T* __restrict__ pa
                                                         const int2* __restrict__ mrange, int E,
                                                         int nvals, double* rpart, int* count,
                                                         double* __restrict__ out) {
+  chain_wait();
   __shared__ double sh[kParamRow][kRedThreads];
   __shared__ bool last;
   const int m = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -229,12 +230,9 @@ ib_status launch_reduce_parts(ib_plan* p, int nvals, int n_mats, cudaStream_t s,
   const dim3 grid(nblk, n_mats);
   // FP32 partials are widened exactly: the sums are those of their doubles
   if (real_parts && p->precision != IB_FP64)
-    k_reduce<float><<<grid, kRedThreads, 0, s>>>(reinterpret_cast<const float*>(p->epart),
-                                                 p->mat_id, p->mat_range, p->E, nvals, p->rpart,
-                                                 p->red_count, out);
+    chain_launch(k_reduce<float>, grid, kRedThreads, 0, s, reinterpret_cast<const float*>(p->epart), p->mat_id, p->mat_range, p->E, nvals, p->rpart, p->red_count, out);
   else
-    k_reduce<double><<<grid, kRedThreads, 0, s>>>(p->epart, p->mat_id, p->mat_range, p->E, nvals,
-                                                  p->rpart, p->red_count, out);
+    chain_launch(k_reduce<double>, grid, kRedThreads, 0, s, p->epart, p->mat_id, p->mat_range, p->E, nvals, p->rpart, p->red_count, out);
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 

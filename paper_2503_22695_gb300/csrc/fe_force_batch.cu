@@ -13,8 +13,7 @@ ib_status fe_run_packed(ib_plan* p, const MatTable& mt, const void* xa, const fl
   const int threads = 128, per_cta = threads / 8;
   const int per_sm = kAdj ? fe8_min_blocks<float, kAdj>() : p->fe_ctas;
   const int blocks = std::min((p->E + per_cta - 1) / per_cta, p->sm_count * per_sm);
-  if (cudaMemsetAsync(A.next, 0, sizeof(int), s) != cudaSuccess) return IB_ERR_CUDA;
-  k_fe8<float, df, false, kAdj, kParams, kLaws, true><<<blocks, threads, 0, s>>>(A, mt);
+  chain_launch(k_fe8<float, df, false, kAdj, kParams, kLaws, true>, blocks, threads, 0, s, A, mt);
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 

@@ -239,6 +239,7 @@ __device__ __forceinline__ df exact_jm1_at(const FeArgs<float>& A, int e) {
 
 template <int kEl>
 __global__ void __launch_bounds__(128) k_exact_jm1(FeArgs<float> A, float2* __restrict__ jx) {
+  chain_wait();
   using EL = El<kEl>;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)EL::QF * A.E) return;
@@ -954,6 +955,12 @@ __device__ __forceinline__ void fe_element(const FeArgs<Real>& A, const MatTable
   }
 }
 
+// The last CTA to run out of blocks zeroes the block counter next[0] and the
+// count of finished CTAs next[2] for the next launch.
+__device__ __forceinline__ void fe_finish(int* next) {
+  if (threadIdx.x == 0 && atomicAdd(next + 2, 1) + 1 == (int)gridDim.x) next[0] = next[2] = 0;
+}
+
 // Persistent grid (a fixed number of CTAs per SM, fewer than fit): the SM
 // room the kernel leaves lets the Gauss-point binning and the interpolation,
 // issued on another stream, run beside it.
@@ -962,6 +969,7 @@ __device__ __forceinline__ void fe_element(const FeArgs<Real>& A, const MatTable
 template <typename Real, typename S, bool kEnergy, bool kAdj, bool kParams, int kLaws, int kEl>
 __global__ void __launch_bounds__(128, fe_min_blocks<Real, kAdj>())
     k_fe(FeArgs<Real> A, MatTable mt) {
+  chain_wait();
   __shared__ int base;
   for (;;) {
     if (threadIdx.x == 0) base = atomicAdd(A.next, 1) * (int)blockDim.x;
@@ -972,6 +980,7 @@ __global__ void __launch_bounds__(128, fe_min_blocks<Real, kAdj>())
     if (b + (int)threadIdx.x < A.E)
       fe_element<Real, S, kEnergy, kAdj, kParams, kLaws, kEl>(A, mt, b + (int)threadIdx.x);
   }
+  fe_finish(A.next);
 }
 
 // Hexahedra: eight lanes per element (lane g: Gauss point g), sixteen
@@ -985,6 +994,7 @@ template <typename Real, typename S, bool kEnergy, bool kAdj, bool kParams, int 
           bool kPacked = false>
 __global__ void __launch_bounds__(128, fe8_min_blocks<Real, kAdj>())
     k_fe8(FeArgs<Real> A, MatTable mt) {
+  chain_wait();
   constexpr int kPer = 128 / 8;
   __shared__ int base;
   for (;;) {
@@ -997,6 +1007,7 @@ __global__ void __launch_bounds__(128, fe8_min_blocks<Real, kAdj>())
     fe_element<Real, S, kEnergy, kAdj, kParams, kLaws, IB_ELEM_HEX8, true, kPacked>(
         A, mt, e < A.E ? e : A.E - 1, e < A.E);
   }
+  fe_finish(A.next);
 }
 
 template <typename Real>
@@ -1086,16 +1097,15 @@ ib_status fe_run(ib_plan* p, const MatTable& mt, const void* xa, const float* of
   const int per_sm = kAdj ? (lanes ? fe8_min_blocks<Real, kAdj>() : fe_min_blocks<Real, kAdj>())
                           : p->fe_ctas;
   const int blocks = std::min((p->E + per_cta - 1) / per_cta, p->sm_count * per_sm);
-  if (cudaMemsetAsync(A.next, 0, sizeof(int), s) != cudaSuccess) return IB_ERR_CUDA;
   if constexpr ((kLaws & kLawVolX) != 0) {
     if (!p->vol_jm1) return IB_ERR_INVALID_ARG;
     const int64_t n = (int64_t)El<kEl>::QF * p->E;
-    k_exact_jm1<kEl><<<(unsigned)((n + 127) / 128), 128, 0, s>>>(A, (float2*)p->vol_jm1);
+    chain_launch(k_exact_jm1<kEl>, (unsigned)((n + 127) / 128), 128, 0, s, A, (float2*)p->vol_jm1);
   }
   if constexpr (lanes)
-    k_fe8<Real, S, kEnergy, kAdj, kParams, kLaws><<<blocks, threads, 0, s>>>(A, mt);
+    chain_launch(k_fe8<Real, S, kEnergy, kAdj, kParams, kLaws>, blocks, threads, 0, s, A, mt);
   else
-    k_fe<Real, S, kEnergy, kAdj, kParams, kLaws, kEl><<<blocks, threads, 0, s>>>(A, mt);
+    chain_launch(k_fe<Real, S, kEnergy, kAdj, kParams, kLaws, kEl>, blocks, threads, 0, s, A, mt);
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 

@@ -494,6 +494,8 @@ __global__ void __launch_bounds__(256) k_advance_split(int32_t* __restrict__ cel
                                                        float* __restrict__ off,
                                                        const float* __restrict__ U, int64_t n,
                                                        float scale) {
+  chain_wait();
+  chain_next();
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n;
        t += (int64_t)gridDim.x * blockDim.x) {
     const float v = off[t] + scale * U[t];
@@ -506,6 +508,8 @@ __global__ void __launch_bounds__(256) k_advance_split(int32_t* __restrict__ cel
 __global__ void __launch_bounds__(256) k_advance_x64(double* __restrict__ x,
                                                      const double* __restrict__ U, int64_t n,
                                                      double dt) {
+  chain_wait();
+  chain_next();
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n;
        t += (int64_t)gridDim.x * blockDim.x)
     x[t] += dt * U[t];
@@ -519,10 +523,9 @@ ib_status launch_advance_positions(ib_plan* p, const ib_pos* x, const void* U, d
   if (n == 0) return IB_OK;
   const int g = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 4096));
   if (p->precision == IB_FP64)
-    k_advance_x64<<<g, 256, 0, s>>>(const_cast<double*>(x->x64), (const double*)U, n, dt);
+    chain_launch(k_advance_x64, g, 256, 0, s, const_cast<double*>(x->x64), (const double*)U, n, dt);
   else
-    k_advance_split<<<g, 256, 0, s>>>(const_cast<int32_t*>(x->cell), const_cast<float*>(x->off),
-                                      (const float*)U, n, (float)(dt / p->grid.h));
+    chain_launch(k_advance_split, g, 256, 0, s, const_cast<int32_t*>(x->cell), const_cast<float*>(x->off), (const float*)U, n, (float)(dt / p->grid.h));
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 

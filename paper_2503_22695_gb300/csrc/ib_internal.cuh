@@ -11,6 +11,38 @@
 
 namespace ibfe {
 
+// Kernel chains: every kernel of the operators' streams is launched with
+// programmatic stream serialisation and begins with chain_wait(), before any
+// access to memory; small kernels then call chain_next(), so that the next
+// kernel of the stream is already resident when they end.  The wait ends when
+// the preceding kernel has completed and its writes are visible (which, as
+// every kernel of the stream waits likewise, holds for all before it).
+// A call on a small structure is a dozen dependent kernels of 2 to 5 us, and
+// the 2 to 4 us between two of them were half its time.  With the memsets of
+// the chains folded into their kernels (one between two kernels would break
+// the chain): forward at 128^3 107 -> 77 us, FP64 block 150 -> 105, nodal
+// spread + interp at 176^3 140 -> 93, 256^3 forward 400 -> 377.  The large
+// kernels (force, accumulation, merge, interpolation, reduction) do not call
+// chain_next: their successors' CTAs would hold SM room from the other branch.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;"); }
+
+template <typename... P, typename... A>
+cudaError_t chain_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                         A&&... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute a[1] = {};
+  a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = a;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 // Calls f(std::integral_constant<int, kEl>) for the plan's element type.
 template <typename F>
 void with_elem(int elem, F&& f) {
@@ -191,11 +223,12 @@ struct ib_plan {
   int32_t* tile_list_near;// [ntiles] near tiles, ascending
   uint32_t* tile_vmax;   // [ntiles] FP32: bits of the largest |carried value| of each tile
   int32_t* tile_done;    // [ntiles] work items of the tile written (FP32 spreading, per call)
-  int32_t* tile_sk;      // [4 ntiles] FP32: first block slot, exponent, item bound, items
   int32_t* tile_bcount;  // [3 * classify CTAs] per-CTA counts
-  int32_t* tile_counters;// [8] [0] work items, [1] push counter, [2] interpolation counter,
-                         //     [3] near count, [4] second interpolation's counter,
-                         //     [6] FE force block counter
+  int32_t* tile_counters;// [16] [0] work items, [1] push counter, [2] interpolation counter,
+                         //      [3] near count, [4] second interpolation's counter, [6] FE
+                         //      force block counter, [8] its finished CTAs; 1, 2, 4, 5 and 7
+                         //      are zeroed by every binning, 6 and 8 by the force kernel
+  int32_t* tile_cnt;     // [ntiles] points counted per tile, zero between binnings
   int32_t* digit_tot;    // [256] radix digit totals
   double* rpart;         // [mat_cap][reduce CTAs][kParamRow] reduction partials
   int* red_count;        // [mat_cap] chunks reduced (zero between calls)
@@ -310,11 +343,9 @@ ib_status launch_sort_points(ib_plan* p, bool with_val, cudaStream_t s);
 // per-tile maxima the FP32 spreading's exponents take).
 ib_status launch_point_values(ib_plan* p, const void* nodal, cudaStream_t s,
                               void* q_out = nullptr);
-// zero_vmax false: the maxima were zeroed by the caller, ahead on the stream
-// (or one it waits for)
+// (the maxima are zeroed by the binning, so one field per binning takes them)
 ib_status launch_permute_values(ib_plan* p, cudaStream_t s, bool vmax = true,
-                                const void* q_in = nullptr, void* p_out = nullptr,
-                                bool zero_vmax = true);
+                                const void* q_in = nullptr, void* p_out = nullptr);
 // The carried values of the nodal field `nodal` at the binned points, into
 // p_out (or p_val), with the per-tile maxima when vmax: FP32 binning in one
 // pass (needs the binning done); FP64 plans through q_tmp (q_val if null)

@@ -51,7 +51,7 @@ struct InterpArgs {
   int64_t Q;
   const int4* items;         // work items
   int32_t* counters;      // [0] work items, [2] the values-only mode's work counter
-  int32_t* work;          // the gradient modes' work counter (zero at launch)
+  int32_t* work;          // the gradient modes' work counter (zeroed by the binning)
   const int32_t* p_cell;
   const Real* p_off;
   const Real* p_val;
@@ -141,6 +141,7 @@ __device__ __forceinline__ int32_t* work_counter(const InterpArgs<Real>& A) {
 
 template <typename Real, int MODE, bool kPacked>
 __global__ void __launch_bounds__(kThreads) k_interp_tile(InterpArgs<Real> A) {
+  chain_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Real* const buf0 = reinterpret_cast<Real*>(smem_raw);
   __shared__ int next;
@@ -332,6 +333,7 @@ __device__ __forceinline__ void local_cell_stage(const InterpArgs<float>& A, con
 template <int MODE, bool kPacked>
 __global__ void __launch_bounds__(kThreads, MODE == 0 ? 3 : 2)
     k_interp_tma(const __grid_constant__ CUtensorMap tmap, InterpArgs<float> A) {
+  chain_wait();
   extern __shared__ unsigned char smem_raw[];
   const uintptr_t base = (reinterpret_cast<uintptr_t>(smem_raw) + kTmaAlign - 1) &
                          ~static_cast<uintptr_t>(kTmaAlign - 1);
@@ -585,7 +587,6 @@ ib_status interp_t(ib_plan* p, const void* u, int mode, double vscale, double gs
   const int cap_ctas = p->interp_per_sm * p->sm_count;
   auto cap = [cap_ctas](int ctas) { return ctas < cap_ctas ? ctas : cap_ctas; };
   const size_t smem = smem_bytes<Real>();
-  cudaMemsetAsync(A.work, 0, sizeof(int32_t), s);
   const bool packed = p->n_inst > 1;
   if constexpr (sizeof(Real) == 4) {
     // packed plans: the instances' maps in device memory (this one unused)
@@ -593,7 +594,7 @@ ib_status interp_t(ib_plan* p, const void* u, int mode, double vscale, double gs
     if (p->interp_tma && (packed ? tmaps != nullptr : make_velocity_map(p->grid.n, u, &tmap))) {
       A.use_tma = 1;
       auto run = [&](auto kernel, int ctas, size_t smem_b) {
-        kernel<<<cap(ctas), kThreads, smem_b, s>>>(tmap, A);
+        chain_launch(kernel, cap(ctas), kThreads, smem_b, s, tmap, A);
       };
       if (mode == 0)
         run(packed ? k_interp_tma<0, true> : k_interp_tma<0, false>, p->interp_ctas_tma[0],
@@ -607,7 +608,9 @@ ib_status interp_t(ib_plan* p, const void* u, int mode, double vscale, double gs
       return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
     }
   }
-  auto run = [&](auto kernel, int ctas) { kernel<<<cap(ctas), kThreads, smem, s>>>(A); };
+  auto run = [&](auto kernel, int ctas) {
+    chain_launch(kernel, cap(ctas), kThreads, smem, s, A);
+  };
   if (mode == 0)
     run(packed ? k_interp_tile<Real, 0, true> : k_interp_tile<Real, 0, false>, p->interp_ctas[0]);
   else if (mode == 1)

@@ -66,6 +66,8 @@ __device__ __forceinline__ double block_sum_pen(double v, double* sh) {
 template <typename Real>
 __global__ void __launch_bounds__(256) k_penalty(PenArgs<Real> A, Real* __restrict__ G,
                                                  double* __restrict__ epart) {
+  chain_wait();
+  chain_next();
   __shared__ double sh[32];
   const int chunk = (A.n + gridDim.x - 1) / gridDim.x;
   const int t0 = blockIdx.x * chunk, t1 = min(A.n, t0 + chunk);
@@ -93,6 +95,8 @@ __global__ void __launch_bounds__(256) k_penalty(PenArgs<Real> A, Real* __restri
 template <typename Real>
 __global__ void __launch_bounds__(256) k_penalty_adj(PenArgs<Real> A, const Real* __restrict__ v,
                                                      Real* __restrict__ Hv, Real mul) {
+  chain_wait();
+  chain_next();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= A.n) return;
   const int a = A.nodes[t];
@@ -104,6 +108,8 @@ __global__ void __launch_bounds__(256) k_penalty_adj(PenArgs<Real> A, const Real
 
 __global__ void __launch_bounds__(64) k_penalty_sum(const double* __restrict__ epart,
                                                     double* __restrict__ out) {
+  chain_wait();
+  chain_next();
   __shared__ double sh[32];
   const double e = block_sum_pen(threadIdx.x < kPenCTAs ? epart[threadIdx.x] : 0.0, sh);
   if (threadIdx.x == 0) *out = e;
@@ -135,10 +141,10 @@ ib_status launch_penalty(ib_plan* p, const ib_pos* x, void* G, bool energy, cuda
   if (!penalty_on(p)) return IB_OK;
   double* ep = energy ? p->pen_part : nullptr;
   if (p->precision == IB_FP64)
-    k_penalty<double><<<kPenCTAs, 256, 0, s>>>(pen_args<double>(p, x), (double*)G, ep);
+    chain_launch(k_penalty<double>, kPenCTAs, 256, 0, s, pen_args<double>(p, x), (double*)G, ep);
   else
-    k_penalty<float><<<kPenCTAs, 256, 0, s>>>(pen_args<float>(p, x), (float*)G, ep);
-  if (energy) k_penalty_sum<<<1, 64, 0, s>>>(p->pen_part, p->pen_part + kPenCTAs);
+    chain_launch(k_penalty<float>, kPenCTAs, 256, 0, s, pen_args<float>(p, x), (float*)G, ep);
+  if (energy) chain_launch(k_penalty_sum, 1, 64, 0, s, p->pen_part, p->pen_part + kPenCTAs);
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 
@@ -149,11 +155,9 @@ ib_status launch_penalty_adj(ib_plan* p, const void* v, void* Hv, cudaStream_t s
   const int g = (p->pen_n + 255) / 256;
   ib_pos none{nullptr, nullptr, nullptr, 0.0};
   if (p->precision == IB_FP64)
-    k_penalty_adj<double><<<g, 256, 0, s>>>(pen_args<double>(p, &none), (const double*)v,
-                                            (double*)Hv, mul);
+    chain_launch(k_penalty_adj<double>, g, 256, 0, s, pen_args<double>(p, &none), (const double*)v, (double*)Hv, mul);
   else
-    k_penalty_adj<float><<<g, 256, 0, s>>>(pen_args<float>(p, &none), (const float*)v,
-                                           (float*)Hv, (float)mul);
+    chain_launch(k_penalty_adj<float>, g, 256, 0, s, pen_args<float>(p, &none), (const float*)v, (float*)Hv, (float)mul);
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 

@@ -5,15 +5,14 @@
 //   V_q   = w_q j0 sum_a N_a(xi_q) V_a / m_a   (optional carried value; for the
 //           spreading of Section 4.4 V = G, the lumped projection of the nodal
 //           forces onto the FE space)
-// and the sort key tile * 512 + cell-in-tile of the (periodically wrapped)
-// cell containing chi_q, for 8^3-cell Eulerian tiles.  The points are then
-// ordered by a stable LSD radix sort on that key (8-bit digits, per-block
-// digit histograms, a per-digit scan across blocks, stable in-block ranks from
-// warp match masks): points are grouped by tile, ordered by cell inside a tile
-// (so neighbouring threads read neighbouring faces), and equal keys keep gq
-// order, so the sorted sequence -- hence every downstream summation order --
-// is identical on every call.  That path serves FP64 plans, whose spreading
-// sums doubles in point order.
+// and the 8^3-cell Eulerian tile of the (periodically wrapped) cell containing
+// chi_q, counting each tile's points.  The points are then ordered by a stable
+// LSD radix sort on the tile (8-bit digits, per-block digit histograms, a
+// per-digit scan across blocks, stable in-block ranks from warp match masks):
+// points are grouped by tile and keep gq order inside it, so the sorted
+// sequence -- hence every downstream summation order -- is identical on every
+// call.  That path serves FP64 plans, whose spreading sums doubles in point
+// order.
 //
 // FP32 plans bin instead of sorting: their spreading accumulates exact
 // integers and their interpolation is per point, so a point's place inside
@@ -29,7 +28,6 @@ namespace {
 constexpr int kSortThreads = 256;
 constexpr int kSortItems = 16;
 constexpr int kSortChunk = kSortThreads * kSortItems;
-constexpr int kLocalBits = 9;  // cell within an 8^3 tile
 
 template <typename Real>
 struct PtArgs {
@@ -48,12 +46,13 @@ struct PtArgs {
   Real* q_val;           // [3][Q]
   uint32_t* key;
   int32_t* val;
-  int32_t* count;        // binning: points per tile
+  int32_t* count;        // points per tile (zero at launch)
   int* status;
 };
 
-// Packed cell, and the tile key with either the point's slot in its tile
-// (binning: one atomic per distinct tile of the warp) or its index (sorting).
+// Packed cell, the tile and its point count (one atomic per distinct tile of
+// the warp), with either the point's slot in its tile (binning) or its index
+// (sorting).
 template <typename Real, bool kBin>
 __device__ __forceinline__ void bin_point(const PtArgs<Real>& A, int64_t gq, const int cw[3],
                                           const TileGeo& geo) {
@@ -61,18 +60,16 @@ __device__ __forceinline__ void bin_point(const PtArgs<Real>& A, int64_t gq, con
   const uint32_t tile = (uint32_t)(geo.base + (cw[0] >> kTileShift) +
                                    geo.nt[0] * ((cw[1] >> kTileShift) +
                                                 geo.nt[1] * (cw[2] >> kTileShift)));
+  const unsigned act = __activemask();
+  const unsigned peers = __match_any_sync(act, tile);
+  const int leader = __ffs(peers) - 1, lane = threadIdx.x & 31;
+  int base = 0;
+  if (lane == leader) base = atomicAdd(A.count + tile, __popc(peers));
+  A.key[gq] = tile;
   if (kBin) {
-    const unsigned act = __activemask();
-    const unsigned peers = __match_any_sync(act, tile);
-    const int leader = __ffs(peers) - 1, lane = threadIdx.x & 31;
-    int base = 0;
-    if (lane == leader) base = atomicAdd(A.count + tile, __popc(peers));
     base = __shfl_sync(peers, base, leader);
-    A.key[gq] = tile;
     A.val[gq] = base + __popc(peers & ((1u << lane) - 1u));
   } else {
-    const uint32_t local = (uint32_t)((((cw[2] & 7) << 3) | (cw[1] & 7)) << 3 | (cw[0] & 7));
-    A.key[gq] = (tile << kLocalBits) | local;
     A.val[gq] = (int32_t)gq;
   }
 }
@@ -81,6 +78,8 @@ __device__ __forceinline__ void bin_point(const PtArgs<Real>& A, int64_t gq, con
 // no per-corner values live (fewer registers, more resident warps)
 template <typename Real, bool kBin, int kEl, bool kPacked, bool kVal = true>
 __global__ void __launch_bounds__(128) k_points(PtArgs<Real> A) {
+  chain_wait();
+  chain_next();
   using EL = El<kEl>;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= A.E) return;
@@ -165,6 +164,8 @@ __global__ void __launch_bounds__(128) k_points(PtArgs<Real> A) {
 // chi_a = x_a (gq = a), and a carried value is V_a itself.
 template <typename Real, bool kBin>
 __global__ void __launch_bounds__(256) k_points_nodal(PtArgs<Real> A) {
+  chain_wait();
+  chain_next();
   const int a = blockIdx.x * blockDim.x + threadIdx.x;
   if (a >= A.N) return;
   const int64_t N = A.N;
@@ -206,6 +207,8 @@ __global__ void __launch_bounds__(128) k_point_values(int E, int64_t N,
                                                      const Real* __restrict__ inv_mass,
                                                      const Real* __restrict__ wj0,
                                                      Real* __restrict__ q_val) {
+  chain_wait();
+  chain_next();
   using EL = El<kEl>;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= E) return;
@@ -253,6 +256,8 @@ __global__ void k_permute_values(const int32_t* __restrict__ p_idx, int64_t Q,
                                  const int32_t* __restrict__ p_cell, GridDev g,
                                  const uint32_t* __restrict__ key,
                                  uint32_t* __restrict__ vmax) {
+  chain_wait();
+  chain_next();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= Q) return;
   const int32_t gi = __ldg(p_idx + i);
@@ -287,6 +292,8 @@ __global__ void __launch_bounds__(128) k_point_values_binned(
     const float* __restrict__ inv_mass, const float* __restrict__ wj0,
     const uint32_t* __restrict__ tile, const int32_t* __restrict__ slot,
     const int32_t* __restrict__ start, float* __restrict__ p_val, uint32_t* __restrict__ vmax) {
+  chain_wait();
+  chain_next();
   using EL = El<kEl>;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= E) return;
@@ -331,6 +338,8 @@ constexpr int kWarpItems = kSortItems * 32;
 __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t* __restrict__ key,
                                                              int64_t Q, int shift, int nblk,
                                                              int32_t* __restrict__ hist) {
+  chain_wait();
+  chain_next();
   __shared__ int cnt[256];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   cnt[t] = 0;
@@ -357,6 +366,8 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t* __r
 // per-block counts hist[d*nblk .. d*nblk + nblk), and the digit total.
 __global__ void __launch_bounds__(256) k_digit_scan(int32_t* __restrict__ hist, int nblk,
                                                     int32_t* __restrict__ dtot) {
+  chain_wait();
+  chain_next();
   __shared__ int tmp[32];
   int32_t* h = hist + (int64_t)blockIdx.x * nblk;
   int carry = 0;
@@ -379,6 +390,8 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(
     const uint32_t* __restrict__ kin, const int32_t* __restrict__ vin, int64_t Q, int shift,
     int nblk, const int32_t* __restrict__ offs, const int32_t* __restrict__ dtot,
     uint32_t* __restrict__ kout, int32_t* __restrict__ vout) {
+  chain_wait();
+  chain_next();
   __shared__ int wpos[kSortWarps][256];
   __shared__ int tmp[32];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -439,6 +452,8 @@ __global__ void k_bin_scatter(int64_t Q, const uint32_t* __restrict__ tile,
                               Real* __restrict__ p_off, Real* __restrict__ p_val,
                               int32_t* __restrict__ p_idx, bool with_val,
                               uint32_t* __restrict__ vmax) {
+  chain_wait();
+  chain_next();
   const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= Q) return;
   const uint32_t t = __ldg(tile + g);
@@ -458,21 +473,14 @@ __global__ void k_bin_scatter(int64_t Q, const uint32_t* __restrict__ tile,
   }
 }
 
-__global__ void k_tile_bounds(const uint32_t* __restrict__ key, int64_t Q,
-                              int32_t* __restrict__ start, int32_t* __restrict__ end) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= Q) return;
-  const uint32_t k = key[i] >> kLocalBits;
-  if (i == 0 || (key[i - 1] >> kLocalBits) != k) start[k] = (int32_t)i;
-  if (i == Q - 1 || (key[i + 1] >> kLocalBits) != k) end[k] = (int32_t)(i + 1);
-}
-
 template <typename Real>
 __global__ void k_permute(const int32_t* __restrict__ order, int64_t Q,
                           const int32_t* __restrict__ q_cell, const Real* __restrict__ q_off,
                           const Real* __restrict__ q_val, int32_t* __restrict__ p_cell,
                           Real* __restrict__ p_off, Real* __restrict__ p_val,
                           int32_t* __restrict__ p_idx, bool with_val) {
+  chain_wait();
+  chain_next();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= Q) return;
   const int32_t g = order[i];
@@ -512,11 +520,9 @@ ib_status points_t<float>(ib_plan* p, const void* xa, const float* off, const vo
   A.key = p->keys[0];
   A.val = p->vals[0];
   A.status = p->dstatus;
-  A.count = p->tile_end;
-  cudaMemsetAsync(p->tile_start, 0, sizeof(int32_t) * p->ntiles, s);
-  cudaMemsetAsync(p->tile_end, 0, sizeof(int32_t) * p->ntiles, s);
+  A.count = p->tile_cnt;
   if (p->quad == IB_QUAD_NODAL)
-    k_points_nodal<float, true><<<(p->N + 255) / 256, 256, 0, s>>>(A);
+    chain_launch(k_points_nodal<float, true>, (p->N + 255) / 256, 256, 0, s, A);
   else
     with_elem(p->elem, [&](auto el) {
       constexpr int kE = decltype(el)::value;
@@ -524,7 +530,7 @@ ib_status points_t<float>(ib_plan* p, const void* xa, const float* off, const vo
                                       : k_points<float, true, kE, true, false>)
                              : (nodal ? k_points<float, true, kE, false, true>
                                       : k_points<float, true, kE, false, false>);
-      k<<<(p->E + 127) / 128, 128, 0, s>>>(A);
+      chain_launch(k, (p->E + 127) / 128, 128, 0, s, A);
     });
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
@@ -552,12 +558,12 @@ ib_status points_t<double>(ib_plan* p, const void* xa, const float*, const void*
   A.key = p->keys[0];
   A.val = p->vals[0];
   A.status = p->dstatus;
-  A.count = nullptr;
+  A.count = p->tile_cnt;
   if (p->quad == IB_QUAD_NODAL)
-    k_points_nodal<double, false><<<(p->N + 255) / 256, 256, 0, s>>>(A);
+    chain_launch(k_points_nodal<double, false>, (p->N + 255) / 256, 256, 0, s, A);
   else
     with_elem(p->elem, [&](auto el) {
-      k_points<double, false, decltype(el)::value, false><<<(p->E + 127) / 128, 128, 0, s>>>(A);
+      chain_launch(k_points<double, false, decltype(el)::value, false>, (p->E + 127) / 128, 128, 0, s, A);
     });
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
@@ -574,47 +580,28 @@ ib_status launch_points(ib_plan* p, const void* xa, const float* off, const void
 
 ib_status launch_sort_points(ib_plan* p, bool with_val, cudaStream_t s) {
   const int64_t Q = p->Q;
-  if (p->precision != IB_FP64) {  // binning: counts in tile_end, tile_start zero
-    if (Q == 0) {  // no points were built: no counts either
-      cudaMemsetAsync(p->tile_start, 0, sizeof(int32_t) * p->ntiles, s);
-      cudaMemsetAsync(p->tile_end, 0, sizeof(int32_t) * p->ntiles, s);
-    }
-    if (launch_classify_tiles(p, s) != IB_OK) return IB_ERR_CUDA;  // also the ranges
-    if (Q == 0) return IB_OK;
-    const int nb = (int)((Q + 255) / 256);
-    if (with_val) cudaMemsetAsync(p->tile_vmax, 0, sizeof(uint32_t) * p->ntiles, s);
-    k_bin_scatter<float><<<nb, 256, 0, s>>>(Q, p->keys[0], p->vals[0], p->tile_start, p->q_cell,
-                                            (const float*)p->q_off, (const float*)p->q_val,
-                                            p->p_cell, (float*)p->p_off, (float*)p->p_val,
-                                            p->p_idx, with_val, p->tile_vmax);
+  if (launch_classify_tiles(p, s) != IB_OK) return IB_ERR_CUDA;  // also the ranges
+  if (Q == 0) return IB_OK;
+  const int nb = (int)((Q + 255) / 256);
+  if (p->precision != IB_FP64) {
+    chain_launch(k_bin_scatter<float>, nb, 256, 0, s, Q, p->keys[0], p->vals[0], p->tile_start,
+                 p->q_cell, (const float*)p->q_off, (const float*)p->q_val, p->p_cell,
+                 (float*)p->p_off, (float*)p->p_val, p->p_idx, with_val, p->tile_vmax);
     return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
   }
-  cudaMemsetAsync(p->tile_start, 0, sizeof(int32_t) * p->ntiles, s);
-  cudaMemsetAsync(p->tile_end, 0, sizeof(int32_t) * p->ntiles, s);
-  if (Q == 0) return launch_classify_tiles(p, s);
   const int bits = sort_key_bits(p->ntiles);
   const int nblk = p->hist_blocks;
   int cur = 0;
   for (int shift = 0; shift < bits; shift += 8) {
-    k_radix_hist<<<nblk, kSortThreads, 0, s>>>(p->keys[cur], Q, shift, nblk, p->hist);
-    k_digit_scan<<<256, 256, 0, s>>>(p->hist, nblk, p->digit_tot);
-    k_radix_scatter<<<nblk, kSortThreads, 0, s>>>(p->keys[cur], p->vals[cur], Q, shift, nblk,
-                                                  p->hist, p->digit_tot, p->keys[cur ^ 1],
-                                                  p->vals[cur ^ 1]);
+    chain_launch(k_radix_hist, nblk, kSortThreads, 0, s, p->keys[cur], Q, shift, nblk, p->hist);
+    chain_launch(k_digit_scan, 256, 256, 0, s, p->hist, nblk, p->digit_tot);
+    chain_launch(k_radix_scatter, nblk, kSortThreads, 0, s, p->keys[cur], p->vals[cur], Q, shift,
+                 nblk, p->hist, p->digit_tot, p->keys[cur ^ 1], p->vals[cur ^ 1]);
     cur ^= 1;
   }
-  const int tb = 256;
-  const int nb = (int)((Q + tb - 1) / tb);
-  k_tile_bounds<<<nb, tb, 0, s>>>(p->keys[cur], Q, p->tile_start, p->tile_end);
-  if (launch_classify_tiles(p, s) != IB_OK) return IB_ERR_CUDA;
-  if (p->precision == IB_FP64)
-    k_permute<double><<<nb, tb, 0, s>>>(p->vals[cur], Q, p->q_cell, (const double*)p->q_off,
-                                        (const double*)p->q_val, p->p_cell, (double*)p->p_off,
-                                        (double*)p->p_val, p->p_idx, with_val);
-  else
-    k_permute<float><<<nb, tb, 0, s>>>(p->vals[cur], Q, p->q_cell, (const float*)p->q_off,
-                                       (const float*)p->q_val, p->p_cell, (float*)p->p_off,
-                                       (float*)p->p_val, p->p_idx, with_val);
+  chain_launch(k_permute<double>, nb, 256, 0, s, p->vals[cur], Q, p->q_cell,
+               (const double*)p->q_off, (const double*)p->q_val, p->p_cell, (double*)p->p_off,
+               (double*)p->p_val, p->p_idx, with_val);
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 
@@ -630,34 +617,27 @@ ib_status launch_point_values(ib_plan* p, const void* nodal, cudaStream_t s, voi
   with_elem(p->elem, [&](auto el) {
     constexpr int kE = decltype(el)::value;
     if (p->precision == IB_FP64)
-      k_point_values<double, kE><<<g, 128, 0, s>>>(p->E, p->N, p->conn, (const double*)nodal,
-                                                   (const double*)p->inv_mass,
-                                                   (const double*)p->wj0, (double*)q);
+      chain_launch(k_point_values<double, kE>, g, 128, 0, s, p->E, p->N, p->conn, (const double*)nodal, (const double*)p->inv_mass, (const double*)p->wj0, (double*)q);
     else
-      k_point_values<float, kE><<<g, 128, 0, s>>>(p->E, p->N, p->conn, (const float*)nodal,
-                                                  (const float*)p->inv_mass,
-                                                  (const float*)p->wj0, (float*)q);
+      chain_launch(k_point_values<float, kE>, g, 128, 0, s, p->E, p->N, p->conn, (const float*)nodal, (const float*)p->inv_mass, (const float*)p->wj0, (float*)q);
   });
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 
 ib_status launch_permute_values(ib_plan* p, cudaStream_t s, bool vmax, const void* q_in,
-                                void* p_out, bool zero_vmax) {
+                                void* p_out) {
   if (p->Q == 0) return IB_OK;
   const int nb = (int)((p->Q + 255) / 256);
   const void* const q = q_in ? q_in : p->q_val;
   void* const out = p_out ? p_out : p->p_val;
   if (p->precision == IB_FP64) {
-    k_permute_values<double, false, false><<<nb, 256, 0, s>>>(p->p_idx, p->Q, (const double*)q,
-                                                       (double*)out, p->p_cell, p->grid,
-                                                       nullptr, nullptr);
+    chain_launch(k_permute_values<double, false, false>, nb, 256, 0, s, p->p_idx, p->Q, (const double*)q, (double*)out, p->p_cell, p->grid, nullptr, nullptr);
   } else {
-    if (vmax && zero_vmax) cudaMemsetAsync(p->tile_vmax, 0, sizeof(uint32_t) * p->ntiles, s);
     auto permute = p->n_inst > 1 ? (vmax ? k_permute_values<float, true, true>
                                          : k_permute_values<float, true, false>)
                                   : (vmax ? k_permute_values<float, false, true>
                                           : k_permute_values<float, false, false>);
-    permute<<<nb, 256, 0, s>>>(p->p_idx, p->Q, (const float*)q, (float*)out, p->p_cell,
+    chain_launch(permute, nb, 256, 0, s, p->p_idx, p->Q, (const float*)q, (float*)out, p->p_cell,
                                p->grid, p->keys[0], p->tile_vmax);
   }
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
@@ -673,12 +653,11 @@ ib_status launch_binned_values(ib_plan* p, const void* nodal, cudaStream_t s, bo
     return st == IB_OK ? launch_permute_values(p, s, vmax, q_tmp, p_out) : st;
   }
   float* const out = static_cast<float*>(p_out ? p_out : p->p_val);
-  if (vmax) cudaMemsetAsync(p->tile_vmax, 0, sizeof(uint32_t) * p->ntiles, s);
   const int g = (p->E + 127) / 128;
   with_elem(p->elem, [&](auto el) {
     constexpr int kE = decltype(el)::value;
     auto k = vmax ? k_point_values_binned<kE, true> : k_point_values_binned<kE, false>;
-    k<<<g, 128, 0, s>>>(p->E, p->N, p->conn, (const float*)nodal, (const float*)p->inv_mass,
+    chain_launch(k, g, 128, 0, s, p->E, p->N, p->conn, (const float*)nodal, (const float*)p->inv_mass,
                         (const float*)p->wj0, p->keys[0], p->vals[0], p->tile_start, out,
                         p->tile_vmax);
   });
@@ -694,7 +673,7 @@ int sort_hist_blocks(int64_t Q) { return (int)((Q + kSortChunk - 1) / kSortChunk
 int sort_key_bits(int ntiles) {
   int bits = 1;
   while ((1 << bits) < ntiles) ++bits;
-  return bits + kLocalBits;
+  return bits;
 }
 
 }  // namespace ibfe

@@ -356,6 +356,8 @@ __device__ __forceinline__ void line_passes(const SpecArgs& A, float2* z) {
 template <int kV>
 __global__ void __launch_bounds__(256, 5) k_spec_rhs(SpecArgs A, const float* __restrict__ u,
                                                   const float* __restrict__ f) {
+  chain_wait();
+  chain_next();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* z = reinterpret_cast<float2*>(smem_raw);
   const LineSmem L = line_smem(A, z);
@@ -454,11 +456,13 @@ __global__ void __launch_bounds__(256, 5) k_spec_rhs(SpecArgs A, const float* __
 
 // One line of n1 places x kTX adjacent modes of one field and plane.
 template <bool kInv, bool k16>
-__global__ void __launch_bounds__(256, k16 ? 3 : 5) k_spec_y(SpecArgs A, int tile0) {
+__global__ void __launch_bounds__(256, k16 ? 3 : 5) k_spec_y(SpecArgs A) {
+  chain_wait();
+  chain_next();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int n1 = A.y.n, np = A.y.np;
   const int col = threadIdx.x & (kTX - 1), j0 = threadIdx.x / kTX, step = blockDim.x / kTX;
-  const int kx = (blockIdx.x + tile0) * kTX + col;
+  const int kx = blockIdx.x * kTX + col;
   const GlobalCol g{A.spec + (int64_t)(blockIdx.z * A.z.n + blockIdx.y) * n1 * A.pitch + kx,
                     A.pitch, 0, kx <= A.x.n / 2};
   const SharedCol<kTX> s{reinterpret_cast<float2*>(smem_raw) + col, 0, 0, 0};
@@ -514,11 +518,13 @@ __device__ __forceinline__ void solve_pass(const SpecArgs& A, const SharedCol<kT
 }
 
 template <bool k16>
-__global__ void __launch_bounds__(256, 3) k_spec_solve(SpecArgs A, int tile0) {
+__global__ void __launch_bounds__(256, 3) k_spec_solve(SpecArgs A) {
+  chain_wait();
+  chain_next();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int n2 = A.z.n, np = A.z.np;
   const int col = threadIdx.x & (kTZ - 1), j0 = threadIdx.x / kTZ, step = blockDim.x / kTZ;
-  const int kx = (blockIdx.x + tile0) * kTZ + col;
+  const int kx = blockIdx.x * kTZ + col;
   const bool on = kx <= A.x.n / 2;
   const int plane = A.y.n * A.pitch;
   const GlobalCol g{A.spec + (int64_t)blockIdx.y * A.pitch + kx, plane, (int64_t)n2 * plane, on};
@@ -552,6 +558,8 @@ __global__ void __launch_bounds__(256, 3) k_spec_solve(SpecArgs A, int tile0) {
 template <bool kKeep>
 __global__ void __launch_bounds__(256, 5) k_spec_out(SpecArgs A, const float* u, float* un,
                                                   float* __restrict__ p) {
+  chain_wait();
+  chain_next();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* z = reinterpret_cast<float2*>(smem_raw);
   const LineSmem L = line_smem(A, z);
@@ -859,15 +867,16 @@ ib_status spectral_step(const Spectral* sp, const float* u, const float* f, floa
   const bool y16 = A.y.rad[0] == 16, z16 = A.z.rad[0] == 16;  // radices descend
   // cell pairs by 8-byte loads where the arrays' bases allow (rows are even)
   const bool pairs = ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(f)) & 7) == 0;
-  (pairs ? k_spec_rhs<2> : k_spec_rhs<1>)<<<gx, sp->threads_x, sp->smem_x, s>>>(A, u, f);
-  (y16 ? k_spec_y<false, true> : k_spec_y<false, false>)<<<dim3(ty, n2, 4), sp->threads_y,
-                                                           sp->smem_y, s>>>(A, 0);
-  (z16 ? k_spec_solve<true> : k_spec_solve<false>)<<<dim3(tz, n1), sp->threads_z, sp->smem_z,
-                                                     s>>>(A, 0);
-  (y16 ? k_spec_y<true, true> : k_spec_y<true, false>)<<<dim3(ty, n2, 4), sp->threads_y,
-                                                         sp->smem_y, s>>>(A, 0);
-  (keep ? k_spec_out<true> : k_spec_out<false>)<<<gx, sp->threads_x, sp->smem_x, s>>>(A, u, un,
-                                                                                      p);
+  const dim3 gy(ty, n2, 4), gz(tz, n1);
+  chain_launch(pairs ? k_spec_rhs<2> : k_spec_rhs<1>, gx, sp->threads_x, sp->smem_x, s, A, u, f);
+  chain_launch(y16 ? k_spec_y<false, true> : k_spec_y<false, false>, gy, sp->threads_y,
+               sp->smem_y, s, A);
+  chain_launch(z16 ? k_spec_solve<true> : k_spec_solve<false>, gz, sp->threads_z, sp->smem_z, s,
+               A);
+  chain_launch(y16 ? k_spec_y<true, true> : k_spec_y<true, false>, gy, sp->threads_y, sp->smem_y,
+               s, A);
+  chain_launch(keep ? k_spec_out<true> : k_spec_out<false>, gx, sp->threads_x, sp->smem_x, s, A,
+               u, un, p);
   return ok(cudaGetLastError()) ? IB_OK : IB_ERR_CUDA;
 }
 

@@ -67,8 +67,7 @@ struct SpreadArgs {
   Real* scratch;               // [items][3][12^3]
   Real* f;
   const uint32_t* tile_vmax;   // FP32: bits of max |value| over each tile's points
-  int32_t* tile_done;          // FP32: work items of each tile written in this call
-  int4* tile_sk;               // FP32: (first block slot or -1, exponent k + 11, item bound, items)
+  int32_t* tile_done;          // FP32: work items of each tile written (zeroed by the binning)
 };
 
 // cp.async of 4 bytes global -> shared (completion awaited with cp_async_wait)
@@ -240,6 +239,7 @@ __device__ __forceinline__ void push_item(const SpreadArgs<Real>& A, int slot, S
 
 template <typename Real>
 __global__ void __launch_bounds__(kPT) k_spread_push(SpreadArgs<Real> A) {
+  chain_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Staged<Real>* stage = reinterpret_cast<Staged<Real>*>(smem_raw);
   Real* acc = reinterpret_cast<Real*>(smem_raw + sizeof(Staged<Real>) * kBatch);
@@ -462,6 +462,7 @@ __device__ __forceinline__ long long fx_align(long long v, int sh) {
 
 template <bool kPacked>
 __global__ void __launch_bounds__(kFxThreads) k_spread_push_fx(SpreadArgs<float> A) {
+  chain_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float4* groups = reinterpret_cast<float4*>(smem_raw);
   unsigned* acc_hi = reinterpret_cast<unsigned*>(smem_raw + sizeof(float4) * kFxWarps * kFxGroup *
@@ -517,11 +518,13 @@ __global__ void __launch_bounds__(kFxThreads) k_spread_push_fx(SpreadArgs<float>
     FxRaw raw = {0, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
     int g0 = s + warp * kFxGroup;
     if (stager && g0 + pt < e) fx_fetch(A, g0 + pt, raw);
-    const int4 tsk = A.tile_sk[tile];
+    const uint32_t vmax = A.tile_vmax[tile];
+    const int npts = A.tile_end[tile] - A.tile_start[tile];
     int tx, ty, tz;
     tile_coords(geo, tile, tx, ty, tz);
     const int lc0[3] = {tx * kTile, ty * kTile, tz * kTile};
-    const float vscale = call_scale<kPacked>(A, geo.inst) * ldexpf(1.f, tsk.y - 11);
+    const float scale = call_scale<kPacked>(A, geo.inst);
+    const float vscale = scale * ldexpf(1.f, fx_tile_exp(vmax, npts, scale));
     for (int i = tid; i < 2 * kFxWords / 4; i += kFxThreads)
       reinterpret_cast<uint4*>(acc_hi)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();  // accumulators zeroed; `last` of the previous item known
@@ -590,26 +593,6 @@ __global__ void __launch_bounds__(kFxThreads) k_spread_push_fx(SpreadArgs<float>
   }
 }
 
-// Per tile (FP32 plans), one thread each: the exponent k of its fixed-point
-// words, its first block slot, the bound m = ceil(n / 512) on its work items
-// under any tuning, and its work items; read by every push item of the tile
-// and by the merge of each of its 27 neighbours.  Also zeroes the
-// accumulation's counters (its work counter and the tiles' written items),
-// which saves two memsets ahead of the push.
-template <bool kPacked>
-__global__ void __launch_bounds__(256) k_tile_info(SpreadArgs<float> A, int ntiles) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t == 0) A.counters[1] = 0;  // the accumulation's work counter
-  if (t >= ntiles) return;
-  A.tile_done[t] = 0;             // items of the tile written in this call
-  const int ns = A.tile_nitems[t];
-  const int npts = A.tile_end[t] - A.tile_start[t];
-  const float scale = call_scale<kPacked>(A, kPacked ? __ldg(A.tile_inst + t) : 0);
-  A.tile_sk[t] = make_int4(ns > 0 ? A.tile_slot[t] : -1,
-                           ns > 0 ? fx_tile_exp(__ldg(A.tile_vmax + t), npts, scale) + 11 : 0,
-                           (npts + kMinChunk - 1) / kMinChunk, ns);
-}
-
 // One CTA per near tile, one thread per face pair of each component, no
 // barrier: lanes 0..26 of each warp load the records of the 27 tiles whose
 // blocks cover the tile, the warp reduces the merge exponent
@@ -618,6 +601,7 @@ __global__ void __launch_bounds__(256) k_tile_info(SpreadArgs<float> A, int ntil
 // then, component by component, loads their blocks together and sums them.
 template <bool kPacked>
 __global__ void __launch_bounds__(kMT, 4) k_spread_merge_fx(SpreadArgs<float> A) {
+  chain_wait();
   static_assert(kMT == 8 * 8 * 4, "one thread per face pair of a tile component");
   const unsigned full = 0xffffffffu;
   const int tid = threadIdx.x, lane = tid & 31;
@@ -635,10 +619,17 @@ __global__ void __launch_bounds__(kMT, 4) k_spread_merge_fx(SpreadArgs<float> A)
     const TileGeo geo = tile_geo<kPacked>(A.g, A.inst, A.tile_inst, tile);
     int tx, ty, tz;
     tile_coords(geo, tile, tx, ty, tz);
+    // (first block slot or -1, exponent k + 11, bound on the work items under
+    // any tuning, items) of each source
     int4 r = make_int4(-1, 0, 0, 0);
-    if (lane < 27)
-      r = __ldg(A.tile_sk + tile_of(tx + lane % 3 - 1, ty + (lane / 3) % 3 - 1,
-                                    tz + lane / 9 - 1, geo));
+    if (lane < 27) {
+      const int t = tile_of(tx + lane % 3 - 1, ty + (lane / 3) % 3 - 1, tz + lane / 9 - 1, geo);
+      const int slot = __ldg(A.tile_slot + t), n = __ldg(A.tile_end + t) - __ldg(A.tile_start + t);
+      const uint32_t vmax = __ldg(A.tile_vmax + t);
+      if (n > 0)
+        r = make_int4(slot, fx_tile_exp(vmax, n, call_scale<kPacked>(A, geo.inst)) + 11,
+                      (n + kMinChunk - 1) / kMinChunk, 1);
+    }
     const int kmax = __reduce_max_sync(full, r.w > 0 ? r.y : -1000);
     const int kcap = __reduce_min_sync(full, r.w > 0 ? r.y + 17 - ceil_log2(r.z) : 1000);
     const int kref = min(kmax, kcap);
@@ -704,6 +695,8 @@ __global__ void __launch_bounds__(kMT, 4) k_spread_merge_fx(SpreadArgs<float> A)
 // Far tiles: one warp per tile, 3 components x 64 rows x 16-byte zeros.
 template <typename Real, bool kPacked>
 __global__ void __launch_bounds__(kMT) k_spread_zero(SpreadArgs<Real> A) {
+  chain_wait();
+  chain_next();
   const int lane = threadIdx.x & 31;
   const int tile = blockIdx.x * kMW + (threadIdx.x >> 5);
   if (tile >= A.ntiles || A.tile_near[tile]) return;
@@ -734,6 +727,7 @@ __global__ void __launch_bounds__(kMT) k_spread_zero(SpreadArgs<Real> A) {
 // and adds them face by face in the order (oz, oy, ox).
 template <typename Real>
 __global__ void __launch_bounds__(kMT) k_spread_merge(SpreadArgs<Real> A) {
+  chain_wait();
   __shared__ int src_slot[27], src_n[27];
   const int tid = threadIdx.x;
   const int count = A.counters[3];
@@ -801,19 +795,16 @@ constexpr size_t kFxSmem =
 
 template <bool kPacked>
 void launch_push(ib_plan* p, const SpreadArgs<float>& A, cudaStream_t s) {
-  k_tile_info<kPacked><<<(p->ntiles + 255) / 256, 256, 0, s>>>(A, p->ntiles);
   p->prof_calls[IB_STAGE_SPREAD_PUSH] += 1;
   const int ev = prof_begin(p, IB_STAGE_SPREAD_PUSH, s);
-  k_spread_push_fx<kPacked><<<std::min(p->push_ctas, p->push_per_sm * p->sm_count), kFxThreads,
-                              kFxSmem, s>>>(A);
+  chain_launch(k_spread_push_fx<kPacked>, std::min(p->push_ctas, p->push_per_sm * p->sm_count), kFxThreads, kFxSmem, s, A);
   prof_end(p, ev, s);
 }
 
 template <bool kPacked>
 void launch_push(ib_plan* p, const SpreadArgs<double>& A, cudaStream_t s) {
   static_assert(!kPacked, "packed plans are FP32");
-  k_spread_push<double><<<std::min(p->push_ctas, p->push_per_sm * p->sm_count), kPT,
-                          push_smem<double>(), s>>>(A);
+  chain_launch(k_spread_push<double>, std::min(p->push_ctas, p->push_per_sm * p->sm_count), kPT, push_smem<double>(), s, A);
 }
 
 template <typename Real>
@@ -842,7 +833,6 @@ SpreadArgs<Real> spread_args(ib_plan* p, double scale, void* f, const GridCall* 
   A.f = (Real*)f;
   A.tile_vmax = p->tile_vmax;
   A.tile_done = p->tile_done;
-  A.tile_sk = reinterpret_cast<int4*>(p->tile_sk);
   return A;
 }
 
@@ -850,21 +840,19 @@ template <typename Real, bool kPacked>
 ib_status spread_t(ib_plan* p, double scale, void* f, bool zero_fill, cudaStream_t s,
                    const GridCall* calls, const void* vals) {
   SpreadArgs<Real> A = spread_args<Real>(p, scale, f, calls, vals);
-  // the FP32 accumulation's counter is reset by k_tile_info
-  if constexpr (sizeof(Real) == 8) cudaMemsetAsync(p->tile_counters + 1, 0, sizeof(int32_t), s);
   // far-tile zeros on the side stream, concurrent with the push (unless the
   // caller has already issued them)
   if (zero_fill) {
     cudaEventRecord(p->ev_fork, s);
     cudaStreamWaitEvent(p->zside, p->ev_fork, 0);
-    k_spread_zero<Real, kPacked><<<(p->ntiles + kMW - 1) / kMW, kMT, 0, p->zside>>>(A);
+    chain_launch(k_spread_zero<Real, kPacked>, (p->ntiles + kMW - 1) / kMW, kMT, 0, p->zside, A);
     cudaEventRecord(p->ev_join, p->zside);
   }
   launch_push<kPacked>(p, A, s);
   if constexpr (sizeof(Real) == 4)
-    k_spread_merge_fx<kPacked><<<p->merge_ctas, kMT, 0, s>>>(A);
+    chain_launch(k_spread_merge_fx<kPacked>, p->merge_ctas, kMT, 0, s, A);
   else
-    k_spread_merge<Real><<<p->merge_ctas, kMT, 0, s>>>(A);
+    chain_launch(k_spread_merge<Real>, p->merge_ctas, kMT, 0, s, A);
   if (zero_fill) cudaStreamWaitEvent(s, p->ev_join, 0);
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
@@ -926,8 +914,8 @@ ib_status spread_prepare(ib_plan* p) {
   return p->precision == IB_FP64 ? prepare_t<double>(p) : prepare_t<float>(p);
 }
 
-// zeros, accumulation, merge (FP32: and the merge exponents)
-int spread_launches(int precision) { return precision == IB_FP64 ? 3 : 4; }
+// zeros, accumulation, merge
+int spread_launches(int) { return 3; }
 
 ib_status launch_spread(ib_plan* p, double scale, void* f, cudaStream_t s, bool zero_fill,
                         const GridCall* calls, const void* vals) {
@@ -943,13 +931,13 @@ ib_status launch_spread_zero(ib_plan* p, void* f, cudaStream_t s, const GridCall
   if ((p->n_inst > 1) != (calls != nullptr)) return IB_ERR_INVALID_ARG;
   if (p->precision == IB_FP64) {
     SpreadArgs<double> A = spread_args<double>(p, 1.0, f, calls);
-    k_spread_zero<double, false><<<(p->ntiles + kMW - 1) / kMW, kMT, 0, s>>>(A);
+    chain_launch(k_spread_zero<double, false>, (p->ntiles + kMW - 1) / kMW, kMT, 0, s, A);
   } else {
     SpreadArgs<float> A = spread_args<float>(p, 1.0, f, calls);
     if (p->n_inst > 1)
-      k_spread_zero<float, true><<<(p->ntiles + kMW - 1) / kMW, kMT, 0, s>>>(A);
+      chain_launch(k_spread_zero<float, true>, (p->ntiles + kMW - 1) / kMW, kMT, 0, s, A);
     else
-      k_spread_zero<float, false><<<(p->ntiles + kMW - 1) / kMW, kMT, 0, s>>>(A);
+      chain_launch(k_spread_zero<float, false>, (p->ntiles + kMW - 1) / kMW, kMT, 0, s, A);
   }
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }

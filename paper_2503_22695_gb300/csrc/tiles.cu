@@ -1,5 +1,5 @@
-// Classification of the 8^3-cell Eulerian tiles after the Gauss points have
-// been sorted by tile (the tiles of a packed plan are those of all its
+// Classification of the 8^3-cell Eulerian tiles after the Gauss points of each
+// have been counted (the tiles of a packed plan are those of all its
 // structures, each with the neighbours on its own periodic grid):
 //   non-empty  the tile holds points              -> spread push / interp work
 //   near       a tile of its 3x3x3 neighbourhood holds points
@@ -66,11 +66,12 @@ __device__ __forceinline__ int wrap_one(int i, int n) { return i < 0 ? i + n : (
 template <bool kPacked>
 __global__ void __launch_bounds__(kT) k_classify(GridDev g, const InstDev* __restrict__ inst,
                                                  const int32_t* __restrict__ tile_inst,
-                                                 const int32_t* __restrict__ start,
-                                                 const int32_t* __restrict__ end, int ntiles,
+                                                 const int32_t* __restrict__ points, int ntiles,
                                                  int32_t* __restrict__ nonempty,
                                                  int32_t* __restrict__ near,
                                                  int32_t* __restrict__ bcount, ItemRule rule) {
+  chain_wait();
+  chain_next();
   __shared__ int sum[kCounts];
   if (threadIdx.x < kCounts) sum[threadIdx.x] = 0;
   const int t = blockIdx.x * kT + threadIdx.x;
@@ -80,10 +81,10 @@ __global__ void __launch_bounds__(kT) k_classify(GridDev g, const InstDev* __res
     const int nt0 = geo.nt[0], nt1 = geo.nt[1], nt2 = geo.nt[2];
     int tx, ty, tz;
     tile_coords(geo, t, tx, ty, tz);
-    npt = end[t] - start[t];
+    npt = points[t];
     const int per = item_points(npt, rule);
     nch = (npt + per - 1) / per;
-    // all 27 neighbours' ranges loaded at once (most tiles are far from the
+    // all 27 neighbours' counts loaded at once (most tiles are far from the
     // structure and would otherwise wait for 27 dependent round trips)
     nr = 0;
 #pragma unroll
@@ -94,7 +95,7 @@ __global__ void __launch_bounds__(kT) k_classify(GridDev g, const InstDev* __res
         for (int c = -1; c <= 1; ++c) {
           const int nb = geo.base + wrap_one(tx + c, nt0) +
                          nt0 * (wrap_one(ty + b, nt1) + nt1 * wrap_one(tz + a, nt2));
-          nr |= __ldg(end + nb) > __ldg(start + nb);
+          nr |= __ldg(points + nb) > 0;
         }
     nonempty[t] = nch;
     near[t] = nr;
@@ -112,19 +113,25 @@ __global__ void __launch_bounds__(kT) k_classify(GridDev g, const InstDev* __res
   if (threadIdx.x < kCounts) bcount[kCounts * blockIdx.x + threadIdx.x] = sum[threadIdx.x];
 }
 
-// counters: [0] work items, [1] push / [2] interp work counters, [3] near tiles.
-// Also rewrites the tile point ranges as start = points of the tiles before,
-// end = start + points (the same ranges for sorted points; the ranges
-// themselves for binned points, whose counts arrive as start 0, end n).
+// counters: [0] work items, [3] near tiles; the work counters (1: push; 2, 4, 5,
+// 7: interpolations) are zeroed for the calls that follow this binning, with
+// the tiles' largest values and finished items, and the point counts for the
+// next binning.  The tiles' point ranges: start = points of the tiles before,
+// end = start + points.
 __global__ void __launch_bounds__(kT) k_compact(const int32_t* __restrict__ nonempty,
                                                 const int32_t* __restrict__ near, int ntiles,
                                                 const int32_t* __restrict__ bcount, int nblocks,
+                                                int32_t* __restrict__ points,
+                                                uint32_t* __restrict__ vmax,
+                                                int32_t* __restrict__ done,
                                                 int32_t* __restrict__ start,
                                                 int32_t* __restrict__ end,
                                                 int32_t* __restrict__ slot,
                                                 int4* __restrict__ work, ItemRule rule,
                                                 int32_t* __restrict__ list_near,
                                                 int32_t* __restrict__ counters) {
+  chain_wait();
+  chain_next();
   __shared__ int tmp[kCounts * 32];
   __shared__ int base[2 * kCounts];  // counts of the CTAs before this one, and of all
   if (threadIdx.x < 2 * kCounts) base[threadIdx.x] = 0;
@@ -146,13 +153,16 @@ __global__ void __launch_bounds__(kT) k_compact(const int32_t* __restrict__ none
   __syncthreads();
   const int t2 = base[kCounts], t3 = base[kCounts + 1];
   const int t = blockIdx.x * kT + threadIdx.x;
-  const int np = t < ntiles ? end[t] - start[t] : 0;
+  const int np = t < ntiles ? points[t] : 0;
   const int per = item_points(np, rule);
   const int cnt[kCounts] = {t < ntiles ? nonempty[t] : 0, t < ntiles ? near[t] : 0, np};
   int cpre[kCounts], ctot[kCounts];
   block_scan_k<kCounts>(cnt, cpre, ctot, tmp);
   const int ne = cnt[0], first = base[0] + cpre[0], s0 = base[2] + cpre[2];
   if (t < ntiles) {
+    points[t] = 0;
+    vmax[t] = 0u;
+    done[t] = 0;
     start[t] = s0;
     end[t] = s0 + np;
     slot[t] = ne ? first : -1;
@@ -162,9 +172,8 @@ __global__ void __launch_bounds__(kT) k_compact(const int32_t* __restrict__ none
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     counters[0] = t2;
-    counters[1] = 0;
-    counters[2] = 0;
     counters[3] = t3;
+    counters[1] = counters[2] = counters[4] = counters[5] = counters[7] = 0;
   }
 }
 
@@ -198,12 +207,11 @@ int64_t max_work_items(int ntiles, int64_t Q, int item) {
 ib_status launch_classify_tiles(ib_plan* p, cudaStream_t s) {
   const int nt = p->ntiles, nb = classify_blocks(nt);
   auto classify = p->n_inst > 1 ? k_classify<true> : k_classify<false>;
-  classify<<<nb, kT, 0, s>>>(p->grid, p->inst, p->tile_inst, p->tile_start, p->tile_end, nt,
-                             p->tile_nonempty, p->tile_near, p->tile_bcount,
-                             item_rule(p));
-  k_compact<<<nb, kT, 0, s>>>(p->tile_nonempty, p->tile_near, nt, p->tile_bcount, nb,
-                              p->tile_start, p->tile_end, p->tile_slot, p->items,
-                              item_rule(p), p->tile_list_near, p->tile_counters);
+  chain_launch(classify, nb, kT, 0, s, p->grid, p->inst, p->tile_inst, p->tile_cnt, nt,
+               p->tile_nonempty, p->tile_near, p->tile_bcount, item_rule(p));
+  chain_launch(k_compact, nb, kT, 0, s, p->tile_nonempty, p->tile_near, nt, p->tile_bcount, nb,
+               p->tile_cnt, p->tile_vmax, p->tile_done, p->tile_start, p->tile_end, p->tile_slot,
+               p->items, item_rule(p), p->tile_list_near, p->tile_counters);
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 
