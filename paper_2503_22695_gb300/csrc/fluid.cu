@@ -44,6 +44,7 @@ struct ib_fluid {
   void* lphi[kMaxLevels];  // levels >= 1: correction [3][cells]
   void* lrhs[kMaxLevels];  // levels >= 1: right-hand side [3][cells]
   int cyc_h, cyc_p, pre, post, coarse_sweeps;
+  char* arena;             // the device arrays below
   void* rhs0;              // [3][cells] Helmholtz right-hand side
   void* div;               // [cells] Poisson right-hand side
   void* ptmp;              // [cells] pressure when the caller passes none
@@ -688,20 +689,39 @@ ib_status ib_fluid_create(const ib_grid* grid, int32_t precision, double rho, do
   cudaDeviceGetAttribute(&fl->sm_count, cudaDevAttrMultiProcessorCount, dev);
   bool good = true;
   const int64_t cells = (int64_t)grid->n[0] * grid->n[1] * grid->n[2];
-  good = good && ok(cudaMalloc(&fl->rhs0, 3 * cells * fl->rsize));
-  good = good && ok(cudaMalloc(&fl->div, cells * fl->rsize));
-  good = good && ok(cudaMalloc(&fl->ptmp, cells * fl->rsize));
-  good = good && ok(cudaMalloc(&fl->red, sizeof(double) * (2 * kFluidRedCTAs + 4)));
-  good = good && ok(cudaStreamCreateWithFlags(&fl->cap, cudaStreamNonBlocking));
   {
+    // one allocation, cut into the solver's arrays
     const dim3 blk = block_for(grid->n[0]);
     const dim3 grd = grid_for(grid->n[0], grid->n[1], grid->n[2] * 3, blk);
-    good = good && ok(cudaMalloc(&fl->rpart, sizeof(double) * 2 * grd.x * grd.y * grd.z));
-  }
-  for (int k = 1; good && k < fl->nlev; ++k) {
-    const int64_t c = (int64_t)fl->ln[k][0] * fl->ln[k][1] * fl->ln[k][2];
-    good = ok(cudaMalloc(&fl->lphi[k], 3 * c * fl->rsize)) &&
-           ok(cudaMalloc(&fl->lrhs[k], 3 * c * fl->rsize));
+    size_t total = 0;
+    auto place = [&](size_t bytes) {
+      const size_t at = total;
+      total += (bytes + 255) / 256 * 256;
+      return at;
+    };
+    const size_t rhs0 = place(3 * cells * fl->rsize), div = place(cells * fl->rsize),
+                 ptmp = place(cells * fl->rsize),
+                 red = place(sizeof(double) * (2 * kFluidRedCTAs + 4)),
+                 rpart = place(sizeof(double) * 2 * grd.x * grd.y * grd.z);
+    size_t lphi[ib_fluid::kMaxLevels] = {}, lrhs[ib_fluid::kMaxLevels] = {};
+    for (int k = 1; k < fl->nlev; ++k) {
+      const size_t c = 3 * (size_t)fl->ln[k][0] * fl->ln[k][1] * fl->ln[k][2] * fl->rsize;
+      lphi[k] = place(c);
+      lrhs[k] = place(c);
+    }
+    good = good && ok(cudaMalloc((void**)&fl->arena, total)) &&
+           ok(cudaStreamCreateWithFlags(&fl->cap, cudaStreamNonBlocking));
+    if (good) {
+      fl->rhs0 = fl->arena + rhs0;
+      fl->div = fl->arena + div;
+      fl->ptmp = fl->arena + ptmp;
+      fl->red = reinterpret_cast<double*>(fl->arena + red);
+      fl->rpart = reinterpret_cast<double*>(fl->arena + rpart);
+      for (int k = 1; k < fl->nlev; ++k) {
+        fl->lphi[k] = fl->arena + lphi[k];
+        fl->lrhs[k] = fl->arena + lrhs[k];
+      }
+    }
   }
   if (good) {
     // dynamic shared memory of the coarsest solve: the limit is a property of
@@ -737,15 +757,7 @@ ib_status ib_fluid_destroy(ib_fluid* fl) {
   if (fl->gexec) cudaGraphExecDestroy(fl->gexec);
   if (fl->cap) cudaStreamDestroy(fl->cap);
   spectral_destroy(&fl->spec);
-  cudaFree(fl->rhs0);
-  cudaFree(fl->div);
-  cudaFree(fl->ptmp);
-  cudaFree(fl->red);
-  cudaFree(fl->rpart);
-  for (int k = 0; k < fl->nlev; ++k) {
-    cudaFree(fl->lphi[k]);
-    cudaFree(fl->lrhs[k]);
-  }
+  cudaFree(fl->arena);
   delete fl;
   return IB_OK;
 }

@@ -815,11 +815,10 @@ ib_status spectral_create(Spectral* sp, const int n[3], double h, double rho, do
     }
   }
   A.pitch = (n[0] / 2 + 1 + 3) / 4 * 4;  // rows start on 32-byte sectors
-  const size_t spec = sizeof(float2) * 4 * (size_t)n[2] * n[1] * A.pitch;
-  if (!ok(cudaMalloc(&sp->tables, host.size())) || !ok(cudaMalloc((void**)&A.spec, spec)) ||
-      !ok(cudaMemcpy(sp->tables, host.data(), host.size(), cudaMemcpyHostToDevice)))
-    return IB_ERR_CUDA;
-  const char* t = static_cast<const char*>(sp->tables);
+  const size_t spec = (sizeof(float2) * 4 * (size_t)n[2] * n[1] * A.pitch + 255) / 256 * 256;
+  if (!ok(cudaMalloc((void**)&A.spec, spec + host.size()))) return IB_ERR_CUDA;
+  char* const t = reinterpret_cast<char*>(A.spec) + spec;  // the tables behind the modes
+  if (!ok(cudaMemcpy(t, host.data(), host.size(), cudaMemcpyHostToDevice))) return IB_ERR_CUDA;
   for (int d = 0; d < 3; ++d) dims[d]->tw = reinterpret_cast<const float2*>(t + tw_at[d]);
   A.symx = reinterpret_cast<const float4*>(t + sym_at[0]);
   A.symy = reinterpret_cast<const float4*>(t + sym_at[1]);
@@ -839,22 +838,22 @@ ib_status spectral_create(Spectral* sp, const int n[3], double h, double rho, do
   sp->threads_x = col_threads(n[0], A.x.rad[0], kXL);
   sp->threads_y = col_threads(n[1], A.y.rad[0], kTX);
   sp->threads_z = col_threads(n[2], A.z.rad[0], kTZ);
-  auto opt = [](auto k) {
-    return ok(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)kMaxSmem));
+  // lines longer than the default 48 KB of shared memory holds
+  auto opt = [](size_t smem, auto... k) {
+    return smem <= 48 * 1024 ||
+           (ok(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)kMaxSmem)) && ...);
   };
-  return opt(k_spec_rhs<1>) && opt(k_spec_rhs<2>) && opt(k_spec_out<false>) &&
-                 opt(k_spec_out<true>) && opt(k_spec_y<false, false>) &&
-                 opt(k_spec_y<true, false>) && opt(k_spec_y<false, true>) &&
-                 opt(k_spec_y<true, true>) && opt(k_spec_solve<false>) && opt(k_spec_solve<true>)
+  return opt(sp->smem_x, k_spec_rhs<1>, k_spec_rhs<2>, k_spec_out<false>, k_spec_out<true>) &&
+                 opt(sp->smem_y, k_spec_y<false, false>, k_spec_y<true, false>,
+                     k_spec_y<false, true>, k_spec_y<true, true>) &&
+                 opt(sp->smem_z, k_spec_solve<false>, k_spec_solve<true>)
              ? IB_OK
              : IB_ERR_CUDA;
 }
 
 void spectral_destroy(Spectral* sp) {
-  cudaFree(sp->tables);
   cudaFree(sp->a.spec);
-  sp->tables = nullptr;
   sp->a.spec = nullptr;
 }
 

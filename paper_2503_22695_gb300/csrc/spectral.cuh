@@ -26,7 +26,7 @@ struct SpecArgs {
   // the modes are stored in (x: natural; y, z: digit-reversed)
   const float4 *symx, *symy, *symz;
   const int* posx;       // place of mode k in a transformed x line
-  float2* spec;          // [4][n2][n1][pitch] modes 0 .. n0/2 of the four fields
+  float2* spec;          // [4][n2][n1][pitch] modes 0 .. n0/2 of the four fields; then the tables
   int pitch;
   int xskew;             // shared-memory skew of the x lines per first-pass block
   int zsh, zen;          // shared-memory swap of the z lines
@@ -36,7 +36,6 @@ struct SpecArgs {
 
 struct Spectral {
   SpecArgs a;
-  void* tables;
   size_t smem_x, smem_y, smem_z;
   int threads_x, threads_y, threads_z;
 };
