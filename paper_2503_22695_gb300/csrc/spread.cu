@@ -298,8 +298,13 @@ __global__ void __launch_bounds__(kPT) k_spread_push(SpreadArgs<Real> A) {
 // ---------------------------------------------------------------------------
 constexpr float kMagic = 12582912.0f;             // M = 1.5 * 2^23
 constexpr float kMagicZ = 12582912.0f * 2049.0f;  // M (1 + 2^11), exact in float
-constexpr int kFxThreads = 256;
-constexpr int kFxWarps = kFxThreads / 32;
+// Threads of an accumulation CTA.  Plans whose items are all full: 256, three
+// CTAs per SM, which leave registers to the other branch's small kernels (the
+// 256^3 forward 373 us; 387 with 512).  Plans cut into smaller items, which do
+// not fill the SMs: 512, two CTAs per SM, half the points per warp (a warp's
+// step from point to point takes about 430 cycles whatever else runs: 128^3
+// shell 31 -> 24 us, tetrahedra at 104^3 41 -> 32).
+constexpr int kFxLarge = 256, kFxSmall = 512;
 constexpr int kFxGroup = 16;  // points a warp stages at a time: 2 lanes per point
 // Lane mapping: a warp takes one point at a time; lane (dz, dy, xh) adds the
 // faces xh and xh + 2 of stencil row (dz, dy), one instruction per face,
@@ -460,8 +465,10 @@ __device__ __forceinline__ long long fx_align(long long v, int sh) {
   return sh >= 0 ? (long long)((unsigned long long)v << sh) : (v >> min(-sh, 63));
 }
 
-template <bool kPacked>
-__global__ void __launch_bounds__(kFxThreads) k_spread_push_fx(SpreadArgs<float> A) {
+template <bool kPacked, int kFxThreads>
+__global__ void __launch_bounds__(kFxThreads, 1024 / kFxThreads)  // 64 registers
+    k_spread_push_fx(SpreadArgs<float> A) {
+  constexpr int kFxWarps = kFxThreads / 32;
   chain_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float4* groups = reinterpret_cast<float4*>(smem_raw);
@@ -790,14 +797,23 @@ size_t push_smem() {
   return sizeof(Staged<Real>) * kBatch + sizeof(Real) * kCopies * kAcc + sizeof(RawItem<Real>);
 }
 
-constexpr size_t kFxSmem =
-    sizeof(float4) * kFxWarps * kFxGroup * kFxRec + sizeof(unsigned) * 2 * kFxWords;
+constexpr size_t fx_smem(int threads) {
+  return sizeof(float4) * (threads / 32) * kFxGroup * kFxRec + sizeof(unsigned) * 2 * kFxWords;
+}
 
 template <bool kPacked>
 void launch_push(ib_plan* p, const SpreadArgs<float>& A, cudaStream_t s) {
   p->prof_calls[IB_STAGE_SPREAD_PUSH] += 1;
   const int ev = prof_begin(p, IB_STAGE_SPREAD_PUSH, s);
-  chain_launch(k_spread_push_fx<kPacked>, std::min(p->push_ctas, p->push_per_sm * p->sm_count), kFxThreads, kFxSmem, s, A);
+  // the tuning's cap counts CTAs of 256 threads
+  const int cap = p->push_per_sm * p->sm_count;
+  if (p->item < kChunk)
+    chain_launch(k_spread_push_fx<kPacked, kFxSmall>,
+                 std::min(p->push_ctas, (cap * kFxLarge + kFxSmall - 1) / kFxSmall), kFxSmall,
+                 fx_smem(kFxSmall), s, A);
+  else
+    chain_launch(k_spread_push_fx<kPacked, kFxLarge>, std::min(p->push_ctas, cap), kFxLarge,
+                 fx_smem(kFxLarge), s, A);
   prof_end(p, ev, s);
 }
 
@@ -867,19 +883,23 @@ ib_status prepare_t(ib_plan* p) {
   if (sizeof(Real) == 4) {
     // both variants (one structure, packed): the grid takes the smaller
     // occupancy of the two
-    int per_sm_packed = 0;
-    e = cudaFuncSetAttribute(k_spread_push_fx<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kFxSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_spread_push_fx<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)kFxSmem);
-    if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spread_push_fx<false>,
-                                                        kFxThreads, kFxSmem);
-    if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_packed, k_spread_push_fx<true>,
-                                                        kFxThreads, kFxSmem);
-    per_sm = std::min(per_sm, per_sm_packed);
+    auto prepare = [&](auto one, auto packed, int threads) {
+      const int smem = (int)fx_smem(threads);
+      int a = 0, b = 0;
+      cudaError_t r =
+          cudaFuncSetAttribute(one, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      if (r == cudaSuccess)
+        r = cudaFuncSetAttribute(packed, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+      if (r == cudaSuccess) r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, one, threads, smem);
+      if (r == cudaSuccess)
+        r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, packed, threads, smem);
+      per_sm = std::min(a, b);
+      return r;
+    };
+    e = p->item < kChunk ? prepare(k_spread_push_fx<false, kFxSmall>,
+                                   k_spread_push_fx<true, kFxSmall>, kFxSmall)
+                         : prepare(k_spread_push_fx<false, kFxLarge>,
+                                   k_spread_push_fx<true, kFxLarge>, kFxLarge);
   } else {
     const int smem = (int)push_smem<Real>();
     e = cudaFuncSetAttribute(k_spread_push<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
