@@ -60,6 +60,7 @@ __global__ void __launch_bounds__(256) k_elem_project(const Real* __restrict__ v
   for (int q = 0; q < EL::Q; ++q) wq[q] = w ? __ldg(w + (int64_t)q * E + e) : Real(1);
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
+    if (gridDim.y > 1 && c != (int)blockIdx.y) continue;  // components on their own CTAs
     Real v[EL::Q];
 #pragma unroll
     for (int q = 0; q < EL::Q; ++q) v[q] = __ldg(vals + c * Q + (int64_t)q * E + e) * wq[q];
@@ -171,11 +172,14 @@ template <typename Real>
 ib_status gather_t(ib_plan* p, const void* elem, const void* scale, const void* add, void* out,
                    int nc, cudaStream_t s, double mul = 1.0) {
   if (p->N == 0) return IB_OK;
-  const int blocks = (p->N + 255) / 256;
+  // small meshes: CTAs of 64 nodes, over more SMs
+  const int t = p->N < 256 * p->sm_count ? 64 : 256, blocks = (p->N + t - 1) / t;
   if (nc == 3)
-    chain_launch(k_node_gather<Real, 3>, blocks, 256, 0, s, p->inc_off, p->inc_idx, (const Real*)elem, (const Real*)scale, (const Real*)add, p->N, p->E, (Real*)out, (Real)mul);
+    chain_launch(k_node_gather<Real, 3>, blocks, t, 0, s, p->inc_off, p->inc_idx, (const Real*)elem,
+                 (const Real*)scale, (const Real*)add, p->N, p->E, (Real*)out, (Real)mul);
   else
-    chain_launch(k_node_gather<Real, 1>, blocks, 256, 0, s, p->inc_off, p->inc_idx, (const Real*)elem, (const Real*)scale, (const Real*)add, p->N, p->E, (Real*)out, (Real)mul);
+    chain_launch(k_node_gather<Real, 1>, blocks, t, 0, s, p->inc_off, p->inc_idx, (const Real*)elem,
+                 (const Real*)scale, (const Real*)add, p->N, p->E, (Real*)out, (Real)mul);
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 
@@ -183,13 +187,18 @@ template <typename Real>
 ib_status project_t(ib_plan* p, const void* vals, const void* w, void* out, int nc,
                     cudaStream_t s) {
   if (p->E == 0) return IB_OK;
-  const int blocks = (p->E + 255) / 256;
+  // small meshes: CTAs of 64 elements and one component
+  const bool small = p->E < 256 * p->sm_count;
+  const int t = small ? 64 : 256;
+  const dim3 blocks((p->E + t - 1) / t, small ? nc : 1);
   with_elem(p->elem, [&](auto el) {
     constexpr int kE = decltype(el)::value;
     if (nc == 3)
-      chain_launch(k_elem_project<Real, 3, kE>, blocks, 256, 0, s, (const Real*)vals, (const Real*)w, p->E, (Real*)out);
+      chain_launch(k_elem_project<Real, 3, kE>, blocks, t, 0, s, (const Real*)vals, (const Real*)w,
+                   p->E, (Real*)out);
     else
-      chain_launch(k_elem_project<Real, 1, kE>, blocks, 256, 0, s, (const Real*)vals, (const Real*)w, p->E, (Real*)out);
+      chain_launch(k_elem_project<Real, 1, kE>, blocks, t, 0, s, (const Real*)vals, (const Real*)w,
+                   p->E, (Real*)out);
   });
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
@@ -218,7 +227,8 @@ ib_status static_t(ib_plan* p, cudaStream_t s) {
         k_mass_corner_d<Real, kE><<<(p->E + 255) / 256, 256, 0, s>>>((const Real*)p->wj0, p->E,
                                                                      ed);
       });
-    chain_launch(k_node_gather<double, 1>, (p->N + 255) / 256, 256, 0, s, p->inc_off, p->inc_idx, ed, nullptr, nullptr, p->N, p->E, md, 1.0);
+    chain_launch(k_node_gather<double, 1>, (p->N + 255) / 256, 256, 0, s, p->inc_off, p->inc_idx,
+                 ed, nullptr, nullptr, p->N, p->E, md, 1.0);
     if (sizeof(Real) == 4)
       k_mass_round<<<(p->N + 255) / 256, 256, 0, s>>>(md, (float*)p->mass, (float*)p->inv_mass,
                                                       p->N);
@@ -255,9 +265,11 @@ ib_status launch_node_copy(ib_plan* p, const void* src, void* out, const void* a
   if (n == 0) return IB_OK;
   const unsigned blocks = (unsigned)((n + 255) / 256);
   if (p->precision == IB_FP64)
-    chain_launch(k_node_copy<double>, blocks, 256, 0, s, (const double*)src, (const double*)add, n, (double*)out);
+    chain_launch(k_node_copy<double>, blocks, 256, 0, s, (const double*)src, (const double*)add, n,
+                 (double*)out);
   else
-    chain_launch(k_node_copy<float>, blocks, 256, 0, s, (const float*)src, (const float*)add, n, (float*)out);
+    chain_launch(k_node_copy<float>, blocks, 256, 0, s, (const float*)src, (const float*)add, n,
+                 (float*)out);
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 

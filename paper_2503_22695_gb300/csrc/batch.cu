@@ -166,10 +166,12 @@ ib_status run_forward(ib_batch* b, cudaStream_t s) {
   const ib_pos x = packed_pos(b);
   MatTable none;
   std::memset(&none, 0, sizeof(none));
-  chain_launch(k_nodes<kPackPos>, node_grid(b), 256, 0, s, b->segs, b->N, b->cell, b->off, nullptr, nullptr);
+  chain_launch(k_nodes<kPackPos>, node_grid(b), 256, 0, s, b->segs, b->N, b->cell, b->off, nullptr,
+               nullptr);
   ib_status st = forward_body(b->P, none, &x, b->inst[0].u, b->G, b->inst[0].f, b->U, s, &b->pc);
   if (st == IB_OK)
-    chain_launch(k_nodes<kUnpackFwd>, node_grid(b), 256, 0, s, b->segs, b->N, nullptr, b->G, b->U, nullptr);
+    chain_launch(k_nodes<kUnpackFwd>, node_grid(b), 256, 0, s, b->segs, b->N, nullptr, b->G, b->U,
+                 nullptr);
   return st == IB_OK && ok(cudaGetLastError()) ? IB_OK : (st == IB_OK ? IB_ERR_CUDA : st);
 }
 
@@ -177,8 +179,10 @@ ib_status run_adjoint(ib_batch* b, cudaStream_t s) {
   const ib_pos x = packed_pos(b);
   MatTable none;
   std::memset(&none, 0, sizeof(none));
-  chain_launch(k_nodes<kPackPos>, node_grid(b), 256, 0, s, b->segs, b->N, b->cell, b->off, nullptr, nullptr);
-  chain_launch(k_nodes<kPackAdj>, node_grid(b), 256, 0, s, b->segs, b->N, nullptr, b->Gin, b->gU, b->any_gG ? b->gG : nullptr);
+  chain_launch(k_nodes<kPackPos>, node_grid(b), 256, 0, s, b->segs, b->N, b->cell, b->off, nullptr,
+               nullptr);
+  chain_launch(k_nodes<kPackAdj>, node_grid(b), 256, 0, s, b->segs, b->N, nullptr, b->Gin, b->gU,
+               b->any_gG ? b->gG : nullptr);
   // the instances' own fields come from the call tables; the pointers passed
   // here only mark which adjoint terms are wanted
   const ib_instance& i0 = b->inst[0];
@@ -187,7 +191,8 @@ ib_status run_adjoint(ib_batch* b, cudaStream_t s) {
                                /*params=*/true, nullptr, s, &b->pc);
   if (st == IB_OK) {
     chain_launch(k_gparams, b->n, 128, 0, s, b->P->ered, b->gp_rows, b->gparams);
-    chain_launch(k_nodes<kUnpackAdj>, node_grid(b), 256, 0, s, b->segs, b->N, nullptr, b->gx, nullptr, nullptr);
+    chain_launch(k_nodes<kUnpackAdj>, node_grid(b), 256, 0, s, b->segs, b->N, nullptr, b->gx,
+                 nullptr, nullptr);
   }
   return st == IB_OK && ok(cudaGetLastError()) ? IB_OK : (st == IB_OK ? IB_ERR_CUDA : st);
 }

@@ -579,7 +579,15 @@ ib_status forward_body(ib_plan* p, const MatTable& mt, const ib_pos* x, const vo
   if (!ok(cudaEventRecord(p->ev_ffork, s)) || !ok(cudaStreamWaitEvent(b, p->ev_ffork, 0)) ||
       (m != s && !ok(cudaStreamWaitEvent(m, p->ev_ffork, 0))))
     return IB_ERR_CUDA;
-  ib_status st = do_points_sorted(p, x, nullptr, b);
+  // Issued force first, then the side branch, whose interpolation is best over
+  // when the accumulation, which fills the SMs, starts (issued after it: 73 ->
+  // 77 us at 128^3), then the rest of the critical one.
+  ib_status st;
+  {
+    Stage sc(p, IB_STAGE_FORCE, m, 1);
+    st = launch_fe_force(p, mt, pos_a(p, x), x->off, p->elem_scratch, false, m);
+  }
+  if (st == IB_OK) st = do_points_sorted(p, x, nullptr, b);
   if (st == IB_OK && !ok(cudaEventRecord(p->ev_fsorted, b))) st = IB_ERR_CUDA;
   // the far-tile zeros of f (HBM writes) on the side branch, beside the
   // force kernel and ahead of the interpolation
@@ -589,21 +597,20 @@ ib_status forward_body(ib_plan* p, const MatTable& mt, const ib_pos* x, const vo
   }
   if (st == IB_OK && U) st = do_interp_tail(p, u, U, b, p->elem_scratch2, pc);
   if (st == IB_OK && !ok(cudaEventRecord(p->ev_fjoin, b))) st = IB_ERR_CUDA;
-  if (st == IB_OK) {
-    Stage sc(p, IB_STAGE_FORCE, m, 1);
-    st = launch_fe_force(p, mt, pos_a(p, x), x->off, p->elem_scratch, false, m);
-  }
   if (st == IB_OK) st = do_gather(p, p->elem_scratch, nullptr, G, m);
   if (st == IB_OK) st = launch_penalty(p, x, G, false, m);
   if (st == IB_OK) {
-    // the carried values before the binning is waited for, then their binned
+    // The carried values before the binning is waited for, then their binned
     // copy: the values overlap the binning's end (computing them at the binned
-    // positions in one pass after the wait, as the backward does, measured
-    // 0.404 -> 0.418 ms here)
-    Stage sc(p, IB_STAGE_POINTS, m, 2);
-    st = launch_point_values(p, G, m);
+    // positions in one pass after the wait measured 0.404 -> 0.418 ms at
+    // 256^3, 67 -> 71 us for the tetrahedra at 104^3).  The nodal rule's values
+    // are the nodal ones: binned directly.
+    const bool one = p->quad == IB_QUAD_NODAL;
+    Stage sc(p, IB_STAGE_POINTS, m, one ? binned_values_launches(p) : 2);
+    if (!one) st = launch_point_values(p, G, m);
     if (st == IB_OK && !ok(cudaStreamWaitEvent(m, p->ev_fsorted, 0))) st = IB_ERR_CUDA;
-    if (st == IB_OK) st = launch_permute_values(p, m, true);
+    if (st == IB_OK)
+      st = one ? launch_binned_values(p, G, m, true) : launch_permute_values(p, m, true);
   }
   if (st == IB_OK)
     st = do_spread(p, 1.0 / (p->grid.h * p->grid.h * p->grid.h), f, m, /*zero_fill=*/false,

@@ -230,9 +230,11 @@ ib_status launch_reduce_parts(ib_plan* p, int nvals, int n_mats, cudaStream_t s,
   const dim3 grid(nblk, n_mats);
   // FP32 partials are widened exactly: the sums are those of their doubles
   if (real_parts && p->precision != IB_FP64)
-    chain_launch(k_reduce<float>, grid, kRedThreads, 0, s, reinterpret_cast<const float*>(p->epart), p->mat_id, p->mat_range, p->E, nvals, p->rpart, p->red_count, out);
+    chain_launch(k_reduce<float>, grid, kRedThreads, 0, s, reinterpret_cast<const float*>(p->epart),
+                 p->mat_id, p->mat_range, p->E, nvals, p->rpart, p->red_count, out);
   else
-    chain_launch(k_reduce<double>, grid, kRedThreads, 0, s, p->epart, p->mat_id, p->mat_range, p->E, nvals, p->rpart, p->red_count, out);
+    chain_launch(k_reduce<double>, grid, kRedThreads, 0, s, p->epart, p->mat_id, p->mat_range, p->E,
+                 nvals, p->rpart, p->red_count, out);
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 

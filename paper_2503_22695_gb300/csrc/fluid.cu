@@ -526,7 +526,8 @@ ib_status launch_advance_positions(ib_plan* p, const ib_pos* x, const void* U, d
   if (p->precision == IB_FP64)
     chain_launch(k_advance_x64, g, 256, 0, s, const_cast<double*>(x->x64), (const double*)U, n, dt);
   else
-    chain_launch(k_advance_split, g, 256, 0, s, const_cast<int32_t*>(x->cell), const_cast<float*>(x->off), (const float*)U, n, (float)(dt / p->grid.h));
+    chain_launch(k_advance_split, g, 256, 0, s, const_cast<int32_t*>(x->cell),
+                 const_cast<float*>(x->off), (const float*)U, n, (float)(dt / p->grid.h));
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 

@@ -467,7 +467,7 @@ int classify_blocks(int ntiles);
 int item_size(int precision, int64_t Q, int sms);
 int64_t max_work_items(int ntiles, int64_t Q, int item);
 inline ItemRule item_rule(const ib_plan* p) {
-  const int gran = p->precision == IB_FP64 ? 32 : 128;
+  const int gran = p->precision == IB_FP64 ? 64 : 128;
   return ItemRule{p->chunk, p->item < p->chunk ? p->item : p->chunk, gran};
 }
 int sort_key_bits(int ntiles);

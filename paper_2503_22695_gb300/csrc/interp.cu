@@ -87,6 +87,10 @@ __device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
   const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(smem));
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
+__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
+  const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(smem));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait_group() {
@@ -114,11 +118,10 @@ __device__ __forceinline__ void stage_block(const InterpArgs<Real>& A, const Til
     gz += gz < 0 ? n2 : (gz >= n2 ? -n2 : 0);
     Real* dst = ub + c * kComp + bz * kSZ + by * kSY + bx;
     const Real* src = u + c * cells + ((int64_t)gz * n1 + gy) * n0 + gx;
-    if (sizeof(Real) == 4) {
+    if (sizeof(Real) == 4)
       cp_async4(dst, src);
-    } else {
-      *dst = *src;
-    }
+    else
+      cp_async8(dst, src);
   }
 }
 
@@ -408,6 +411,36 @@ __global__ void __launch_bounds__(kThreads, MODE == 0 ? 3 : 2)
   }
 }
 
+// Component c alone (values only), from its own block ub.
+template <typename Real>
+__device__ __forceinline__ Real interp_comp(const Real* ub, const int lc[3], const Real off[3],
+                                            int c) {
+  Real w[3][4];
+  int b[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    Real th;
+    b[d] = lc[d] + stencil_axis(off[d], d != c, th) + 2;
+    delta_weights(th, w[d]);
+  }
+  const Real* uc = ub + b[2] * kSZ + b[1] * kSY + b[0];
+  Real tot = Real(0);
+#pragma unroll
+  for (int kz = 0; kz < 4; ++kz) {
+    Real py = Real(0);
+#pragma unroll
+    for (int ky = 0; ky < 4; ++ky) {
+      const Real* row = uc + kz * kSZ + ky * kSY;
+      Real rx = Real(0);
+#pragma unroll
+      for (int kx = 0; kx < 4; ++kx) rx += w[0][kx] * row[kx];
+      py += w[1][ky] * rx;
+    }
+    tot += w[2][kz] * py;
+  }
+  return tot;
+}
+
 // One point: the three stencil sums at local cell lc with offsets off, and
 // (MODE != 0) their position derivatives weighted by val; results written at
 // the point's original index gq.
@@ -503,6 +536,53 @@ __device__ __forceinline__ void interp_points(const InterpArgs<Real>& A, int slo
       for (int c = 0; c < 3; ++c) val[c] = __ldg(A.p_val + c * A.Q + i);
     }
     interp_one<Real, MODE>(A, ub, lc, off, __ldg(A.p_idx + i), val, vs, gs);
+  }
+}
+
+// FP64 plans with few points, values only: one unit per item and component,
+// staging that component's block alone.  An SM's FP64 pipe takes 16 cycles per
+// warp instruction and a point's three sums some 500 of them, so the work is
+// spread over as many SMs as it has units (128 hexahedra: 24 us with whole
+// items, 10 with components).  Larger plans fill the SMs with whole items,
+// which form each axis's weights once per staggering instead of per component.
+__global__ void __launch_bounds__(kThreads) k_interp_comp(InterpArgs<double> A) {
+  chain_wait();
+  __shared__ __align__(16) double ub[kComp];
+  __shared__ int next;
+  const int tid = threadIdx.x;
+  const int count = 3 * A.counters[0];
+  for (int k = blockIdx.x; k < count;) {
+    const int c = k % 3;
+    const Item item = load_item(A.items, k / 3);
+    const TileGeo geo = tile_geo<false>(A.g, nullptr, nullptr, item.tile);
+    int tx, ty, tz;
+    tile_coords(geo, item.tile, tx, ty, tz);
+    const int x0 = tx * kTile, y0 = ty * kTile, z0 = tz * kTile;
+    const int n0 = geo.n[0], n1 = geo.n[1], n2 = geo.n[2];
+    const double* const u = A.u + (int64_t)c * n0 * n1 * n2;
+    for (int t = tid; t < kB * kB * kB; t += kThreads) {
+      const int bz = t / (kB * kB), by = (t / kB) % kB, bx = t % kB;
+      int gx = x0 - 2 + bx, gy = y0 - 2 + by, gz = z0 - 2 + bz;  // within one period
+      gx += gx < 0 ? n0 : (gx >= n0 ? -n0 : 0);
+      gy += gy < 0 ? n1 : (gy >= n1 ? -n1 : 0);
+      gz += gz < 0 ? n2 : (gz >= n2 ? -n2 : 0);
+      cp_async8(ub + bz * kSZ + by * kSY + bx, u + ((int64_t)gz * n1 + gy) * n0 + gx);
+    }
+    cp_async_commit();
+    cp_async_wait_group<0>();
+    __syncthreads();
+    for (int i = item.begin + tid; i < item.begin + item.n; i += kThreads) {
+      int cx, cy, cz;
+      unpack_cell(__ldg(A.p_cell + i), cx, cy, cz);
+      const int lc[3] = {cx - x0, cy - y0, cz - z0};
+      const double off[3] = {__ldg(A.p_off + i), __ldg(A.p_off + A.Q + i),
+                             __ldg(A.p_off + 2 * A.Q + i)};
+      A.out_a[c * A.Q + __ldg(A.p_idx + i)] = A.vscale * interp_comp<double>(ub, lc, off, c);
+    }
+    if (tid == 0) next = (int)gridDim.x + atomicAdd(work_counter<0>(A), 1);
+    __syncthreads();  // block read; next unit known
+    k = next;
+    __syncthreads();
   }
 }
 
@@ -605,6 +685,12 @@ ib_status interp_t(ib_plan* p, const void* u, int mode, double vscale, double gs
       else
         run(packed ? k_interp_tma<2, true> : k_interp_tma<2, false>, p->interp_ctas_tma[2],
             tma_smem<2>());
+      return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
+    }
+  }
+  if constexpr (sizeof(Real) == 8) {
+    if (mode == 0 && p->item < kChunk) {
+      chain_launch(k_interp_comp, 4 * p->sm_count, kThreads, 0, s, A);
       return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
     }
   }

@@ -155,9 +155,11 @@ ib_status launch_penalty_adj(ib_plan* p, const void* v, void* Hv, cudaStream_t s
   const int g = (p->pen_n + 255) / 256;
   ib_pos none{nullptr, nullptr, nullptr, 0.0};
   if (p->precision == IB_FP64)
-    chain_launch(k_penalty_adj<double>, g, 256, 0, s, pen_args<double>(p, &none), (const double*)v, (double*)Hv, mul);
+    chain_launch(k_penalty_adj<double>, g, 256, 0, s, pen_args<double>(p, &none), (const double*)v,
+                 (double*)Hv, mul);
   else
-    chain_launch(k_penalty_adj<float>, g, 256, 0, s, pen_args<float>(p, &none), (const float*)v, (float*)Hv, (float)mul);
+    chain_launch(k_penalty_adj<float>, g, 256, 0, s, pen_args<float>(p, &none), (const float*)v,
+                 (float*)Hv, (float)mul);
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 

@@ -75,6 +75,10 @@ __device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
   const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
 }
+__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
+  const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
+}
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_all;\n" ::: "memory");
 }
@@ -123,19 +127,19 @@ __device__ __forceinline__ void zero_shared(Real* p, int n, int tid, int nthread
   for (int i = tid; i < n4; i += nthreads) v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// Work item `slot` of the list.
 // Raw point data of one work item, copied to shared memory once.
 template <typename Real>
 struct RawItem {
   int32_t cell[kChunk];
   Real off[3][kChunk];
-  Real val[3][kChunk];
+  Real val[kChunk];  // the component's
 };
 
 template <typename Real>
-__device__ __forceinline__ void push_item(const SpreadArgs<Real>& A, int slot, Staged<Real>* stage,
-                                          Real* acc, RawItem<Real>* raw, int tid) {
-  const Item item = load_item(A.items, slot);
+__device__ __forceinline__ void push_item(const SpreadArgs<Real>& A, int k, int c,
+                                          Staged<Real>* stage, Real* acc, RawItem<Real>* raw,
+                                          int tid) {
+  const Item item = load_item(A.items, k);
   const int tile = item.tile;
   const TileGeo geo = tile_geo<false>(A.g, nullptr, nullptr, tile);  // FP64: one structure
   int tx, ty, tz;
@@ -152,88 +156,80 @@ __device__ __forceinline__ void push_item(const SpreadArgs<Real>& A, int slot, S
   for (int i = tid; i < n; i += kPT) {
     cp_async4(&raw->cell[i], A.p_cell + s + i);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      if (sizeof(Real) == 4) {
-        cp_async4(&raw->off[d][i], A.p_off + d * A.Q + s + i);
-        cp_async4(&raw->val[d][i], A.p_val + d * A.Q + s + i);
-      } else {
-        raw->off[d][i] = A.p_off[d * A.Q + s + i];
-        raw->val[d][i] = A.p_val[d * A.Q + s + i];
+    for (int d = 0; d < 3; ++d) cp_async8(&raw->off[d][i], A.p_off + d * A.Q + s + i);
+    cp_async8(&raw->val[i], A.p_val + c * A.Q + s + i);
+  }
+  // Private copies in use: summing them takes one FP64 add per face and copy,
+  // more than the points of a small item (eight copies: 7000 cycles).
+  const int copies = n <= 64 ? 2 : (n <= 256 ? 4 : kCopies);
+  zero_shared(acc, copies * kAcc, tid, kPT);
+  cp_async_wait();
+  for (int b0 = s; b0 < e; b0 += kBatch) {
+    const int nb = min(kBatch, e - b0);
+    __syncthreads();  // previous batch consumed, accumulators zeroed
+    if (tid < nb) {
+      const int i = b0 - s + tid;
+      int cx, cy, cz;
+      unpack_cell(raw->cell[i], cx, cy, cz);
+      Staged<Real> st;
+      Real th;
+      const int bx = cx - x0 + stencil_axis(raw->off[0][i], c != 0, th) + 2;
+      delta_weights(th, st.wx);
+      const int by = cy - y0 + stencil_axis(raw->off[1][i], c != 1, th) + 2;
+      delta_weights(th, st.wy);
+      const int bz = cz - z0 + stencil_axis(raw->off[2][i], c != 2, th) + 2;
+      delta_weights(th, st.wz);
+      st.val = raw->val[i] * scale;
+      st.org = bz * kSZ + by * kSY + bx;
+      stage[tid] = st;
+    }
+    __syncthreads();
+    // The warp's two half-warps take points hw + copies k (those of warps
+    // without a copy none); the loop runs the even half's trip count (never
+    // smaller) so __syncwarp sees the full warp.  The next point's staged
+    // values are read before the current point's read-modify-writes.
+    const int steps =
+        nb > 2 * warp && 2 * warp < copies ? (nb - 2 * warp + copies - 1) / copies : 0;
+    int p = hw < copies ? hw : nb;
+    Real w = Real(0), wx[4] = {Real(0), Real(0), Real(0), Real(0)};
+    int o = 0;
+    if (p < nb) {
+      const Staged<Real>& st = stage[p];
+      w = st.val * st.wz[dz] * st.wy[dy];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) wx[k] = st.wx[k];
+      o = st.org + lane_off;
+    }
+    for (int t = 0; t < steps; ++t, p += copies) {
+      Real wn = Real(0), wxn[4] = {Real(0), Real(0), Real(0), Real(0)};
+      int on = 0;
+      if (p + copies < nb) {
+        const Staged<Real>& st = stage[p + copies];
+        wn = st.val * st.wz[dz] * st.wy[dy];
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) wxn[kk] = st.wx[kk];
+        on = st.org + lane_off;
       }
+      if (p < nb) {
+        Real* q = my + o;
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) add_shared(q + kk, w * wx[kk]);
+      }
+      __syncwarp();
+      w = wn;
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) wx[kk] = wxn[kk];
+      o = on;
     }
   }
-  cp_async_wait();
-
-  for (int c = 0; c < 3; ++c) {
-    zero_shared(acc, kCopies * kAcc, tid, kPT);
-    for (int b0 = s; b0 < e; b0 += kBatch) {
-      const int nb = min(kBatch, e - b0);
-      __syncthreads();  // previous batch consumed, accumulators zeroed
-      if (tid < nb) {
-        const int i = b0 - s + tid;
-        int cx, cy, cz;
-        unpack_cell(raw->cell[i], cx, cy, cz);
-        Staged<Real> st;
-        Real th;
-        const int bx = cx - x0 + stencil_axis(raw->off[0][i], c != 0, th) + 2;
-        delta_weights(th, st.wx);
-        const int by = cy - y0 + stencil_axis(raw->off[1][i], c != 1, th) + 2;
-        delta_weights(th, st.wy);
-        const int bz = cz - z0 + stencil_axis(raw->off[2][i], c != 2, th) + 2;
-        delta_weights(th, st.wz);
-        st.val = raw->val[c][i] * scale;
-        st.org = bz * kSZ + by * kSY + bx;
-        stage[tid] = st;
-      }
-      __syncthreads();
-      // The warp's two half-warps take points hw + 8k; the loop runs the
-      // even half's trip count (never smaller) so __syncwarp sees the full
-      // warp.  The next point's staged values are read before the current
-      // point's read-modify-writes.
-      const int steps = nb > 2 * warp ? (nb - 2 * warp + kCopies - 1) / kCopies : 0;
-      int p = hw;
-      Real w = Real(0), wx[4] = {Real(0), Real(0), Real(0), Real(0)};
-      int o = 0;
-      if (p < nb) {
-        const Staged<Real>& st = stage[p];
-        w = st.val * st.wz[dz] * st.wy[dy];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) wx[k] = st.wx[k];
-        o = st.org + lane_off;
-      }
-      for (int k = 0; k < steps; ++k, p += kCopies) {
-        Real wn = Real(0), wxn[4] = {Real(0), Real(0), Real(0), Real(0)};
-        int on = 0;
-        if (p + kCopies < nb) {
-          const Staged<Real>& st = stage[p + kCopies];
-          wn = st.val * st.wz[dz] * st.wy[dy];
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk) wxn[kk] = st.wx[kk];
-          on = st.org + lane_off;
-        }
-        if (p < nb) {
-          Real* q = my + o;
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk) add_shared(q + kk, w * wx[kk]);
-        }
-        __syncwarp();
-        w = wn;
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) wx[kk] = wxn[kk];
-        o = on;
-      }
-    }
-    __syncthreads();
-    Real* out = A.scratch + ((int64_t)item.slot * 3 + c) * kBlk;
-    for (int idx = tid; idx < kBlk; idx += kPT) {
-      const int z = idx / (kB * kB), y = (idx / kB) % kB, x = idx % kB;
-      const int o = z * kSZ + y * kSY + x;
-      Real sum = Real(0);
-#pragma unroll
-      for (int w = 0; w < kCopies; ++w) sum += acc[w * kAcc + o];
-      out[idx] = sum;
-    }
-    __syncthreads();
+  __syncthreads();
+  Real* out = A.scratch + ((int64_t)item.slot * 3 + c) * kBlk;
+  for (int idx = tid; idx < kBlk; idx += kPT) {
+    const int z = idx / (kB * kB), y = (idx / kB) % kB, x = idx % kB;
+    const int o = z * kSZ + y * kSY + x;
+    Real sum = Real(0);
+    for (int w = 0; w < copies; ++w) sum += acc[w * kAcc + o];
+    out[idx] = sum;
   }
 }
 
@@ -247,14 +243,14 @@ __global__ void __launch_bounds__(kPT) k_spread_push(SpreadArgs<Real> A) {
       smem_raw + sizeof(Staged<Real>) * kBatch + sizeof(Real) * kCopies * kAcc);
   __shared__ int next;
   const int tid = threadIdx.x;
-  const int count = A.counters[0];
-  for (;;) {
+  // each component of an item is a unit of its own
+  const int count = 3 * A.counters[0];
+  for (int k = blockIdx.x; k < count;) {
+    push_item(A, k / 3, k % 3, stage, acc, raw, tid);
+    if (tid == 0) next = (int)gridDim.x + atomicAdd(A.counters + 1, 1);
+    __syncthreads();  // accumulators read out; next unit known
+    k = next;
     __syncthreads();
-    if (tid == 0) next = atomicAdd(A.counters + 1, 1);
-    __syncthreads();
-    const int k = next;
-    if (k >= count) break;
-    push_item(A, k, stage, acc, raw, tid);
   }
 }
 
@@ -724,70 +720,83 @@ __global__ void __launch_bounds__(kMT) k_spread_zero(SpreadArgs<Real> A) {
   }
 }
 
-// Near tiles: fixed-order sum of the halo'd blocks that cover each face.
-// Source (ox, oy, oz) covers local face (x, y, z) when each offset is 0, or
-// -1 with the coordinate <= 1, or +1 with it >= 6; the face is then at block
-// index (x - 8 ox + 2, y - 8 oy + 2, z - 8 oz + 2).  One thread per x-row of 8
-// faces (component, z, y): for each (oz, oy) source pair in order it reads
-// the row's own-tile part (block x 2..9) and, for faces 0,1 and 6,7, the
-// x-neighbours' halo pairs (block x 10,11 of ox = -1 and 0,1 of ox = +1),
-// and adds them face by face in the order (oz, oy, ox).
+// Near tiles (FP64 plans): fixed-order sum of the halo'd blocks that cover
+// each face, with k_spread_merge_fx's threads and sources (one thread per face
+// pair of each component; up to eight covering source tiles, two per axis).
+// The j-th blocks of all sources are loaded together, summed per source in
+// item order, the sources in ascending order (oz, oy, ox): a small structure's
+// merge is a chain of load latencies (one row of 8 faces per thread, source
+// after source: 14 us for 27 near tiles of 4 items).
 template <typename Real>
 __global__ void __launch_bounds__(kMT) k_spread_merge(SpreadArgs<Real> A) {
   chain_wait();
-  __shared__ int src_slot[27], src_n[27];
-  const int tid = threadIdx.x;
+  using Real2 = double2;
+  static_assert(sizeof(Real) == 8, "FP64 plans");
+  const unsigned full = 0xffffffffu;
+  const int tid = threadIdx.x, lane = tid & 31;
   const int count = A.counters[3];
+  const int z = tid >> 5, y = (tid >> 2) & 7, xq = tid & 3;
+  const int lz = z <= 1 ? -1 : 0, ly = y <= 1 ? -1 : 0, lx = xq == 0 ? -1 : 0;
+  const int nz = (z <= 1 || z >= 6) ? 2 : 1, ny = (y <= 1 || y >= 6) ? 2 : 1,
+            nx = (xq == 0 || xq == 3) ? 2 : 1;
   for (int k = blockIdx.x; k < count; k += gridDim.x) {
     const int tile = A.tile_list_near[k];
     const TileGeo geo = tile_geo<false>(A.g, nullptr, nullptr, tile);  // FP64: one structure
     int tx, ty, tz;
     tile_coords(geo, tile, tx, ty, tz);
+    int slot = 0, items = 0;
+    if (lane < 27) {
+      const int t = tile_of(tx + lane % 3 - 1, ty + (lane / 3) % 3 - 1, tz + lane / 9 - 1, geo);
+      slot = __ldg(A.tile_slot + t);
+      items = __ldg(A.tile_nitems + t);
+    }
+    const int most = __reduce_max_sync(full, items);
+    int sl[8], ns[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int iz = i >> 2, iy = (i >> 1) & 1, ix = i & 1;
+      const bool use = iz < nz && iy < ny && ix < nx;
+      const int src = (lz + iz + 1) * 9 + (ly + iy + 1) * 3 + lx + ix + 1;
+      sl[i] = __shfl_sync(full, slot, use ? src : 0);
+      ns[i] = __shfl_sync(full, items, use ? src : 0);
+      if (!use) ns[i] = 0;
+    }
     const int n0 = geo.n[0], n1 = geo.n[1];
     const int64_t cells = (int64_t)n0 * n1 * geo.n[2];
-    const int x0 = tx * kTile, y0 = ty * kTile, z0 = tz * kTile;
-    __syncthreads();
-    if (tid < 27) {
-      const int a = tid / 9 - 1, b = (tid / 3) % 3 - 1, c = tid % 3 - 1;
-      const int nb = tile_of(tx + c, ty + b, tz + a, geo);
-      src_slot[tid] = A.tile_slot[nb];
-      src_n[tid] = A.tile_nitems[nb];
-    }
-    __syncthreads();
-    if (tid < 3 * 64) {
-      const int c = tid >> 6, z = (tid >> 3) & 7, y = tid & 7;
-      const int ly = y <= 1 ? -1 : 0, lz = z <= 1 ? -1 : 0;
-      const int hy = y >= 6 ? 1 : 0, hz = z >= 6 ? 1 : 0;
-      Real sum[8];
+    Real* const row0 =
+        A.f + ((int64_t)(tz * kTile + z) * n1 + (ty * kTile + y)) * n0 + tx * kTile;
+#pragma unroll 1
+    for (int c = 0; c < 3; ++c) {
+      Real2 acc[8];
 #pragma unroll
-      for (int x = 0; x < 8; ++x) sum[x] = Real(0);
-      for (int oz = lz; oz <= hz; ++oz)
-        for (int oy = ly; oy <= hy; ++oy) {
-          const int rowoff = c * kBlk + ((z - oz * kTile + 2) * kB + (y - oy * kTile + 2)) * kB;
-          const int s0 = (oz + 1) * 9 + (oy + 1) * 3;
-          for (int ox = -1; ox <= 1; ++ox) {
-            const int sl = src_slot[s0 + ox + 1], ns = src_n[s0 + ox + 1];
-            for (int j = 0; j < ns; ++j) {
-              const Real* r = A.scratch + (int64_t)(sl + j) * kItemBlk + rowoff;
-              if (ox < 0) {          // faces 0,1 from the left neighbour's block x 10,11
-                sum[0] += r[10];
-                sum[1] += r[11];
-              } else if (ox > 0) {   // faces 6,7 from the right neighbour's block x 0,1
-                sum[6] += r[0];
-                sum[7] += r[1];
-              } else {
-                Real v[8];
+      for (int i = 0; i < 8; ++i) acc[i] = make_double2(0.0, 0.0);
+      for (int j = 0; j < most; ++j) {
+        Real2 v[8];
 #pragma unroll
-                for (int x = 0; x < 8; ++x) v[x] = r[2 + x];
-#pragma unroll
-                for (int x = 0; x < 8; ++x) sum[x] += v[x];
-              }
-            }
+        for (int i = 0; i < 8; ++i) {
+          v[i] = make_double2(0.0, 0.0);
+          if (j < ns[i]) {
+            // this face pair in the source tile's halo'd block
+            const int oz = lz + (i >> 2), oy = ly + ((i >> 1) & 1), ox = lx + (i & 1);
+            const int q = ((z - oz * kTile + 2) * kB + (y - oy * kTile + 2)) * (kB / 2) + xq + 1 -
+                          (kTile / 2) * ox;
+            v[i] = __ldcg(reinterpret_cast<const Real2*>(A.scratch) +
+                          ((int64_t)(sl[i] + j) * 3 + c) * (kBlk / 2) + q);
           }
         }
-      Real* out = A.f + c * cells + ((int64_t)(z0 + z) * n1 + (y0 + y)) * n0 + x0;
 #pragma unroll
-      for (int x = 0; x < 8; ++x) out[x] = sum[x];
+        for (int i = 0; i < 8; ++i) {
+          acc[i].x += v[i].x;
+          acc[i].y += v[i].y;
+        }
+      }
+      Real2 t = acc[0];
+#pragma unroll
+      for (int i = 1; i < 8; ++i) {
+        t.x += acc[i].x;
+        t.y += acc[i].y;
+      }
+      reinterpret_cast<Real2*>(row0 + c * cells)[xq] = t;
     }
   }
 }
@@ -820,7 +829,8 @@ void launch_push(ib_plan* p, const SpreadArgs<float>& A, cudaStream_t s) {
 template <bool kPacked>
 void launch_push(ib_plan* p, const SpreadArgs<double>& A, cudaStream_t s) {
   static_assert(!kPacked, "packed plans are FP32");
-  chain_launch(k_spread_push<double>, std::min(p->push_ctas, p->push_per_sm * p->sm_count), kPT, push_smem<double>(), s, A);
+  chain_launch(k_spread_push<double>, std::min(p->push_ctas, p->push_per_sm * p->sm_count), kPT,
+               push_smem<double>(), s, A);
 }
 
 template <typename Real>

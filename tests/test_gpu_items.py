@@ -68,3 +68,36 @@ def test_item_edges(N, tiles, fp64):
     tf, tU = (1e-12, 1e-12) if fp64 else (1e-5, 1e-6)
     assert rel_l2(np_(f).reshape(3, -1), fo) <= tf
     assert rel_l2(np_(U), Uo) <= tU
+
+
+@pytest.mark.parametrize("fp64", [False, True])
+def test_full_items(fp64):
+    """Enough points for full items on every SM: the kernels of large plans."""
+    import torch
+    from paper_2503_22695_gb300 import ibfe
+    n, h, N = 32, 1.0 / 32, 650_000
+    rng = np.random.default_rng(7)
+    dt = np.float64 if fp64 else np.float32
+    t = np.concatenate([I.HEX_CORNERS.T * 0.25 + 12.0,
+                        n * rng.uniform(0.001, 0.999, size=(3, N - 8))], axis=1)
+    g = I.Grid((n, n, n), h)
+    cell, off = I.to_split(t * h, g)
+    x = t * h if fp64 else I.from_split(cell, off, g)
+    conn = torch.arange(8, dtype=torch.int32, device="cuda").reshape(8, 1)
+    plan = ibfe.Plan(conn, torch.from_numpy((t * h).astype(dt)).cuda(), g.n, h,
+                     quad=ibfe.IB_QUAD_NODAL,
+                     precision=ibfe.IB_FP64 if fp64 else ibfe.IB_FP32_SPLIT)
+    pos = (ibfe.Pos(x64=torch.from_numpy(x).cuda()) if fp64 else
+           ibfe.Pos(cell=torch.from_numpy(cell).cuda(), off=torch.from_numpy(off).cuda()))
+    G = rng.normal(size=(3, N)).astype(dt)
+    u = rng.normal(size=(3, n, n, n)).astype(dt)
+    f = ibfe.ib_spread(plan, pos, torch.from_numpy(G).cuda())
+    U = ibfe.ib_interp(plan, pos, torch.from_numpy(u).cuda())
+    fo, Uo = np.zeros((3, n ** 3)), np.zeros((3, N))
+    for c in range(3):
+        flat, w = _stencil(x / h, c, n)
+        fo[c] = np.bincount(flat.ravel(), (w * G[c].astype(np.float64)).ravel(), n ** 3) / h ** 3
+        Uo[c] = (u[c].astype(np.float64).ravel()[flat] * w).sum(0)
+    tf, tU = (1e-12, 1e-12) if fp64 else (1e-5, 1e-6)
+    assert rel_l2(np_(f).reshape(3, -1), fo) <= tf
+    assert rel_l2(np_(U), Uo) <= tU
