@@ -77,6 +77,21 @@ def test_direct_solve_matches_oracle(n):
         assert torch.equal(b, un) and torch.equal(pb, p)
 
 
+@pytest.mark.parametrize("L", [32, 40, 48, 64, 80, 96, 128, 160, 192, 256, 320, 384, 512])
+def test_compile_time_lengths_match_oracle(L):
+    """Each length with transforms of its own, along each dimension."""
+    import torch
+    from paper_2503_22695_gb300 import ibfe
+    for n in ((L, 4, 6), (6, L, 4), (4, 6, L)):
+        g, u, f = _fields(n, sum(n))
+        fl = ibfe.Fluid(g.n, g.h, RHO, MU, DT)
+        un, p, _ = ibfe.ib_fluid_step(fl, torch.from_numpy(u).cuda(), torch.from_numpy(f).cuda())
+        us, po, uo = OF.fluid_step(u, f, RHO, MU, DT, g.h)
+        tu, tp = _bounds(u, us, uo, g.h)
+        assert _rms(np_(un) - uo) <= tu, n
+        assert _rms(np_(p) - po) <= tp, n
+
+
 @pytest.mark.parametrize("n", [(56, 8, 8), (8, 22, 8), (8, 8, 28), (4, 4, 1024)])
 def test_other_lattices_keep_the_cycles(n):
     import torch
