@@ -30,14 +30,23 @@
 // order the modes are stored in.  Each transform's first pass reads global
 // memory and its last pass writes it.
 //
+// Order of the planes: each kernel starts with what the one before it wrote
+// last, which L2 still holds (k_spec_y<0> and k_spec_out walk the planes
+// backwards): at 256^3 k_spec_out 157 -> 140 us.  Loads that would wait for
+// memory behind the transforms are asked for early: k_spec_out's velocity rows
+// at its start (177 -> 157 us), the y transforms' lines one wave of CTAs ahead
+// (106 -> 91 us).  The same for k_spec_rhs (171 -> 204), the solve (158 -> 168)
+// and k_spec_out's modes (140 -> 159) costs more than it hides.
+//
 // Measured on GB300 (us; V-cycles of fluid.cu before, this after): 32^3 step
-// 631 -> 46, 192^3 3425 -> 371, 256^3 6550 -> 770.  At 256^3 the five passes
-// take 198, 107, 175, 104 and 184 us for 0.57, 0.54, 0.54, 0.54 and 0.74 GB:
-// the y passes run at 5 TB/s, the others at 3 to 4 TB/s (instruction issue at
-// 50% beside the loads' latency).  x lines use radices up to 8 (48 registers,
-// 5 CTAs per SM: 184 against 250 us with radix 16 for k_spec_out); y lines up
-// to 16 (two passes at 256: 104 against 114..130 us); the z transform holds
-// four fields, 3 CTAs per SM (175 us; 2: 208, 4 with spills: 211).
+// 631 -> 46, 192^3 3417 -> 308, 256^3 6550 -> 656.  At 256^3 the five kernels
+// take 171, 91, 157, 99 and 139 us for 0.67, 0.54, 0.54, 0.54 and 0.74 GB:
+// 3.9, 5.9, 3.4, 5.4 and 5.3 TB/s; k_spec_rhs is bound by the L1 data pipe
+// (77% at 192^3), the solve by instruction issue (58%) beside its loads'
+// latency.  x lines use radices up to 8 (48 registers, 5 CTAs per SM: 184
+// against 250 us with radix 16 for k_spec_out); y lines up to 16 (two passes
+// at 256: 104 against 114..130 us); the z transform holds four fields, 3 CTAs
+// per SM (175 us; 2: 208, 4 with spills: 211).
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -440,6 +449,19 @@ __device__ __forceinline__ void ld_cells(float* v, const float* __restrict__ g) 
   }
 }
 
+// Requests to bring memory to L2: the 128-byte line at g; the 16-byte blocks
+// that lie within [g, g + bytes).
+__device__ __forceinline__ void prefetch_line(const void* g) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(g));
+}
+__device__ __forceinline__ void prefetch_rows(const void* g, int bytes) {
+  const uintptr_t a = (reinterpret_cast<uintptr_t>(g) + 15) & ~(uintptr_t)15;
+  const uintptr_t e = (reinterpret_cast<uintptr_t>(g) + bytes) & ~(uintptr_t)15;
+  if (e > a)
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((unsigned)(e - a))
+                 : "memory");
+}
+
 // Transforms the 16 lines held in shared memory.
 template <bool kInv, int N>
 __device__ __forceinline__ void line_passes(const SpecArgs& A, float2* z) {
@@ -568,11 +590,17 @@ __global__ void __launch_bounds__(256, has16(N, 1) ? 3 : 5) k_spec_y(SpecArgs A)
   chain_wait();
   chain_next();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int n1 = N > 0 ? N : A.y.n;
+  const int n1 = N > 0 ? N : A.y.n, n2 = A.z.n;
   const int col = threadIdx.x & (kTX - 1), j0 = threadIdx.x / kTX;
   const int kx = blockIdx.x * kTX + col;
-  const GlobalCol g{A.spec + (int64_t)(blockIdx.z * A.z.n + blockIdx.y) * n1 * A.pitch + kx,
-                    A.pitch, 0, kx <= A.x.n / 2};
+  const int k = kInv ? blockIdx.z : n2 - 1 - blockIdx.z;
+  const GlobalCol g{A.spec + (int64_t)(blockIdx.y * n2 + k) * n1 * A.pitch + kx, A.pitch, 0,
+                    kx <= A.x.n / 2};
+  // one wave of CTAs ahead, where the modes come from memory
+  if ((int)blockIdx.z + A.ahead < n2)
+    for (int r = threadIdx.x; r < n1; r += blockDim.x)
+      prefetch_line(A.spec + ((int64_t)(blockIdx.y * n2 + (kInv ? k + A.ahead : k - A.ahead)) * n1 +
+                              r) * A.pitch + blockIdx.x * kTX);
   const SharedCol<kTX> s{reinterpret_cast<float2*>(smem_raw) + col, 0, 0, 0};
   if constexpr (N > 0) {
     constexpr int np = Dim<N, 1>::P.np, step = col_threads(N, Dim<N, 1>::P.rad[0], kTX) / kTX;
@@ -698,8 +726,11 @@ __global__ void __launch_bounds__(256, 5) k_spec_out(SpecArgs A, const float* u,
   float2* z = reinterpret_cast<float2*>(smem_raw);
   const LineSmem<N> L(A, z);
   const int n0 = N > 0 ? N : A.x.n, n1 = A.y.n, n2 = A.z.n;
-  const int k = blockIdx.y, jp0 = blockIdx.x * 4, np = min(4, n1 / 2 - jp0);
+  const int k = n2 - 1 - blockIdx.y, jp0 = blockIdx.x * 4, np = min(4, n1 / 2 - jp0);
   const int nx = n0 / 2 + 1;
+  const int cells = n0 * n1 * n2;
+  if (threadIdx.x < 3)
+    prefetch_rows(u + threadIdx.x * cells + (k * n1 + 2 * jp0) * n0, sizeof(float) * 2 * np * n0);
   // a warp takes a line, four groups of 32 modes of both rows in flight
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   for (int l = warp; l < kXL; l += nwarps) {
@@ -740,7 +771,6 @@ __global__ void __launch_bounds__(256, 5) k_spec_out(SpecArgs A, const float* u,
   }
   __syncthreads();
   line_passes<true, N>(A, z);
-  const int cells = n0 * n1 * n2;
   int rp = threadIdx.x / n0, i = threadIdx.x - rp * n0;
   while (rp < np) {
     const int row = (k * n1 + 2 * (jp0 + rp)) * n0 + i;
@@ -830,7 +860,7 @@ __global__ void __launch_bounds__(256) k_spec_resid(SpecArgs A, const float* __r
 
 // f(std::integral_constant<int, N>): N the length where it has compile-time
 // transforms (2^k, 3 2^k and 5 2^k from 32 to 512: the lattices that halve well,
-// which users pick), else 0, any length.  Measured at 192^3: 330 us a step
+// which users pick), else 0, any length.  Measured at 192^3: 328 us a step
 // against 362 us with every length from the arguments; 128^3 115 / 131 us.
 template <int N, typename F>
 bool if_length(int n, F&& f) {
@@ -944,6 +974,14 @@ ib_status spectral_create(Spectral* sp, const int n[3], double h, double rho, do
            (ok(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)kMaxSmem)) && ...);
   };
+  // Planes whose CTAs of the y transforms are resident at once: what a CTA asks
+  // for ahead belongs to the CTA that takes its place.  Only for modes that L2
+  // does not hold (256^3: 106 -> 91 and 113 -> 99 us; 128^3, held, 17.2 -> 17.8).
+  int dev = 0, sms = 0, l2 = 0, per_sm = 0;
+  if (!ok(cudaGetDevice(&dev)) ||
+      !ok(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) ||
+      !ok(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev)))
+    return IB_ERR_CUDA;
   bool good = true;
   with_length(n[0], [&](auto N) {
     constexpr int L = decltype(N)::value;
@@ -952,11 +990,15 @@ ib_status spectral_create(Spectral* sp, const int n[3], double h, double rho, do
   });
   with_length(n[1], [&](auto N) {
     constexpr int L = decltype(N)::value;
-    good = good && opt(sp->smem_y, k_spec_y<false, L>, k_spec_y<true, L>);
+    good = good && opt(sp->smem_y, k_spec_y<false, L>, k_spec_y<true, L>) &&
+           ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spec_y<true, L>,
+                                                            sp->threads_y, sp->smem_y));
   });
   with_length(n[2], [&](auto N) {
     good = good && opt(sp->smem_z, k_spec_solve<decltype(N)::value>);
   });
+  const int plane = (n[0] / 2 + kTX) / kTX * 4;  // CTAs of a plane
+  A.ahead = spec > (size_t)l2 ? (per_sm * sms + plane - 1) / plane : n[2];
   return good ? IB_OK : IB_ERR_CUDA;
 }
 
@@ -973,7 +1015,7 @@ ib_status spectral_step(const Spectral* sp, const float* u, const float* f, floa
   const int ty = (nx + kTX - 1) / kTX, tz = (nx + kTZ - 1) / kTZ;
   // cell pairs by 8-byte loads where the arrays' bases allow (rows are even)
   const bool pairs = ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(f)) & 7) == 0;
-  const dim3 gy(ty, n2, 4), gz(tz, n1);
+  const dim3 gy(ty, 4, n2), gz(tz, n1);
   with_length(A.x.n, [&](auto N) {
     constexpr int L = decltype(N)::value;
     chain_launch(pairs ? k_spec_rhs<2, L> : k_spec_rhs<1, L>, gx, sp->threads_x, sp->smem_x, s, A,

@@ -30,6 +30,7 @@ struct SpecArgs {
   int pitch;
   int xskew;             // shared-memory skew of the x lines per first-pass block
   int zsh, zen;          // shared-memory swap of the z lines
+  int ahead;             // planes that a CTA of the y transforms prefetches ahead
   float alpha, nu;       // rho / dt, mu / h^2
   float inv_n, pscale;   // 1 / cells, -h / dt
 };

@@ -92,6 +92,20 @@ def test_compile_time_lengths_match_oracle(L):
         assert _rms(np_(p) - po) <= tp, n
 
 
+def test_modes_larger_than_l2_match_oracle():
+    """172 MB of modes: the y transforms ask for later planes ahead."""
+    import torch
+    from paper_2503_22695_gb300 import ibfe
+    n = (320, 256, 128)
+    g, u, f = _fields(n, 11)
+    fl = ibfe.Fluid(g.n, g.h, RHO, MU, DT)
+    un, p, _ = ibfe.ib_fluid_step(fl, torch.from_numpy(u).cuda(), torch.from_numpy(f).cuda())
+    us, po, uo = OF.fluid_step(u, f, RHO, MU, DT, g.h)
+    tu, tp = _bounds(u, us, uo, g.h)
+    assert _rms(np_(un) - uo) <= tu
+    assert _rms(np_(p) - po) <= tp
+
+
 @pytest.mark.parametrize("n", [(56, 8, 8), (8, 22, 8), (8, 8, 28), (4, 4, 1024)])
 def test_other_lattices_keep_the_cycles(n):
     import torch
