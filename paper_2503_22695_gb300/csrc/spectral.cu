@@ -34,16 +34,16 @@
 // last, which L2 still holds (k_spec_y<0> and k_spec_out walk the planes
 // backwards): at 256^3 k_spec_out 157 -> 140 us.  Loads that would wait for
 // memory behind the transforms are asked for early: k_spec_out's velocity rows
-// at its start (177 -> 157 us), the y transforms' lines one wave of CTAs ahead
-// (106 -> 91 us).  The same for k_spec_rhs (171 -> 204), the solve (158 -> 168)
+// at its start (177 -> 157 us), the rows that k_spec_rhs is the first to read
+// (171 -> 163), the y transforms' lines one wave of CTAs ahead (106 -> 91).  A wave ahead for k_spec_rhs (171 -> 204), the solve (158 -> 168)
 // and k_spec_out's modes (140 -> 159) costs more than it hides.
 //
 // Measured on GB300 (us; V-cycles of fluid.cu before, this after): 32^3 step
-// 631 -> 46, 192^3 3417 -> 308, 256^3 6550 -> 656.  At 256^3 the five kernels
-// take 171, 91, 157, 99 and 139 us for 0.67, 0.54, 0.54, 0.54 and 0.74 GB:
-// 3.9, 5.9, 3.4, 5.4 and 5.3 TB/s; k_spec_rhs is bound by the L1 data pipe
-// (77% at 192^3), the solve by instruction issue (58%) beside its loads'
-// latency.  x lines use radices up to 8 (48 registers, 5 CTAs per SM: 184
+// 631 -> 46, 192^3 3423 -> 305, 256^3 6550 -> 648.  At 256^3 the five kernels
+// take 163, 90, 157, 99 and 139 us for 0.67, 0.54, 0.54, 0.54 and 0.74 GB:
+// 4.1, 6.0, 3.4, 5.4 and 5.3 TB/s; k_spec_rhs and the solve issue on 56 and
+// 58% of their cycles beside their loads' latency (bank conflicts and L1
+// requests taken out of k_spec_rhs change nothing).  x lines use radices up to 8 (48 registers, 5 CTAs per SM: 184
 // against 250 us with radix 16 for k_spec_out); y lines up to 16 (two passes
 // at 256: 104 against 114..130 us); the z transform holds four fields, 3 CTAs
 // per SM (175 us; 2: 208, 4 with spills: 211).
@@ -493,6 +493,12 @@ __global__ void __launch_bounds__(256, 5) k_spec_rhs(SpecArgs A, const float* __
   const int n0 = N > 0 ? N : A.x.n, n1 = A.y.n, n2 = A.z.n;
   const int k = blockIdx.y, jp0 = blockIdx.x * 4, np = min(4, n1 / 2 - jp0);
   const int cells = n0 * n1 * n2;
+  // the rows that no CTA of an earlier plane has read: u above, f here
+  if (threadIdx.x < 6 && (threadIdx.x < 3 || f))
+    prefetch_rows((threadIdx.x < 3 ? u + threadIdx.x * cells + up(k, n2) * n1 * n0
+                                   : f + (threadIdx.x - 3) * cells + k * n1 * n0) +
+                      2 * jp0 * n0,
+                  sizeof(float) * 2 * np * n0);
   const int kp = up(k, n2) * n1, km = dn(k, n2) * n1, kc = k * n1;
   // a thread forms kV cells of a row pair; work (pair, cells) laid out flat
   const int nv = n0 / kV;
