@@ -167,8 +167,9 @@ struct Stage {
 
 int sort_launches(const ib_plan* p) {
   // FP32 binning: classify, compact (ranges), scatter.  FP64: classify,
-  // compact, radix passes (hist, digit scan, scatter), reorder
-  if (p->precision != IB_FP64) return 3;
+  // compact, radix passes (hist, digit scan, scatter), reorder; few points:
+  // classify, compact, rank
+  if (p->precision != IB_FP64 || rank_sorts(p)) return 3;
   return 3 * ((sort_key_bits(p->ntiles) + 7) / 8) + 3;
 }
 

@@ -337,6 +337,7 @@ ib_status launch_plan_static(ib_plan* p, cudaStream_t s);
 // val_kind: 0 = no value, 1 = w j0 sum_a N_a V_a / m_a from nodal V.
 ib_status launch_points(ib_plan* p, const void* x_cell_or_x64, const float* off,
                         const void* nodal, int val_kind, cudaStream_t s);
+bool rank_sorts(const ib_plan* p);
 ib_status launch_sort_points(ib_plan* p, bool with_val, cudaStream_t s);
 // Carried values of already-built points (unsorted, into q_out or q_val), and
 // their binned copy (from q_in or q_val into p_out or p_val; vmax: also the

@@ -101,3 +101,31 @@ def test_full_items(fp64):
     tf, tU = (1e-12, 1e-12) if fp64 else (1e-5, 1e-6)
     assert rel_l2(np_(f).reshape(3, -1), fo) <= tf
     assert rel_l2(np_(U), Uo) <= tU
+
+
+@pytest.mark.parametrize("N", [513, 16385, 65536, 65537])
+def test_fp64_point_order(N):
+    """FP64 points in every one of 512 tiles, up to and beyond the number that
+    is ordered tile by tile; twice, the same bits."""
+    import torch
+    from paper_2503_22695_gb300 import ibfe
+    n, h = 64, 1.0 / 64
+    rng = np.random.default_rng(N)
+    t = np.concatenate([I.HEX_CORNERS.T * 0.25 + 12.0,
+                        n * rng.uniform(0.001, 0.999, size=(3, N - 8))], axis=1)
+    g = I.Grid((n, n, n), h)
+    conn = torch.arange(8, dtype=torch.int32, device="cuda").reshape(8, 1)
+    plan = ibfe.Plan(conn, torch.from_numpy(t * h).cuda(), g.n, h, quad=ibfe.IB_QUAD_NODAL,
+                     precision=ibfe.IB_FP64)
+    pos = ibfe.Pos(x64=torch.from_numpy(t * h).cuda())
+    G, u = rng.normal(size=(3, N)), rng.normal(size=(3, n, n, n))
+    f = ibfe.ib_spread(plan, pos, torch.from_numpy(G).cuda())
+    assert torch.equal(f, ibfe.ib_spread(plan, pos, torch.from_numpy(G).cuda()))
+    U = ibfe.ib_interp(plan, pos, torch.from_numpy(u).cuda())
+    fo, Uo = np.zeros((3, n ** 3)), np.zeros((3, N))
+    for c in range(3):
+        flat, w = _stencil(t, c, n)
+        fo[c] = np.bincount(flat.ravel(), (w * G[c]).ravel(), n ** 3) / h ** 3
+        Uo[c] = (u[c].ravel()[flat] * w).sum(0)
+    assert rel_l2(np_(f).reshape(3, -1), fo) <= 1e-12
+    assert rel_l2(np_(U), Uo) <= 1e-12
