@@ -375,15 +375,19 @@ ib_status ib_batch_destroy(ib_batch* batch);
  *   rho/dt (u* - u^n) - mu Lap_h u* = f,   Lap_h p = div_h u* / dt,
  *   u^{n+1} = u* - dt grad_h p,
  * with (div u)(i) = sum_c (u^c(i+e_c) - u^c(i))/h, (grad p)^c(i) =
- * (p(i) - p(i-e_c))/h and the 7-point Lap_h = div_h grad_h; both solves by
- * geometric multigrid V-cycles (red-black Gauss-Seidel, 2 pre- and 2
+ * (p(i) - p(i-e_c))/h and the 7-point Lap_h = div_h grad_h.
+ * FP32, lattices whose lengths are even, at most 1024 and have no prime
+ * factor above 5 (n2 at most 900), at the default cycle counts: both solves
+ * directly, by one discrete Fourier transform of the increment
+ * u^{n+1} - u^n (five launches).  Otherwise: geometric multigrid V-cycles
+ * (red-black Gauss-Seidel, 2 pre- and 2
  * post-sweeps; levels halve every dimension while all are even, none is
  * below 4 and the largest exceeds 8; the coarsest is solved in one CTA's
  * shared memory).
  * The cycle counts are fixed (default 2 Helmholtz and 6 Poisson cycles in
- * FP32, 3 and 12 in FP64), so a step involves no host round trip (without
- * residuals it runs as one CUDA graph, captured per set of field pointers);
- * ib_fluid_step can report the residuals reached.  Fields: u, f, u_next device Real [3][n2][n1][n0] (component c on
+ * FP32, 3 and 12 in FP64), so a step involves no host round trip (V-cycles
+ * without residuals run as one CUDA graph, captured per set of field
+ * pointers); ib_fluid_step can report the residuals reached.  Fields: u, f, u_next device Real [3][n2][n1][n0] (component c on
  * the lower c-faces, as everywhere in this API), p device Real [n2][n1][n0]
  * at cell centres with zero mean.  Real is float for the split precisions and
  * double for IB_FP64.  The box is periodic; the paper's no-slip walls are not
@@ -395,12 +399,15 @@ typedef struct ib_fluid ib_fluid;
  * odd size or a coarsest level above 8192 cells, IB_ERR_CAPACITY for
  * 3 n0 n1 n2 >= 2^31) with density rho > 0,
  * viscosity mu >= 0 and time step dt > 0.  Allocates its multigrid hierarchy
- * (about 1.6 field volumes) on the current device. */
+ * (about 1.6 field volumes) and, where the direct solve applies, its modes
+ * (1.4 field volumes) on the current device; without room for the modes every
+ * step runs V-cycles. */
 ib_status ib_fluid_create(const ib_grid* grid, int32_t precision, double rho, double mu,
                           double dt, void* stream, ib_fluid** out);
 ib_status ib_fluid_destroy(ib_fluid* fluid);
 /* V-cycles per Helmholtz solve (all three components together) and per
- * Poisson solve, each in [1, 100]. */
+ * Poisson solve, each in [1, 100].  Counts other than the defaults make every
+ * step run that many V-cycles, also where the direct solve applies. */
 ib_status ib_fluid_set_cycles(ib_fluid* fluid, int32_t helmholtz_cycles, int32_t poisson_cycles);
 ib_status ib_fluid_get_cycles(const ib_fluid* fluid, int32_t cycles[2]);
 /* Number of multigrid levels (the finest included). */
@@ -466,7 +473,7 @@ typedef enum {
   IB_STAGE_FORCE = 0,   /* per-element stress and corner forces */
   IB_STAGE_GATHER = 1,  /* element -> node gathers */
   IB_STAGE_POINTS = 2,  /* Gauss-point positions and carried values */
-  IB_STAGE_SORT = 3,    /* stable radix sort by Eulerian tile + reorder */
+  IB_STAGE_SORT = 3,    /* points ordered by Eulerian tile */
   IB_STAGE_SPREAD = 4,  /* tile-owned spreading onto the grid */
   IB_STAGE_INTERP = 5,  /* Gauss-point interpolation (and its gradients) */
   IB_STAGE_PROJECT = 6, /* Gauss point -> element corner projection */

@@ -4,7 +4,9 @@
 //   Lap_h p = div_h u* / dt                       (Poisson, cell centres)
 //   u^{n+1} = u* - dt grad_h p                    (correction)
 // with a geometric multigrid for both solves (the paper accelerates its
-// solvers with geometric multigrid).
+// solvers with geometric multigrid).  FP32 steps on most lattices take the
+// direct solve of spectral.cu instead (use_direct); the multigrid serves FP64,
+// the other lattices and callers who choose cycle counts.
 //
 // Layout: fields [3][n2][n1][n0] as in the coupling operators (component c on
 // the lower c-faces), p [n2][n1][n0] at cell centres, so that
@@ -576,11 +578,10 @@ ib_status step_spectral(ib_fluid* fl, const float* u, const float* f, float* un,
 }
 }  // namespace
 
-// Advance the fluid one step (internal entry shared with ib_step).  V-cycles
-// without
-// residuals (which need host round trips) the step's ~300 launches run as
-// one CUDA graph, captured on the solver's own stream the first time a set
-// of field pointers is seen; a caller's stream that is itself being
+// Advance the fluid one step (internal entry shared with ib_step).  Without
+// residuals (which need host round trips) the ~300 launches of a V-cycle step
+// run as one CUDA graph, captured on the solver's own stream the first time a
+// set of field pointers is seen; a caller's stream that is itself being
 // captured gets the launches directly.
 ib_status fluid_step_async(ib_fluid* fl, const void* u, const void* f, void* u_next, void* p,
                            double* residuals, cudaStream_t s) {

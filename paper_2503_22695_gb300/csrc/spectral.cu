@@ -16,7 +16,7 @@
 //   d_c = r_c / (a + mu S / h^2),   q = (r_3 + sum_d D_d d_d) / S   (0 at k = 0),
 //   w_c = d_c - conj(D_c) q,        p = -(h / dt) q.
 //
-// Five kernels, all bound by memory (each reads and writes every mode once):
+// Five kernels (each reads and writes every mode once):
 //   k_spec_rhs    stencils and the x transform; two rows of a field make one
 //                 complex line, unpacked to n0/2 + 1 modes per row
 //   k_spec_y<0>   y transform, 16 adjacent modes x one line per thread group
@@ -43,10 +43,11 @@
 // take 163, 90, 157, 99 and 139 us for 0.67, 0.54, 0.54, 0.54 and 0.74 GB:
 // 4.1, 6.0, 3.4, 5.4 and 5.3 TB/s; k_spec_rhs and the solve issue on 56 and
 // 58% of their cycles beside their loads' latency (bank conflicts and L1
-// requests taken out of k_spec_rhs change nothing).  x lines use radices up to 8 (48 registers, 5 CTAs per SM: 184
-// against 250 us with radix 16 for k_spec_out); y lines up to 16 (two passes
-// at 256: 104 against 114..130 us); the z transform holds four fields, 3 CTAs
-// per SM (175 us; 2: 208, 4 with spills: 211).
+// requests taken out of k_spec_rhs change nothing).  Choices measured before
+// the lengths were compiled in: x lines use radices up to 8 (48 registers, 5
+// CTAs per SM: 184 against 250 us with radix 16 for k_spec_out); y lines up to
+// 16 (two passes at 256: 104 against 114..130 us); the z transform holds four
+// fields, 3 CTAs per SM (175 us; 2: 208, 4 with spills: 211).
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -983,11 +984,12 @@ ib_status spectral_create(Spectral* sp, const int n[3], double h, double rho, do
   // Planes whose CTAs of the y transforms are resident at once: what a CTA asks
   // for ahead belongs to the CTA that takes its place.  Only for modes that L2
   // does not hold (256^3: 106 -> 91 and 113 -> 99 us; 128^3, held, 17.2 -> 17.8).
-  int dev = 0, sms = 0, l2 = 0, per_sm = 0;
+  int dev = 0, sms = 0, l2 = 0, per_sm = 1;
   if (!ok(cudaGetDevice(&dev)) ||
       !ok(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) ||
       !ok(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev)))
     return IB_ERR_CUDA;
+  const bool beyond_l2 = spec > (size_t)l2;
   bool good = true;
   with_length(n[0], [&](auto N) {
     constexpr int L = decltype(N)::value;
@@ -997,14 +999,15 @@ ib_status spectral_create(Spectral* sp, const int n[3], double h, double rho, do
   with_length(n[1], [&](auto N) {
     constexpr int L = decltype(N)::value;
     good = good && opt(sp->smem_y, k_spec_y<false, L>, k_spec_y<true, L>) &&
-           ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spec_y<true, L>,
-                                                            sp->threads_y, sp->smem_y));
+           (!beyond_l2 ||
+            ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spec_y<true, L>,
+                                                             sp->threads_y, sp->smem_y)));
   });
   with_length(n[2], [&](auto N) {
     good = good && opt(sp->smem_z, k_spec_solve<decltype(N)::value>);
   });
   const int plane = (n[0] / 2 + kTX) / kTX * 4;  // CTAs of a plane
-  A.ahead = spec > (size_t)l2 ? (per_sm * sms + plane - 1) / plane : n[2];
+  A.ahead = beyond_l2 ? (per_sm * sms + plane - 1) / plane : n[2];
   return good ? IB_OK : IB_ERR_CUDA;
 }
 

@@ -613,7 +613,7 @@ __global__ void __launch_bounds__(kFxThreads, 1024 / kFxThreads)  // 64 register
 // near because of one or two neighbours) is skipped by the whole warp, the
 // sources' offsets are formed once for the three components, and left shifts
 // below 32 take two instructions.  256^3 36 -> 32 us alone (beside the
-// interpolation's end 56 -> 58: the forward 374 -> 376), 118 k nodal points at
+// interpolation's end 56 -> 58: the forward 374 -> 376), 102 k nodal points at
 // 176^3 17.3 -> 14.9, 16 packed shells, both spreadings, 100 -> 90.
 template <bool kPacked>
 __global__ void __launch_bounds__(kMT, 4) k_spread_merge_fx(SpreadArgs<float> A) {
