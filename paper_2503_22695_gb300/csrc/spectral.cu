@@ -39,9 +39,9 @@
 // and k_spec_out's modes (140 -> 159) costs more than it hides.
 //
 // Measured on GB300 (us; V-cycles of fluid.cu before, this after): 32^3 step
-// 631 -> 46, 192^3 3423 -> 305, 256^3 6550 -> 648.  At 256^3 the five kernels
-// take 163, 90, 157, 99 and 139 us for 0.67, 0.54, 0.54, 0.54 and 0.74 GB:
-// 4.1, 6.0, 3.4, 5.4 and 5.3 TB/s; k_spec_rhs and the solve issue on 56 and
+// 631 -> 46, 192^3 3416 -> 285, 256^3 6550 -> 640.  At 256^3 the five kernels
+// take 162, 90, 153, 97 and 137 us for 0.67, 0.54, 0.54, 0.54 and 0.74 GB:
+// 4.1, 6.0, 3.5, 5.6 and 5.4 TB/s; k_spec_rhs and the solve issue on 56 and
 // 58% of their cycles beside their loads' latency (bank conflicts and L1
 // requests taken out of k_spec_rhs change nothing).  Choices measured before
 // the lengths were compiled in: x lines use radices up to 8 (48 registers, 5
@@ -64,8 +64,31 @@ constexpr int kTX = 16;   // modes per tile of the y transform (128-byte rows)
 constexpr int kTZ = 8;    // modes per tile of the z transform (four fields in shared memory)
 constexpr int kMaxN = 1024;
 
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// Sums and differences of both parts in one instruction (the packed FP32
+// arithmetic of this GPU; each part is rounded as by its own instruction).
+// The compiler forms none from the scalar code: the solve at 192^3 75.6 ->
+// 72.2 us, the inverse y transform 59.7 -> 56.3.  Products stay scalar: a
+// complex one would need its factors swapped and doubled in registers.
+__device__ __forceinline__ unsigned long long as_pair(float2 a) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+  return r;
+}
+__device__ __forceinline__ float2 from_pair(unsigned long long r) {
+  float2 a;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a.x), "=f"(a.y) : "l"(r));
+  return a;
+}
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(as_pair(a)), "l"(as_pair(b)));
+  return from_pair(r);
+}
+__device__ __forceinline__ float2 csub(float2 a, float2 b) {
+  unsigned long long r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(as_pair(a)), "l"(as_pair(b)));
+  return from_pair(r);
+}
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
@@ -248,6 +271,20 @@ __host__ __device__ constexpr int col_threads(int n, int r0, int w) {
   const int th = w * (rows / t);
   return th < 32 ? 32 : th;
 }
+
+// Threads of the x and y kernels' CTAs, known with the length, and how many
+// such CTAs 48 registers a thread let an SM hold.  Bounding each instance by
+// its own CTA instead of 256 threads gives the 192-thread ones 56 registers at
+// the same occupancy: the forward y transform at 192^3 58 -> 51 us, the
+// inverse x transform 72 -> 69.
+template <int N, int d>
+constexpr int cta_threads() {
+  if constexpr (N == 0)
+    return 256;
+  else
+    return col_threads(N, make_plan(N, d).rad[0], 16);
+}
+constexpr int ctas_at_48(int threads) { return 1280 / threads; }
 
 // One pass over blocks of L = R Q places: butterfly j takes the places
 // b R Q + m + r Q, r < R, with b = j / Q and m = j mod Q.  magic = 2^20 / Q + 1
@@ -484,7 +521,8 @@ __device__ __forceinline__ void line_passes(const SpecArgs& A, float2* z) {
 // imaginary), their x transform, and the modes 0 .. n0/2 of every row.  Line
 // l = 4 (pair) + field.
 template <int kV, int N>
-__global__ void __launch_bounds__(256, 5) k_spec_rhs(SpecArgs A, const float* __restrict__ u,
+__global__ void __launch_bounds__(cta_threads<N, 0>(), ctas_at_48(cta_threads<N, 0>()))
+    k_spec_rhs(SpecArgs A, const float* __restrict__ u,
                                                   const float* __restrict__ f) {
   chain_wait();
   chain_next();
@@ -593,7 +631,10 @@ __global__ void __launch_bounds__(256, 5) k_spec_rhs(SpecArgs A, const float* __
 // One line of n1 places x kTX adjacent modes of one field and plane.
 constexpr bool has16(int n, int d) { return n == 0 || make_plan(n, d).rad[0] == 16; }
 template <bool kInv, int N>
-__global__ void __launch_bounds__(256, has16(N, 1) ? 3 : 5) k_spec_y(SpecArgs A) {
+__global__ void __launch_bounds__(cta_threads<N, 1>(),
+                                  has16(N, 1) ? 768 / cta_threads<N, 1>()
+                                              : ctas_at_48(cta_threads<N, 1>()))
+    k_spec_y(SpecArgs A) {
   chain_wait();
   chain_next();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -725,7 +766,8 @@ __global__ void __launch_bounds__(256, 3) k_spec_solve(SpecArgs A) {
 // u_next = u + w and p.  kKeep: the increment w is also left in the rows of
 // spec (for the residuals).
 template <bool kKeep, int N>
-__global__ void __launch_bounds__(256, 5) k_spec_out(SpecArgs A, const float* u, float* un,
+__global__ void __launch_bounds__(cta_threads<N, 0>(), ctas_at_48(cta_threads<N, 0>()))
+    k_spec_out(SpecArgs A, const float* u, float* un,
                                                   float* __restrict__ p) {
   chain_wait();
   chain_next();
