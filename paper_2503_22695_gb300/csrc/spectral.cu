@@ -39,7 +39,7 @@
 // and k_spec_out's modes (140 -> 159) costs more than it hides.
 //
 // Measured on GB300 (us; V-cycles of fluid.cu before, this after): 32^3 step
-// 631 -> 46, 192^3 3416 -> 285, 256^3 6550 -> 640.  At 256^3 the five kernels
+// 632 -> 30, 192^3 3416 -> 285, 256^3 6550 -> 640.  At 256^3 the five kernels
 // take 162, 90, 153, 97 and 137 us for 0.67, 0.54, 0.54, 0.54 and 0.74 GB:
 // 4.1, 6.0, 3.5, 5.6 and 5.4 TB/s; k_spec_rhs and the solve issue on 56 and
 // 58% of their cycles beside their loads' latency (bank conflicts and L1
