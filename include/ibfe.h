@@ -500,7 +500,9 @@ double ib_active_tension(double t);
  * returns, and the call returns IB_ERR_TIMEOUT with the context intact.
  * Synchronises `stream`.  Error-path tests may also set the environment
  * variable IBFE_FAULT="entry[:code]", which makes that C entry point (for
- * example ib_forward) return `code` (default IB_ERR_CUDA) before any work. */
+ * example ib_forward) return `code` (default IB_ERR_CUDA) before any work;
+ * the name "points" makes every operator that builds the coupling points
+ * return it there, with that kernel queued. */
 ib_status ib_diag_wait_timeout(double ms, void* stream);
 
 /* Static string for a status code. */

@@ -64,7 +64,9 @@ cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
 // Host-side fault injection for error-path tests: IBFE_FAULT="entry[:code]"
 // makes that C entry point return `code` (default IB_ERR_CUDA) before doing
-// anything.  Read on every call; no device is touched.
+// anything; "points" stands for the stage that builds the coupling points,
+// which then fails with its kernel queued.  Read on every call; no device is
+// touched.
 ib_status injected(const char* entry) {
   const char* spec = std::getenv("IBFE_FAULT");
   if (!spec) return IB_OK;
@@ -173,16 +175,32 @@ int sort_launches(const ib_plan* p) {
   return 3 * ((sort_key_bits(p->ntiles) + 7) / 8) + 3;
 }
 
+bool clear_counts(ib_plan* p, cudaStream_t s) {
+  p->counts_left = !ok(cudaMemsetAsync(p->tile_cnt, 0, 4 * (size_t)p->ntiles, s));
+  return !p->counts_left;
+}
+
 // forward pieces shared by the entry points
+//
+// The points are counted onto tile_cnt, which the binning reads and zeroes.  A
+// call that fails between the two zeroes it instead, behind the points already
+// queued on s (counts left there would add to the next binning's, whose places
+// and work items would then run past the arrays); where that fails too, the
+// next binning begins with it.
 ib_status do_points_sorted(ib_plan* p, const ib_pos* x, const void* nodal, cudaStream_t s) {
+  if (p->counts_left && !clear_counts(p, s)) return IB_ERR_CUDA;
   ib_status st;
   {
     Stage sc(p, IB_STAGE_POINTS, s, 1);
     st = launch_points(p, pos_a(p, x), x->off, nodal, nodal ? 1 : 0, s);
   }
-  if (st != IB_OK) return st;
-  Stage sc(p, IB_STAGE_SORT, s, sort_launches(p));
-  return launch_sort_points(p, nodal != nullptr, s);
+  if (st == IB_OK) st = injected("points");
+  if (st == IB_OK) {
+    Stage sc(p, IB_STAGE_SORT, s, sort_launches(p));
+    st = launch_sort_points(p, nodal != nullptr, s);
+  }
+  if (st != IB_OK) clear_counts(p, s);
+  return st;
 }
 
 ib_status do_interp(ib_plan* p, const void* u, int mode, double vs, double gs, cudaStream_t s,

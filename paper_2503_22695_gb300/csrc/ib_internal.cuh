@@ -229,6 +229,7 @@ struct ib_plan {
                          //      force block counter, [8] its finished CTAs; 1, 2, 4, 5 and 7
                          //      are zeroed by every binning, 6 and 8 by the force kernel
   int32_t* tile_cnt;     // [ntiles] points counted per tile, zero between binnings
+  bool counts_left;      // tile_cnt may hold the counts of a binning that failed half-way
   int32_t* digit_tot;    // [256] radix digit totals
   double* rpart;         // [mat_cap][reduce CTAs][kParamRow] reduction partials
   int* red_count;        // [mat_cap] chunks reduced (zero between calls)
