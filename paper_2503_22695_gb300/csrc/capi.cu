@@ -65,8 +65,9 @@ cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 // Host-side fault injection for error-path tests: IBFE_FAULT="entry[:code]"
 // makes that C entry point return `code` (default IB_ERR_CUDA) before doing
 // anything; "points" stands for the stage that builds the coupling points,
-// which then fails with its kernel queued.  Read on every call; no device is
-// touched.
+// which then fails with its kernel queued, "gather" for the gather from the
+// elements to the nodes, which fails with everything before it queued.  Read on
+// every call; no device is touched.
 ib_status injected(const char* entry) {
   const char* spec = std::getenv("IBFE_FAULT");
   if (!spec) return IB_OK;
@@ -219,6 +220,7 @@ ib_status do_project(ib_plan* p, const void* vals, void* elem, cudaStream_t s) {
 
 ib_status do_gather(ib_plan* p, const void* elem, const void* scale, void* out, cudaStream_t s,
                     const void* add = nullptr, double mul = 1.0) {
+  if (const ib_status f = injected("gather")) return f;
   Stage sc(p, IB_STAGE_GATHER, s, 1);
   return launch_node_gather(p, elem, scale, out, s, add, mul);
 }
@@ -582,6 +584,16 @@ ib_status ib_interp(ib_plan* p, const ib_pos* x, const void* u, void* U, void* s
 
 namespace ibfe {
 
+namespace {
+// A call that fails after forking to a stream of the plan lets s wait for it
+// all the same: what was queued there uses the plan's workspaces and counters,
+// which the calls that follow on s take over, and a capture of s that the
+// stream has joined can only end once it is back.
+void rejoin(cudaStream_t s, cudaStream_t forked, cudaEvent_t ev) {
+  if (ok(cudaEventRecord(ev, forked))) cudaStreamWaitEvent(s, ev, 0);
+}
+}  // namespace
+
 // (U null: without the interpolation)
 ib_status forward_body(ib_plan* p, const MatTable& mt, const ib_pos* x, const void* u, void* G,
                        void* f, void* U, cudaStream_t s, const PackedCalls* pc) {
@@ -595,14 +607,14 @@ ib_status forward_body(ib_plan* p, const MatTable& mt, const ib_pos* x, const vo
   // a packed batch, whose merge and interpolation balance differently, was
   // slower that way (1.17 -> 1.28 ms) and keeps m = s.
   cudaStream_t b = p->side, m = p->n_inst > 1 ? s : p->hi;
-  if (!ok(cudaEventRecord(p->ev_ffork, s)) || !ok(cudaStreamWaitEvent(b, p->ev_ffork, 0)) ||
-      (m != s && !ok(cudaStreamWaitEvent(m, p->ev_ffork, 0))))
+  if (!ok(cudaEventRecord(p->ev_ffork, s)) || !ok(cudaStreamWaitEvent(b, p->ev_ffork, 0)))
     return IB_ERR_CUDA;
+  const bool forked_m = m != s && ok(cudaStreamWaitEvent(m, p->ev_ffork, 0));
   // Issued force first, then the side branch, whose interpolation is best over
   // when the accumulation, which fills the SMs, starts (issued after it: 73 ->
   // 77 us at 128^3), then the rest of the critical one.
-  ib_status st;
-  {
+  ib_status st = m == s || forked_m ? IB_OK : IB_ERR_CUDA;
+  if (st == IB_OK) {
     Stage sc(p, IB_STAGE_FORCE, m, 1);
     st = launch_fe_force(p, mt, pos_a(p, x), x->off, p->elem_scratch, false, m);
   }
@@ -638,6 +650,10 @@ ib_status forward_body(ib_plan* p, const MatTable& mt, const ib_pos* x, const vo
       (!ok(cudaEventRecord(p->ev_hjoin, m)) || !ok(cudaStreamWaitEvent(s, p->ev_hjoin, 0))))
     st = IB_ERR_CUDA;
   if (st == IB_OK && !ok(cudaStreamWaitEvent(s, p->ev_fjoin, 0))) st = IB_ERR_CUDA;
+  if (st != IB_OK) {
+    rejoin(s, b, p->ev_fjoin);
+    if (forked_m) rejoin(s, m, p->ev_hjoin);
+  }
   return check_launch(st);
 }
 
@@ -707,11 +723,12 @@ ib_status backward_body(ib_plan* p, const MatTable& mt, int n_mats, const ib_pos
   // it after the spreading adjoint, beside the force adjoint alone (forking
   // at the binning took 2.3 -> 3.3 ms for the 48-instance sweep).
   const InterpIO io_u = {p->p_val_b, nullptr, p->gq_c, 4};
+  bool forked_b = false, forked_r = false;
   auto side = [&]() {
-    if (!gU) return;
-    if (st == IB_OK && (!ok(cudaEventRecord(p->ev_ffork, s)) ||
-                        !ok(cudaStreamWaitEvent(b, p->ev_ffork, 0))))
+    if (!gU || st != IB_OK) return;
+    if (!ok(cudaEventRecord(p->ev_ffork, s)) || !ok(cudaStreamWaitEvent(b, p->ev_ffork, 0)))
       st = IB_ERR_CUDA;
+    forked_b = st == IB_OK;
     if (st == IB_OK) {
       Stage sc(p, IB_STAGE_POINTS, b, binned_values_launches(p));
       st = launch_binned_values(p, gU, b, true, p->q_val_b, p->p_val_b);
@@ -752,9 +769,11 @@ ib_status backward_body(ib_plan* p, const MatTable& mt, int n_mats, const ib_pos
   // high-priority stream beside the rest (one structure)
   const bool reduce = force && params;
   cudaStream_t r = pc ? s : p->hi;
-  if (reduce && st == IB_OK && r != s &&
-      (!ok(cudaEventRecord(p->ev_fsorted, s)) || !ok(cudaStreamWaitEvent(r, p->ev_fsorted, 0))))
-    st = IB_ERR_CUDA;
+  if (reduce && st == IB_OK && r != s) {
+    if (!ok(cudaEventRecord(p->ev_fsorted, s)) || !ok(cudaStreamWaitEvent(r, p->ev_fsorted, 0)))
+      st = IB_ERR_CUDA;
+    forked_r = st == IB_OK;
+  }
   if (st == IB_OK && reduce) st = do_reduce(p, kParamRow, n_mats, r, true, gparams);
   if (reduce && st == IB_OK && r != s && !ok(cudaEventRecord(p->ev_hjoin, r))) st = IB_ERR_CUDA;
   if (!pc && st == IB_OK && gf) st = to_nodes(p, p->gq_b, p->elem_scratch2, nullptr, gx, s);
@@ -773,6 +792,10 @@ ib_status backward_body(ib_plan* p, const MatTable& mt, int n_mats, const ib_pos
       !ok(cudaMemsetAsync(gparams ? gparams : p->ered, 0,
                           sizeof(double) * kParamRow * (size_t)n_mats, s)))
     st = IB_ERR_CUDA;
+  if (st != IB_OK) {
+    if (forked_b) rejoin(s, b, p->ev_fjoin);
+    if (forked_r) rejoin(s, r, p->ev_hjoin);
+  }
   return check_launch(st);
 }
 

@@ -48,3 +48,48 @@ def test_points_counted_by_a_failed_call_are_forgotten(fp64, quad, monkeypatch):
         monkeypatch.delenv("IBFE_FAULT")
         assert _equal(ops(), ref)
     assert ibfe.ib_plan_sync_status(c.plan) == ibfe.IB_OK
+
+
+@pytest.mark.parametrize("stage", ["points", "gather"])
+@pytest.mark.parametrize("fp64", [False, True])
+def test_failed_calls_rejoin_the_plans_streams(fp64, stage, monkeypatch):
+    """The fused operators fork to streams of the plan.  One that fails there
+    lets the caller's stream wait for them: the next call on that stream finds
+    the workspaces and counters unused, and a capture of the stream can end."""
+    import torch
+    c = _case(fp64)
+    ibfe = c.ibfe
+    gf = c.to_dev(np.random.default_rng(4).normal(size=c.prob.u.shape) * 1e-3)
+    G, f, U = ibfe.ib_forward(c.plan, c.mats, c.pos, c.u)
+    out = [torch.empty_like(t) for t in (G, f, U, G, f)]
+
+    def forward():
+        return ibfe.ib_forward(c.plan, c.mats, c.pos, c.u, *out[:3])
+
+    def backward():
+        return ibfe.ib_backward(c.plan, c.mats, c.pos, c.u, G, c.gU, gf, c.gU, *out[3:])
+
+    def direct():
+        return (ibfe.ib_fe_force(c.plan, c.mats, c.pos), ibfe.ib_spread(c.plan, c.pos, c.G),
+                *ibfe.ib_fe_force_adj(c.plan, c.mats, c.pos, c.gU))
+
+    refs = [[t.clone() for t in op()] for op in (direct, forward, backward)]
+    side = torch.cuda.Stream()
+    for op in (forward, backward):
+        monkeypatch.setenv("IBFE_FAULT", stage)
+        with pytest.raises(ibfe.IBError):
+            op()
+        monkeypatch.delenv("IBFE_FAULT")
+        assert _equal(direct(), refs[0])
+        # captured: the graph holds what was queued before the failure
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side):
+            monkeypatch.setenv("IBFE_FAULT", stage)
+            with pytest.raises(ibfe.IBError):
+                op()
+            monkeypatch.delenv("IBFE_FAULT")
+        graph.replay()
+        for fn, ref in zip((direct, forward, backward), refs):
+            assert _equal(fn(), ref)
+    assert ibfe.ib_plan_sync_status(c.plan) == ibfe.IB_OK
