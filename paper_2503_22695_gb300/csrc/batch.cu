@@ -424,6 +424,7 @@ extern "C" {
 
 ib_status ib_batch_create(int32_t n, const ib_instance* inst, int32_t precision, void* stream,
                           ib_batch** out) {
+  if (const ib_status f = enter("ib_batch_create")) return f;
   if (!out) return IB_ERR_INVALID_ARG;
   *out = nullptr;
   if (n <= 0 || !inst || precision != IB_FP32_SPLIT) return IB_ERR_INVALID_ARG;
@@ -463,12 +464,14 @@ ib_status ib_batch_create(int32_t n, const ib_instance* inst, int32_t precision,
 }
 
 ib_status ib_batch_forward(ib_batch* b, void* stream) {
+  if (const ib_status f = enter("ib_batch_forward")) return f;
   if (!b || !b->fwd) return IB_ERR_INVALID_ARG;
   return ok(cudaGraphLaunch(b->fwd, reinterpret_cast<cudaStream_t>(stream))) ? IB_OK
                                                                              : IB_ERR_CUDA;
 }
 
 ib_status ib_batch_adjoint(ib_batch* b, void* stream) {
+  if (const ib_status f = enter("ib_batch_adjoint")) return f;
   if (!b || !b->adj) return IB_ERR_INVALID_ARG;
   return ok(cudaGraphLaunch(b->adj, reinterpret_cast<cudaStream_t>(stream))) ? IB_OK
                                                                              : IB_ERR_CUDA;

@@ -66,8 +66,9 @@ cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 // makes that C entry point return `code` (default IB_ERR_CUDA) before doing
 // anything; "points" stands for the stage that builds the coupling points,
 // which then fails with its kernel queued, "gather" for the gather from the
-// elements to the nodes, which fails with everything before it queued.  Read on
-// every call; no device is touched.
+// elements to the nodes, which fails with everything before it queued;
+// "earlier_error" leaves an error with the runtime ahead of every call.  Read
+// on every call; no device is touched.
 ib_status injected(const char* entry) {
   const char* spec = std::getenv("IBFE_FAULT");
   if (!spec) return IB_OK;
@@ -127,6 +128,20 @@ void prof_flush(ib_plan* p) {
 }
 
 }  // namespace
+
+// The first thing an entry point that launches does.  Launches are judged by
+// cudaGetLastError(), which also returns what an earlier call left there (a
+// refused allocation, a failed capture): that is not this call's error, and
+// taking it for one would end the call half-way.
+ib_status ibfe::enter(const char* entry) {
+  if (const char* spec = std::getenv("IBFE_FAULT"))
+    if (!std::strcmp(spec, "earlier_error")) {  // an error of the host API, refused as an argument
+      int v;
+      cudaDeviceGetAttribute(&v, cudaDevAttrWarpSize, -1);
+    }
+  cudaGetLastError();
+  return injected(entry);
+}
 
 // Profiler intervals: a begin reserves an event pair and records its first
 // event; the end records the second.  Intervals may nest (a kernel inside a
@@ -291,7 +306,7 @@ const char* ib_status_str(ib_status s) {
 
 ib_status ib_plan_create(const ib_mesh* mesh, const ib_grid* grid, int32_t quad,
                          int32_t precision, void* stream, ib_plan** out) {
-  if (const ib_status f = injected("ib_plan_create")) return f;
+  if (const ib_status f = enter("ib_plan_create")) return f;
   if (!out) return IB_ERR_INVALID_ARG;
   *out = nullptr;
   if (!mesh || !grid) return IB_ERR_INVALID_ARG;
@@ -526,7 +541,7 @@ ib_status ib_lumped_mass(ib_plan* p, void* mass, void* stream) {
 
 ib_status ib_fe_force(ib_plan* p, const ib_material* mats, int32_t n_mats, const ib_pos* x,
                       void* G, double* energy, void* stream) {
-  if (const ib_status f = injected("ib_fe_force")) return f;
+  if (const ib_status f = enter("ib_fe_force")) return f;
   if (!p || !G) return IB_ERR_INVALID_ARG;
   ib_status st = check_pos(p, x);
   if (st != IB_OK) return st;
@@ -559,7 +574,7 @@ ib_status ib_fe_force(ib_plan* p, const ib_material* mats, int32_t n_mats, const
 }
 
 ib_status ib_spread(ib_plan* p, const ib_pos* x, const void* G, void* f, void* stream) {
-  if (const ib_status f = injected("ib_spread")) return f;
+  if (const ib_status f = enter("ib_spread")) return f;
   if (!p || !G || !f || !aligned16(f)) return IB_ERR_INVALID_ARG;
   ib_status st = check_pos(p, x);
   if (st != IB_OK) return st;
@@ -570,7 +585,7 @@ ib_status ib_spread(ib_plan* p, const ib_pos* x, const void* G, void* f, void* s
 }
 
 ib_status ib_interp(ib_plan* p, const ib_pos* x, const void* u, void* U, void* stream) {
-  if (const ib_status f = injected("ib_interp")) return f;
+  if (const ib_status f = enter("ib_interp")) return f;
   if (!p || !u || !U) return IB_ERR_INVALID_ARG;
   ib_status st = check_pos(p, x);
   if (st != IB_OK) return st;
@@ -663,7 +678,7 @@ extern "C" {
 
 ib_status ib_forward(ib_plan* p, const ib_material* mats, int32_t n_mats, const ib_pos* x,
                      const void* u, void* G, void* f, void* U, void* stream) {
-  if (const ib_status f = injected("ib_forward")) return f;
+  if (const ib_status f = enter("ib_forward")) return f;
   if (!p || !u || !G || !f || !U || !aligned16(f) || p->n_inst > 1) return IB_ERR_INVALID_ARG;
   ib_status st = check_pos(p, x);
   if (st != IB_OK) return st;
@@ -674,7 +689,7 @@ ib_status ib_forward(ib_plan* p, const ib_material* mats, int32_t n_mats, const 
 
 ib_status ib_step(ib_plan* p, ib_fluid* fl, const ib_material* mats, int32_t n_mats,
                   const ib_pos* x, void* u, void* G, void* f, void* U, void* pr, void* stream) {
-  if (const ib_status f = injected("ib_step")) return f;
+  if (const ib_status f = enter("ib_step")) return f;
   if (!p || !fl || !u || !G || !f || !U || !aligned16(f) || !aligned16(u) ||
       !fluid_matches(fl, p))
     return IB_ERR_INVALID_ARG;
@@ -806,7 +821,7 @@ extern "C" {
 ib_status ib_backward(ib_plan* p, const ib_material* mats, int32_t n_mats, const ib_pos* x,
                       const void* u, const void* G, const void* gG, const void* gf,
                       const void* gU, void* gx, void* gu, double* gparams, void* stream) {
-  if (const ib_status f = injected("ib_backward")) return f;
+  if (const ib_status f = enter("ib_backward")) return f;
   if (!p || !gx || (gf && !G) || (gU && (!gu || !u)) || (gu && !aligned16(gu)) || p->n_inst > 1)
     return IB_ERR_INVALID_ARG;
   ib_status st = check_pos(p, x);
@@ -819,7 +834,7 @@ ib_status ib_backward(ib_plan* p, const ib_material* mats, int32_t n_mats, const
 
 ib_status ib_spread_adj(ib_plan* p, const ib_pos* x, const void* G, const void* gf, void* gG,
                         void* gx, void* stream) {
-  if (const ib_status f = injected("ib_spread_adj")) return f;
+  if (const ib_status f = enter("ib_spread_adj")) return f;
   if (!p || !G || !gf || !gG) return IB_ERR_INVALID_ARG;
   ib_status st = check_pos(p, x);
   if (st != IB_OK) return st;
@@ -834,7 +849,7 @@ ib_status ib_spread_adj(ib_plan* p, const ib_pos* x, const void* G, const void* 
 
 ib_status ib_interp_adj(ib_plan* p, const ib_pos* x, const void* u, const void* gU, void* gu,
                         void* gx, void* stream) {
-  if (const ib_status f = injected("ib_interp_adj")) return f;
+  if (const ib_status f = enter("ib_interp_adj")) return f;
   if (!p || !gU || !gu || (gx && !u) || !aligned16(gu)) return IB_ERR_INVALID_ARG;
   ib_status st = check_pos(p, x);
   if (st != IB_OK) return st;
@@ -876,7 +891,7 @@ extern "C" {
 
 ib_status ib_fe_force_adj(ib_plan* p, const ib_material* mats, int32_t n_mats, const ib_pos* x,
                           const void* v, void* Hv, double* gparams, void* stream) {
-  if (const ib_status f = injected("ib_fe_force_adj")) return f;
+  if (const ib_status f = enter("ib_fe_force_adj")) return f;
   cudaStream_t s = S(stream);
   ib_status st = fe_force_adj_async(p, mats, n_mats, x, v, Hv, gparams != nullptr, s);
   if (st == IB_OK && gparams) {
@@ -1000,6 +1015,7 @@ extern "C" {
 
 ib_status ib_plan_autotune(ib_plan* p, const ib_material* mats, int32_t n_mats,
                            const ib_pos* x, const void* u, void* stream, int32_t tuning[4]) {
+  if (const ib_status f = enter("ib_plan_autotune")) return f;
   if (!p || !u) return IB_ERR_INVALID_ARG;
   ib_status st = check_pos(p, x);
   if (st != IB_OK) return st;
@@ -1061,6 +1077,7 @@ ib_status ib_plan_profile(ib_plan* p, void* stream, double* ms, int64_t* calls,
 }
 
 ib_status ib_diag_wait_timeout(double ms, void* stream) {
+  if (const ib_status f = enter("ib_diag_wait_timeout")) return f;
   if (!(ms > 0.0) || ms > 10000.0) return IB_ERR_INVALID_ARG;
   cudaStream_t s = S(stream);
   int* d = nullptr;

@@ -637,6 +637,7 @@ extern "C" {
 ib_status ib_fluid_create(const ib_grid* grid, int32_t precision, double rho, double mu,
                           double dt, void* stream, ib_fluid** out) {
   using namespace ibfe;
+  if (const ib_status e = enter("ib_fluid_create")) return e;
   if (!grid || !out) return IB_ERR_INVALID_ARG;
   *out = nullptr;
   if (precision != IB_FP32_SPLIT && precision != IB_FP64 && precision != IB_FP32_SPLIT_F32STAB)
@@ -788,6 +789,7 @@ ib_status ib_fluid_levels(const ib_fluid* fl, int32_t* levels) {
 
 ib_status ib_fluid_step(ib_fluid* fl, const void* u, const void* f, void* u_next, void* p,
                         double* residuals, void* stream) {
+  if (const ib_status e = ibfe::enter("ib_fluid_step")) return e;
   if (!fl || !u || !u_next) return IB_ERR_INVALID_ARG;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   ib_status st = ibfe::fluid_step_async(fl, u, f, u_next, p, residuals, s);

@@ -43,6 +43,10 @@ cudaError_t chain_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t sme
   return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
 
+// Start of a C entry point that launches: drops an error left by an earlier call;
+// returns the status injected for `entry`, if any (capi.cu).
+ib_status enter(const char* entry);
+
 // Calls f(std::integral_constant<int, kEl>) for the plan's element type.
 template <typename F>
 void with_elem(int elem, F&& f) {

@@ -221,6 +221,7 @@ extern "C" ib_status ib_fe_energy_noalloc(const ib_mesh* mesh, const ib_material
                                           int32_t n_mats, const ib_pos* x, double h,
                                           double* energy, void* stream) {
   using namespace ibfe;
+  if (const ib_status f = enter("ib_fe_energy_noalloc")) return f;
   if (!mesh || !mats || !x || !energy || !x->cell || !x->off || !mesh->X) return IB_ERR_INVALID_ARG;
   if (mesh->n_nodes <= 0 || mesh->n_elems < 0 || (mesh->n_elems > 0 && !mesh->conn))
     return IB_ERR_INVALID_ARG;

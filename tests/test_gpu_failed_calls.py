@@ -93,3 +93,54 @@ def test_failed_calls_rejoin_the_plans_streams(fp64, stage, monkeypatch):
         for fn, ref in zip((direct, forward, backward), refs):
             assert _equal(fn(), ref)
     assert ibfe.ib_plan_sync_status(c.plan) == ibfe.IB_OK
+
+
+@pytest.mark.parametrize("fp64", [False, True])
+def test_an_earlier_error_is_not_the_next_calls(fp64, monkeypatch):
+    """An error that another call left with the runtime (a refused allocation)
+    neither fails a call nor ends it half-way."""
+    import torch
+    c = _case(fp64)
+    ibfe = c.ibfe
+    gf = c.to_dev(np.random.default_rng(4).normal(size=c.prob.u.shape) * 1e-3)
+    prec = ibfe.IB_FP64 if fp64 else ibfe.IB_FP32_SPLIT
+    g = c.prob.grid
+
+    def ops():
+        out = [ibfe.ib_fe_force(c.plan, c.mats, c.pos), ibfe.ib_spread(c.plan, c.pos, c.G),
+               ibfe.ib_interp(c.plan, c.pos, c.u)]
+        out += ibfe.ib_forward(c.plan, c.mats, c.pos, c.u)
+        out += ibfe.ib_backward(c.plan, c.mats, c.pos, c.u, out[3], c.gU, gf, c.gU)
+        out += ibfe.ib_spread_adj(c.plan, c.pos, c.G, gf)
+        out += ibfe.ib_interp_adj(c.plan, c.pos, c.u, c.gU)
+        out += ibfe.ib_fe_force_adj(c.plan, c.mats, c.pos, c.gU)
+        fl = ibfe.Fluid(g.n, g.h, 1.0, 0.02, 2e-4, precision=prec)
+        out += ibfe.ib_fluid_step(fl, c.u, out[4])[:2]
+        if fp64:
+            pos = ibfe.Pos(x64=c.pos.x64.clone())
+        else:
+            pos = ibfe.Pos(cell=c.pos.cell.clone(), off=c.pos.off.clone())
+        out += ibfe.ib_step(c.plan, fl, c.mats, pos, c.u.clone())
+        if not fp64:
+            inst = []
+            for _ in range(2):
+                d = dict(conn=c.conn, X=c.X, fibres=c.fib, mat_id=c.mat_id, n=g.n, h=g.h,
+                         mats=c.mats, cell=c.cell, off=c.off, u=c.u, gU=c.gU, gf=gf)
+                d.update({k: torch.empty_like(c.G) for k in ("G", "U", "gx")})
+                d.update({k: torch.empty_like(c.u) for k in ("f", "gu")})
+                inst.append(d)
+            b = ibfe.Batch(inst)
+            b.forward()
+            b.adjoint()
+            out += [d[k] for d in inst for k in ("G", "U", "gx", "f", "gu")] + [b.gparams()]
+            e = torch.empty(1, device="cuda", dtype=torch.float64)
+            out += [ibfe.ib_fe_energy_noalloc(c.conn, c.X, c.mats, c.pos, g.h, e, fibres=c.fib,
+                                              mat_id=c.mat_id)]
+        return out
+
+    ref = ops()
+    monkeypatch.setenv("IBFE_FAULT", "earlier_error")
+    again = ops()
+    monkeypatch.delenv("IBFE_FAULT")
+    assert _equal(again, ref)
+    assert ibfe.ib_plan_sync_status(c.plan) == ibfe.IB_OK
