@@ -744,7 +744,7 @@ ib_status ib_fluid_create(const ib_grid* grid, int32_t precision, double rho, do
   }
   // without room for its workspace the V-cycles serve every step
   if (precision != IB_FP64 && spectral_supports(fl->n)) {
-    fl->direct = spectral_create(&fl->spec, fl->n, fl->h, rho, mu, dt) == IB_OK;
+    fl->direct = spectral_create(&fl->spec, fl->n, fl->h, rho, mu, dt, fl->cap) == IB_OK;
     if (!fl->direct) {
       spectral_destroy(&fl->spec);
       cudaGetLastError();

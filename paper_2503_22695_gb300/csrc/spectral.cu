@@ -941,7 +941,7 @@ bool spectral_supports(const int n[3]) {
 }
 
 ib_status spectral_create(Spectral* sp, const int n[3], double h, double rho, double mu,
-                          double dt) {
+                          double dt, cudaStream_t up) {
   SpecArgs& A = sp->a;
   SpecDim* dims[3] = {&A.x, &A.y, &A.z};
   const double pi = 3.14159265358979323846;
@@ -997,7 +997,13 @@ ib_status spectral_create(Spectral* sp, const int n[3], double h, double rho, do
   const size_t spec = (sizeof(float2) * 4 * (size_t)n[2] * n[1] * A.pitch + 255) / 256 * 256;
   if (!ok(cudaMalloc((void**)&A.spec, spec + host.size()))) return IB_ERR_CUDA;
   char* const t = reinterpret_cast<char*>(A.spec) + spec;  // the tables behind the modes
-  if (!ok(cudaMemcpy(t, host.data(), host.size(), cudaMemcpyHostToDevice))) return IB_ERR_CUDA;
+  // The tables are on the device when the solver is handed out, whatever stream
+  // it is first used on.  A plain copy from pageable memory may return with its
+  // last part still on the way, in the order of the legacy stream alone, which
+  // non-blocking streams do not wait for; one wait per solver.
+  if (!ok(cudaMemcpyAsync(t, host.data(), host.size(), cudaMemcpyHostToDevice, up)) ||
+      !ok(cudaStreamSynchronize(up)))
+    return IB_ERR_CUDA;
   for (int d = 0; d < 3; ++d) dims[d]->tw = reinterpret_cast<const float2*>(t + tw_at[d]);
   A.symx = reinterpret_cast<const float4*>(t + sym_at[0]);
   A.symy = reinterpret_cast<const float4*>(t + sym_at[1]);

@@ -44,8 +44,10 @@ struct Spectral {
 // Lattices the direct solve takes: every length even, at most 1024, with no
 // prime factor above 5.
 bool spectral_supports(const int n[3]);
+// up: a stream of the caller's that nothing is queued on (the tables' upload,
+// waited for)
 ib_status spectral_create(Spectral* sp, const int n[3], double h, double rho, double mu,
-                          double dt);
+                          double dt, cudaStream_t up);
 void spectral_destroy(Spectral* sp);
 // keep: leave the increment w in the rows of a.spec (for the residuals)
 ib_status spectral_step(const Spectral* sp, const float* u, const float* f, float* un, float* p,

@@ -1,0 +1,43 @@
+"""The fluid solver object: its first step on any stream."""
+import numpy as np
+import pytest
+
+from oracle import fluid as OF
+from paper_2503_22695_gb300 import inputs as I
+
+from helpers import np_, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+RHO, MU, DT = 1.0, 0.02, 2e-4
+
+
+def _fields(n, seed):
+    """As test_gpu_fluid's: solenoidal modes and white noise, a white force."""
+    g = I.Grid(tuple(n), 1.0 / n[0])
+    rng = np.random.Generator(np.random.PCG64(seed))
+    u = I.fourier_velocity(g, 6, rng, dtype=np.float64)
+    u = (u + 0.1 * rng.normal(size=u.shape)).astype(np.float32)
+    f = (50.0 * rng.normal(size=u.shape)).astype(np.float32)
+    return g, u, f
+
+
+@pytest.mark.parametrize("n", [(16, 16, 16), (1024, 8, 8), (48, 40, 360)])
+def test_first_step_on_another_stream(n):
+    """A solver created and used at once on a stream that does not wait for the
+    default one has its tables: the bits of a solver used later."""
+    import torch
+    from paper_2503_22695_gb300 import ibfe
+    g, u, f = _fields(n, 1)
+    ud, fd = torch.from_numpy(u).cuda(), torch.from_numpy(f).cuda()
+    ref = ibfe.Fluid(g.n, g.h, RHO, MU, DT)
+    torch.cuda.synchronize()
+    a, pa, _ = ibfe.ib_fluid_step(ref, ud, fd)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    for _ in range(20):
+        with torch.cuda.stream(side):
+            fl = ibfe.Fluid(g.n, g.h, RHO, MU, DT)
+            b, pb, _ = ibfe.ib_fluid_step(fl, ud, fd)
+        side.synchronize()
+        assert torch.equal(a, b) and torch.equal(pa, pb)
