@@ -500,6 +500,25 @@ __device__ __forceinline__ void prefetch_rows(const void* g, int bytes) {
                  : "memory");
 }
 
+// The lines a warp of a CTA of `threads` threads takes are first_line(warp),
+// and from there every (threads / 32)-th.  CTAs are multiples of 16 threads (a
+// column each per place): the half warp that some end in takes no line, as the
+// full warps take them all.
+__host__ __device__ constexpr int first_line(int warp, int threads) {
+  return warp < threads / 32 ? warp : kXL;
+}
+constexpr bool each_line_once() {
+  for (int threads = 32; threads <= 256; threads += 16)
+    for (int l = 0; l < kXL; ++l) {
+      int takers = 0;
+      for (int w = 0; w < (threads + 31) / 32; ++w)
+        for (int k = first_line(w, threads); k < kXL; k += threads / 32) takers += k == l;
+      if (takers != 1) return false;
+    }
+  return true;
+}
+static_assert(each_line_once(), "two warps on a line would race on its places and modes");
+
 // Transforms the 16 lines held in shared memory.
 template <bool kInv, int N>
 __device__ __forceinline__ void line_passes(const SpecArgs& A, float2* z) {
@@ -614,8 +633,8 @@ __global__ void __launch_bounds__(cta_threads<N, 0>(), ctas_at_48(cta_threads<N,
   //   2 a_k = z_k + conj z_{n-k},  2 b_k = -i (z_k - conj z_{n-k})
   // (the factor 2 is in inv_n)
   const int nx = n0 / 2 + 1;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  for (int l = warp; l < 4 * np; l += nwarps) {
+  const int lane = threadIdx.x & 31, threads = N > 0 ? cta_threads<N, 0>() : (int)blockDim.x;
+  for (int l = first_line(threadIdx.x >> 5, threads); l < 4 * np; l += threads / 32) {
     float2* o = A.spec + ((int64_t)((l & 3) * n2 + k) * n1 + 2 * (jp0 + (l >> 2))) * A.pitch;
     const float2* zl = z + l;
 #pragma unroll 4
@@ -781,8 +800,8 @@ __global__ void __launch_bounds__(cta_threads<N, 0>(), ctas_at_48(cta_threads<N,
   if (threadIdx.x < 3)
     prefetch_rows(u + threadIdx.x * cells + (k * n1 + 2 * jp0) * n0, sizeof(float) * 2 * np * n0);
   // a warp takes a line, four groups of 32 modes of both rows in flight
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  for (int l = warp; l < kXL; l += nwarps) {
+  const int lane = threadIdx.x & 31, threads = N > 0 ? cta_threads<N, 0>() : (int)blockDim.x;
+  for (int l = first_line(threadIdx.x >> 5, threads); l < kXL; l += threads / 32) {
     const bool on = l < 4 * np;
     const float2* g =
         A.spec + ((int64_t)((l & 3) * n2 + k) * n1 + 2 * (jp0 + (on ? l >> 2 : 0))) * A.pitch;
