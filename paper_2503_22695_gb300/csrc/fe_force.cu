@@ -13,8 +13,9 @@ namespace {
 // Deterministic per-material sums of per-element partials, one launch.
 // Material m's elements lie in the range mrange[m] (the whole mesh for a plan
 // of one structure; its instance's elements in a packed plan), cut into at
-// most kReduceCTAs chunks of at least kRedMin elements; CTA (b, m) sums chunk
-// b: each thread its elements in order, then one warp per value the threads'
+// most kReduceCTAs chunks of at least kRedMin elements; CTA per_mat m + b sums
+// its chunk b (one grid dimension: a packed plan may have more materials than
+// the others hold): each thread its elements in order, then one warp per value the threads'
 // sums (eight per lane, then a shuffle tree).  The CTA that completes its
 // material's count adds the chunks' sums, again one warp per value in a fixed
 // order.  The partition and the trees depend only on the range, so an
@@ -39,18 +40,19 @@ template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_reduce(const T* __restrict__ part,
                                                         const int32_t* __restrict__ mat_id,
                                                         const int2* __restrict__ mrange, int E,
-                                                        int nvals, double* rpart, int* count,
-                                                        double* __restrict__ out) {
+                                                        int nvals, int per_mat, double* rpart,
+                                                        int* count, double* __restrict__ out) {
   chain_wait();
   __shared__ double sh[kParamRow][kRedThreads];
   __shared__ bool last;
-  const int m = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int m = blockIdx.x / per_mat, b = blockIdx.x % per_mat;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int2 r = mrange[m];
   const int len = r.y - r.x;
   const int chunk = max(kRedMin, (len + kReduceCTAs - 1) / kReduceCTAs);
   const int nblk = max(1, (len + chunk - 1) / chunk);
-  if ((int)blockIdx.x >= nblk) return;
-  const int e0 = r.x + blockIdx.x * chunk, e1 = min(r.y, e0 + chunk);
+  if (b >= nblk) return;
+  const int e0 = r.x + b * chunk, e1 = min(r.y, e0 + chunk);
   double s[kParamRow];
 #pragma unroll
   for (int k = 0; k < kParamRow; ++k) s[k] = 0.0;
@@ -75,7 +77,7 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce(const T* __restrict__ pa
       if (nblk == 1)
         out[m * kParamRow + k] = v;
       else
-        mine[blockIdx.x * kParamRow + k] = v;
+        mine[b * kParamRow + k] = v;
     }
   }
   if (nblk == 1) return;
@@ -90,7 +92,7 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce(const T* __restrict__ pa
   __threadfence();
   for (int k = warp; k < nvals; k += kRedThreads / 32) {
     double v = 0.0;
-    for (int b = lane; b < nblk; b += 32) v += __ldcg(mine + b * kParamRow + k);
+    for (int i = lane; i < nblk; i += 32) v += __ldcg(mine + i * kParamRow + k);
     v = warp_tree(v);
     if (lane == 0) out[m * kParamRow + k] = v;
   }
@@ -227,14 +229,14 @@ ib_status launch_reduce_parts(ib_plan* p, int nvals, int n_mats, cudaStream_t s,
   }
   // chunks any material can have: the whole mesh's
   const int nblk = std::min(kReduceCTAs, (p->E + kRedMin - 1) / kRedMin);
-  const dim3 grid(nblk, n_mats);
+  const unsigned grid = (unsigned)nblk * (unsigned)n_mats;
   // FP32 partials are widened exactly: the sums are those of their doubles
   if (real_parts && p->precision != IB_FP64)
     chain_launch(k_reduce<float>, grid, kRedThreads, 0, s, reinterpret_cast<const float*>(p->epart),
-                 p->mat_id, p->mat_range, p->E, nvals, p->rpart, p->red_count, out);
+                 p->mat_id, p->mat_range, p->E, nvals, nblk, p->rpart, p->red_count, out);
   else
     chain_launch(k_reduce<double>, grid, kRedThreads, 0, s, p->epart, p->mat_id, p->mat_range, p->E,
-                 nvals, p->rpart, p->red_count, out);
+                 nvals, nblk, p->rpart, p->red_count, out);
   return cudaGetLastError() == cudaSuccess ? IB_OK : IB_ERR_CUDA;
 }
 

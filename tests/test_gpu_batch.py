@@ -178,3 +178,41 @@ def test_batch_sweep_against_fp64_gpu_form(sweep):
         assert rel_l2(o["f"], f64) <= TOL["f"], i
         assert rel_l2(o["U"], U64) <= TOL["U"], i
         del plan
+
+
+def test_more_material_rows_than_a_grid_dimension_holds():
+    """8200 instances of 8 materials: 65,600 rows of parameter gradients.  The
+    first and the last instance have the bits of plans of their own."""
+    import torch
+    from paper_2503_22695_gb300 import ibfe
+    n, g, h = 8200, 16, 1.0 / 16
+    rng = np.random.default_rng(3)
+    X = ((I.HEX_CORNERS.T + 6.0) * h).astype(np.float32)
+    x = X.astype(np.float64) + rng.uniform(-0.1 * h, 0.1 * h, size=X.shape)
+    cell, off = I.to_split(x, I.Grid((g, g, g), h))
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    rnd = lambda *s: dev(rng.normal(size=s).astype(np.float32))
+    shared = dict(conn=torch.arange(8, dtype=torch.int32, device="cuda").reshape(8, 1), X=dev(X),
+                  n=(g, g, g), h=h, cell=dev(cell), off=dev(off), u=rnd(3, g, g, g),
+                  gU=rnd(3, 8), gf=rnd(3, g, g, g))
+    mid = torch.tensor([[2], [7]], dtype=torch.int32, device="cuda")
+    mats = [[ibfe.Material(I.NEO_HOOKEAN, (0.5 + 0.1 * k, 100.0)) for k in range(8)],
+            [ibfe.Material(I.NEO_HOOKEAN, (0.9 + 0.2 * k, 70.0)) for k in range(8)]]
+    nodal = torch.empty((3, n, 3, 8), device="cuda")
+    dense = torch.empty((2, n, 3, g, g, g), device="cuda")
+    inst = [dict(shared, mat_id=mid[int(i == n - 1)], mats=mats[int(i == n - 1)], G=nodal[0, i],
+                 U=nodal[1, i], gx=nodal[2, i], f=dense[0, i], gu=dense[1, i]) for i in range(n)]
+    batch = ibfe.Batch(inst)
+    batch.forward()
+    batch.adjoint()
+    gp = batch.gparams()
+    for i in (0, n - 1):
+        d = inst[i]
+        plan = ibfe.Plan(d["conn"], d["X"], d["n"], h, mat_id=d["mat_id"])
+        pos = ibfe.Pos(cell=d["cell"], off=d["off"])
+        G, f, U = ibfe.ib_forward(plan, d["mats"], pos, d["u"])
+        gx, gu, gpi = ibfe.ib_backward(plan, d["mats"], pos, d["u"], G, None, d["gf"], d["gU"])
+        for a, k in ((G, "G"), (f, "f"), (U, "U"), (gx, "gx"), (gu, "gu")):
+            assert torch.equal(a, d[k]), (i, k)
+        assert torch.equal(gpi.cpu(), gp[i])
+    assert torch.count_nonzero(gp[1:n - 1, 2, 0]) == n - 2
