@@ -635,9 +635,10 @@ def ib_plan_profile(plan: Plan, reset: bool = True):
 # ---------------------------------------------------------------------------
 
 def _mats_from(models, params: torch.Tensor):
-    rows = params.tolist()
-    return [Material(m, r[:N_PARAMS[m]], r[9] if len(r) > 9 else 0.0)
-            for m, r in zip(models, rows)]
+    # (a model without a row, or a table that is not two-dimensional: IndexError)
+    rows, active = params.tolist(), params.shape[1] > 9
+    return [Material(m, rows[i][:N_PARAMS[m]], rows[i][9] if active else 0.0)
+            for i, m in enumerate(models)]
 
 
 def _param_grad(gp: torch.Tensor, models, params: torch.Tensor) -> torch.Tensor:
