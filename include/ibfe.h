@@ -271,7 +271,8 @@ ib_status ib_backward(ib_plan* plan, const ib_material* mats, int32_t n_mats, co
  *   [1] FE-force CTAs per SM in ib_forward, 1..5 (its persistent grid leaves
  *       the rest of each SM to the binning and interpolation beside it);
  *   [2] cap on the spreading CTAs per SM, 1..8;
- *   [3] cap on the interpolation CTAs per SM, 1..8.
+ *   [3] cap on the interpolation CTAs per SM, 1..8 (FP64 plans with few points
+ *       interpolate by component, a CTA of which counts three quarters).
  * Defaults {1024, 4, 8, 3} (a cap above the occupancy limit means none).
  * Results do not depend on the tuning for FP32 plans (bitwise); FP64 plans
  * change only in the summation order of the spreading.  get/set are host
