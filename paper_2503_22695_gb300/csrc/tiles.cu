@@ -189,11 +189,14 @@ int classify_blocks(int ntiles) { return (ntiles + kT - 1) / kT; }
 // Accumulation / interpolation in us, items of 1024, 512, 256, 128 points:
 // 115 k points at 128^3 30 / 25, 30 / 18, 32 / 18, 36 / 20; 102 k points of
 // tetrahedra at 104^3 42 / 26, 33 / 20, 38 / 22, 51 / 23; 1.38 M points at
-// 256^3 149 / 110, 158 / 118, 177 / 124, 192 / 132.  FP64: 4 items per SM in
-// steps of 64 (FP64 arithmetic alone takes microseconds per point and SM).
+// 256^3 149 / 110, 158 / 118, 177 / 124, 192 / 132.  FP64: 4 items per SM of a
+// whole GB300 in steps of 64 (FP64 arithmetic alone takes microseconds per point
+// and SM); its sums are grouped by item, so that their bits must not follow from
+// the SMs that a part of the GPU, or another one, has.
+constexpr int kFullSMs = 152;
 int item_size(int precision, int64_t Q, int sms) {
   const int gran = precision == IB_FP64 ? 64 : 128;
-  const int64_t items = precision == IB_FP64 ? 4 * sms : sms + sms / 2;
+  const int64_t items = precision == IB_FP64 ? 4 * kFullSMs : sms + sms / 2;
   const int64_t item = ((Q + items - 1) / items + gran - 1) / gran * gran;
   return (int)(item < gran ? gran : (item > kChunk ? kChunk : item));
 }
