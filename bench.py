@@ -611,7 +611,10 @@ def run_ours(args):
         t_fl, t_st = sum(ms_fl) / len(ms_fl), sum(ms_st) / len(ms_st)
         fluid_line = {
             "grid": [n, n, n], "rho": FLUID_RHO, "mu": FLUID_MU, "dt": FLUID_DT,
-            "solver": "both solves by one Fourier transform of the increment (five launches)",
+            "solver": ("both solves by one Fourier transform of the increment (five launches)"
+                       if fl.solver() == ibfe.IB_SOLVER_DIRECT else
+                       "multigrid V-cycles in one CUDA graph: %d Helmholtz, %d Poisson, %d levels"
+                       % (*fl.cycles(), fl.levels())),
             "fluid_step_ms": t_fl, "cells_per_s": cells / (t_fl * 1e-3),
             "relative_residuals": {"helmholtz": res[0], "poisson": res[1]},
             "ib_step_ms": t_st,

@@ -781,6 +781,12 @@ ib_status ib_fluid_get_cycles(const ib_fluid* fl, int32_t cycles[2]) {
   return IB_OK;
 }
 
+ib_status ib_fluid_get_solver(const ib_fluid* fl, int32_t* solver) {
+  if (!fl || !solver) return IB_ERR_INVALID_ARG;
+  *solver = ibfe::use_direct(fl) ? IB_SOLVER_DIRECT : IB_SOLVER_CYCLES;
+  return IB_OK;
+}
+
 ib_status ib_fluid_levels(const ib_fluid* fl, int32_t* levels) {
   if (!fl || !levels) return IB_ERR_INVALID_ARG;
   *levels = fl->nlev;

@@ -29,6 +29,7 @@ IB_ERR_CAPACITY, IB_ERR_TIMEOUT, IB_ERR_UNSUPPORTED, IB_ERR_INVERTED = 4, 5, 6, 
 IB_NEO_HOOKEAN, IB_FIBRE1, IB_HO, IB_STD_REINF, IB_FIBRE2 = 0, 1, 2, 3, 4
 IB_FP32_SPLIT, IB_FP64, IB_FP32_SPLIT_F32STAB, IB_FP32_SPLIT_DFVOL = 0, 1, 2, 3
 IB_QUAD_GAUSS2, IB_QUAD_NODAL = 0, 1
+IB_SOLVER_CYCLES, IB_SOLVER_DIRECT = 0, 1
 IB_ELEM_HEX8, IB_ELEM_TET4, IB_ELEM_TET10 = 0, 1, 2
 _ELEM_OF_NODES = {8: IB_ELEM_HEX8, 4: IB_ELEM_TET4, 10: IB_ELEM_TET10}
 _NODES_OF_ELEM = {v: k for k, v in _ELEM_OF_NODES.items()}
@@ -111,6 +112,7 @@ def _load():
         "ib_fluid_destroy": [vp],
         "ib_fluid_set_cycles": [vp, i32, i32],
         "ib_fluid_levels": [vp, C.POINTER(i32)],
+        "ib_fluid_get_solver": [vp, C.POINTER(i32)],
         "ib_fluid_get_cycles": [vp, C.POINTER(i32)],
         "ib_fluid_step": [vp, vp, vp, vp, vp, dp, vp],
         "ib_step": [vp, vp, C.POINTER(_Mat), i32, C.POINTER(_Pos), vp, vp, vp, vp, vp, vp],
@@ -268,6 +270,12 @@ class Fluid:
     def levels(self) -> int:
         v = C.c_int32()
         _chk(_lib.ib_fluid_levels(self._h, C.byref(v)), "ib_fluid_levels")
+        return int(v.value)
+
+    def solver(self) -> int:
+        """IB_SOLVER_DIRECT or IB_SOLVER_CYCLES: what the next step runs."""
+        v = C.c_int32()
+        _chk(_lib.ib_fluid_get_solver(self._h, C.byref(v)), "ib_fluid_get_solver")
         return int(v.value)
 
     def cycles(self):

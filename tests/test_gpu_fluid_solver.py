@@ -1,4 +1,5 @@
-"""The fluid solver object: its first step on any stream."""
+"""The fluid solver object: which of the two solvers serves it, its first step
+on any stream."""
 import numpy as np
 import pytest
 
@@ -41,3 +42,20 @@ def test_first_step_on_another_stream(n):
             b, pb, _ = ibfe.ib_fluid_step(fl, ud, fd)
         side.synchronize()
         assert torch.equal(a, b) and torch.equal(pa, pb)
+
+
+def test_solver_of_a_lattice():
+    from paper_2503_22695_gb300 import ibfe
+    for n, fp64, direct in [((32, 32, 32), False, True), ((90, 36, 20), False, True),
+                            ((4, 4, 900), False, True), ((56, 8, 8), False, False),
+                            ((8, 22, 8), False, False), ((4, 4, 1024), False, False),
+                            ((32, 32, 32), True, False)]:
+        fl = ibfe.Fluid(n, 1.0 / n[0], RHO, MU, DT,
+                        precision=ibfe.IB_FP64 if fp64 else ibfe.IB_FP32_SPLIT)
+        which = {True: ibfe.IB_SOLVER_DIRECT, False: ibfe.IB_SOLVER_CYCLES}
+        assert fl.solver() == which[direct], n
+        default = fl.cycles()
+        fl.set_cycles(default[0], default[1] + 1)
+        assert fl.solver() == ibfe.IB_SOLVER_CYCLES
+        fl.set_cycles(*default)
+        assert fl.solver() == which[direct], n
