@@ -507,7 +507,10 @@ double ib_active_tension(double t);
  * example ib_forward) return `code` (default IB_ERR_CUDA) before any work;
  * the name "points" makes every operator that builds the coupling points
  * return it there, with that kernel queued; "gather" every operator that
- * gathers element values to the nodes, at its first gather; "earlier_error"
+ * gathers element values to the nodes, at its first gather; "modes" fails the
+ * allocation of the direct fluid solve's workspace in ib_fluid_create (with
+ * the code of IB_ERR_CAPACITY as a refused one, which leaves the V-cycles);
+ * "earlier_error"
  * fails nothing, but leaves an error of an earlier call with the runtime. */
 ib_status ib_diag_wait_timeout(double ms, void* stream);
 

@@ -62,14 +62,17 @@ void free_plan(ib_plan* p) {
 
 cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
+}  // namespace
+
 // Host-side fault injection for error-path tests: IBFE_FAULT="entry[:code]"
 // makes that C entry point return `code` (default IB_ERR_CUDA) before doing
 // anything; "points" stands for the stage that builds the coupling points,
 // which then fails with its kernel queued, "gather" for the gather from the
 // elements to the nodes, which fails with everything before it queued;
+// "modes" for the allocation of the direct fluid solve's workspace;
 // "earlier_error" leaves an error with the runtime ahead of every call.  Read
 // on every call; no device is touched.
-ib_status injected(const char* entry) {
+ib_status ibfe::injected(const char* entry) {
   const char* spec = std::getenv("IBFE_FAULT");
   if (!spec) return IB_OK;
   const char* colon = std::strchr(spec, ':');
@@ -78,6 +81,8 @@ ib_status injected(const char* entry) {
   const int code = colon ? std::atoi(colon + 1) : (int)IB_ERR_CUDA;
   return code > 0 ? (ib_status)code : IB_ERR_CUDA;
 }
+
+namespace {
 
 bool aligned16(const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; }
 

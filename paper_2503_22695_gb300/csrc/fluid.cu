@@ -742,13 +742,15 @@ ib_status ib_fluid_create(const ib_grid* grid, int32_t precision, double rho, do
     ib_fluid_destroy(fl);
     return IB_ERR_CUDA;
   }
-  // without room for its workspace the V-cycles serve every step
+  // without room for its workspace the V-cycles serve every step; any other
+  // error is the device's, and hiding it would leave a slower solver unasked
   if (precision != IB_FP64 && spectral_supports(fl->n)) {
-    fl->direct = spectral_create(&fl->spec, fl->n, fl->h, rho, mu, dt, fl->cap) == IB_OK;
-    if (!fl->direct) {
-      spectral_destroy(&fl->spec);
-      cudaGetLastError();
+    const ib_status st = spectral_create(&fl->spec, fl->n, fl->h, rho, mu, dt, fl->cap);
+    if (st != IB_OK && st != IB_ERR_CAPACITY) {
+      ib_fluid_destroy(fl);
+      return st;
     }
+    fl->direct = st == IB_OK;
   }
   (void)stream;
   *out = fl;

@@ -46,6 +46,8 @@ cudaError_t chain_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t sme
 // Start of a C entry point that launches: drops an error left by an earlier call;
 // returns the status injected for `entry`, if any (capi.cu).
 ib_status enter(const char* entry);
+// the status injected for a stage within a call (capi.cu)
+ib_status injected(const char* stage);
 
 // Calls f(std::integral_constant<int, kEl>) for the plan's element type.
 template <typename F>

@@ -1014,7 +1014,12 @@ ib_status spectral_create(Spectral* sp, const int n[3], double h, double rho, do
   }
   A.pitch = (n[0] / 2 + 1 + 3) / 4 * 4;  // rows start on 32-byte sectors
   const size_t spec = (sizeof(float2) * 4 * (size_t)n[2] * n[1] * A.pitch + 255) / 256 * 256;
-  if (!ok(cudaMalloc((void**)&A.spec, spec + host.size()))) return IB_ERR_CUDA;
+  if (const ib_status f = injected("modes")) return f;
+  if (const cudaError_t e = cudaMalloc((void**)&A.spec, spec + host.size())) {
+    A.spec = nullptr;
+    cudaGetLastError();
+    return e == cudaErrorMemoryAllocation ? IB_ERR_CAPACITY : IB_ERR_CUDA;
+  }
   char* const t = reinterpret_cast<char*>(A.spec) + spec;  // the tables behind the modes
   // The tables are on the device when the solver is handed out, whatever stream
   // it is first used on.  A plain copy from pageable memory may return with its

@@ -44,6 +44,7 @@ struct Spectral {
 // Lattices the direct solve takes: every length even, at most 1024, with no
 // prime factor above 5.
 bool spectral_supports(const int n[3]);
+// IB_ERR_CAPACITY: no room for the workspace (the caller keeps its V-cycles).
 // up: a stream of the caller's that nothing is queued on (the tables' upload,
 // waited for)
 ib_status spectral_create(Spectral* sp, const int n[3], double h, double rho, double mu,

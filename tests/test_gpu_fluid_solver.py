@@ -59,3 +59,23 @@ def test_solver_of_a_lattice():
         assert fl.solver() == ibfe.IB_SOLVER_CYCLES
         fl.set_cycles(*default)
         assert fl.solver() == which[direct], n
+
+
+def test_only_a_refused_workspace_leaves_the_cycles(monkeypatch):
+    """No room for the direct solve's modes: the V-cycles serve the solver, at the
+    tolerances that test_gpu_fluid states for them.  Any other error is the call's."""
+    import torch
+    from paper_2503_22695_gb300 import ibfe
+    g, u, f = _fields((64, 32, 32), 2)
+    monkeypatch.setenv("IBFE_FAULT", "modes:%d" % ibfe.IB_ERR_CAPACITY)
+    fl = ibfe.Fluid(g.n, g.h, RHO, MU, DT)
+    monkeypatch.setenv("IBFE_FAULT", "modes")
+    with pytest.raises(ibfe.IBError) as e:
+        ibfe.Fluid(g.n, g.h, RHO, MU, DT)
+    assert e.value.code == ibfe.IB_ERR_CUDA
+    monkeypatch.delenv("IBFE_FAULT")
+    assert fl.solver() == ibfe.IB_SOLVER_CYCLES
+    un, p, _ = ibfe.ib_fluid_step(fl, torch.from_numpy(u).cuda(), torch.from_numpy(f).cuda())
+    _, po, uo = OF.fluid_step(u.astype(np.float64), f.astype(np.float64), RHO, MU, DT, g.h)
+    assert rel_l2(np_(un), uo) <= 1e-5
+    assert rel_l2(np_(p), po) <= 2e-5
