@@ -494,6 +494,7 @@ ib_status ib_batch_get_tuning(const ib_batch* b, int32_t tuning[4]) {
 
 ib_status ib_batch_destroy(ib_batch* b) {
   if (!b) return IB_ERR_INVALID_ARG;
+  RelaxedCapture relaxed;
   destroy(b);
   return IB_OK;
 }

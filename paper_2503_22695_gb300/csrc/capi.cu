@@ -533,6 +533,7 @@ extern "C" {
 
 ib_status ib_plan_destroy(ib_plan* plan) {
   if (!plan) return IB_ERR_INVALID_ARG;
+  RelaxedCapture relaxed;
   free_plan(plan);
   return IB_OK;
 }

@@ -759,6 +759,7 @@ ib_status ib_fluid_create(const ib_grid* grid, int32_t precision, double rho, do
 
 ib_status ib_fluid_destroy(ib_fluid* fl) {
   if (!fl) return IB_ERR_INVALID_ARG;
+  ibfe::RelaxedCapture relaxed;
   if (fl->gexec) cudaGraphExecDestroy(fl->gexec);
   if (fl->cap) cudaStreamDestroy(fl->cap);
   spectral_destroy(&fl->spec);

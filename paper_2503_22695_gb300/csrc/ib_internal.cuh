@@ -49,6 +49,18 @@ ib_status enter(const char* entry);
 // the status injected for a stage within a call (capi.cu)
 ib_status injected(const char* stage);
 
+// While it lives, this thread may free memory beside a capture of another stream.
+// The destroy functions run whenever a garbage collector gets to an object, in
+// the middle of a capture that has nothing to do with it as well, which a plain
+// cudaFree would invalidate.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  RelaxedCapture(const RelaxedCapture&) = delete;
+  RelaxedCapture& operator=(const RelaxedCapture&) = delete;
+};
+
 // Calls f(std::integral_constant<int, kEl>) for the plan's element type.
 template <typename F>
 void with_elem(int elem, F&& f) {

@@ -144,3 +144,38 @@ def test_an_earlier_error_is_not_the_next_calls(fp64, monkeypatch):
     monkeypatch.delenv("IBFE_FAULT")
     assert _equal(again, ref)
     assert ibfe.ib_plan_sync_status(c.plan) == ibfe.IB_OK
+
+
+@pytest.mark.parametrize("fp64", [False, True])
+def test_objects_released_during_a_capture(fp64):
+    """Plans, fluid solvers and sweeps that are collected while an unrelated
+    stream is captured do not invalidate the capture."""
+    import torch
+    c = _case(fp64)
+    ibfe = c.ibfe
+    g = c.prob.grid
+    ref = ibfe.ib_spread(c.plan, c.pos, c.G)
+    f = torch.empty_like(ref)
+    other = [_case(fp64)]
+    ibfe.ib_spread(other[0].plan, other[0].pos, other[0].G)
+    fl = ibfe.Fluid(g.n, g.h, 1.0, 0.02, 2e-4,
+                    precision=ibfe.IB_FP64 if fp64 else ibfe.IB_FP32_SPLIT)
+    un = ibfe.ib_fluid_step(fl, c.u)[0]
+    other.append(fl)
+    if not fp64:
+        inst = [dict(conn=c.conn, X=c.X, fibres=c.fib, mat_id=c.mat_id, n=g.n, h=g.h, mats=c.mats,
+                     cell=c.cell, off=c.off, u=c.u, G=torch.empty_like(c.G),
+                     U=torch.empty_like(c.G), f=torch.empty_like(c.u)) for _ in range(2)]
+        other.append(ibfe.Batch(inst))
+        other[-1].forward()
+    del fl
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ibfe.ib_spread(c.plan, c.pos, c.G, f)
+        while other:
+            other.pop()
+        ibfe.ib_interp(c.plan, c.pos, c.u)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(f, ref) and bool(torch.isfinite(un).all())
