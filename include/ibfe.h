@@ -411,9 +411,13 @@ ib_status ib_fluid_destroy(ib_fluid* fluid);
  * step run that many V-cycles, also where the direct solve applies. */
 ib_status ib_fluid_set_cycles(ib_fluid* fluid, int32_t helmholtz_cycles, int32_t poisson_cycles);
 ib_status ib_fluid_get_cycles(const ib_fluid* fluid, int32_t cycles[2]);
-/* The solver that the next step runs. */
+/* The solver that the next step runs; and the choice: IB_SOLVER_CYCLES, V-cycles
+ * at whatever counts are set, the defaults among them; IB_SOLVER_DIRECT (initial
+ * where the direct solve applies, IB_ERR_UNSUPPORTED elsewhere), the direct solve
+ * at the default counts. */
 typedef enum { IB_SOLVER_CYCLES = 0, IB_SOLVER_DIRECT = 1 } ib_fluid_solver;
 ib_status ib_fluid_get_solver(const ib_fluid* fluid, int32_t* solver);
+ib_status ib_fluid_set_solver(ib_fluid* fluid, int32_t solver);
 /* Number of multigrid levels (the finest included). */
 ib_status ib_fluid_levels(const ib_fluid* fluid, int32_t* levels);
 /* One projection step: u_next (may alias u) and p (NULL: kept internally)

@@ -62,6 +62,7 @@ struct ib_fluid {
   int gcyc[2];
   // the direct solve (spectral.cu), where the lattice has one
   bool direct;
+  bool cycles;  // V-cycles were asked for
   ibfe::Spectral spec;
 };
 
@@ -547,10 +548,11 @@ ib_status step_direct(ib_fluid* fl, const void* u, const void* f, void* un, void
 // The direct solve (spectral.cu) replaces the V-cycles wherever the lattice
 // has one and the cycle counts are the defaults: it gives the discrete
 // solution that the cycles approach, to FP32 rounding, in five launches.  A
-// caller who sets other counts asks for that many V-cycles and gets them.
+// caller who sets other counts asks for that many V-cycles and gets them;
+// ib_fluid_set_solver asks for them at the default counts.
 namespace {
 bool use_direct(const ib_fluid* fl) {
-  return fl->direct && fl->cyc_h == kCycH32 && fl->cyc_p == kCycP32;
+  return fl->direct && !fl->cycles && fl->cyc_h == kCycH32 && fl->cyc_p == kCycP32;
 }
 
 // With residuals, u is kept aside (u_next may alias it) and the increment is
@@ -787,6 +789,13 @@ ib_status ib_fluid_get_cycles(const ib_fluid* fl, int32_t cycles[2]) {
 ib_status ib_fluid_get_solver(const ib_fluid* fl, int32_t* solver) {
   if (!fl || !solver) return IB_ERR_INVALID_ARG;
   *solver = ibfe::use_direct(fl) ? IB_SOLVER_DIRECT : IB_SOLVER_CYCLES;
+  return IB_OK;
+}
+
+ib_status ib_fluid_set_solver(ib_fluid* fl, int32_t solver) {
+  if (!fl || (solver != IB_SOLVER_CYCLES && solver != IB_SOLVER_DIRECT)) return IB_ERR_INVALID_ARG;
+  if (solver == IB_SOLVER_DIRECT && !fl->direct) return IB_ERR_UNSUPPORTED;
+  fl->cycles = solver == IB_SOLVER_CYCLES;
   return IB_OK;
 }
 

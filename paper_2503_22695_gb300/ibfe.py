@@ -113,6 +113,7 @@ def _load():
         "ib_fluid_set_cycles": [vp, i32, i32],
         "ib_fluid_levels": [vp, C.POINTER(i32)],
         "ib_fluid_get_solver": [vp, C.POINTER(i32)],
+        "ib_fluid_set_solver": [vp, i32],
         "ib_fluid_get_cycles": [vp, C.POINTER(i32)],
         "ib_fluid_step": [vp, vp, vp, vp, vp, dp, vp],
         "ib_step": [vp, vp, C.POINTER(_Mat), i32, C.POINTER(_Pos), vp, vp, vp, vp, vp, vp],
@@ -277,6 +278,11 @@ class Fluid:
         v = C.c_int32()
         _chk(_lib.ib_fluid_get_solver(self._h, C.byref(v)), "ib_fluid_get_solver")
         return int(v.value)
+
+    def set_solver(self, solver: int):
+        """IB_SOLVER_CYCLES: V-cycles at any counts; IB_SOLVER_DIRECT: the direct
+        solve at the default counts (where the lattice has one)."""
+        _chk(_lib.ib_fluid_set_solver(self._h, int(solver)), "ib_fluid_set_solver")
 
     def cycles(self):
         """[Helmholtz, Poisson] V-cycles per step."""

@@ -79,3 +79,38 @@ def test_only_a_refused_workspace_leaves_the_cycles(monkeypatch):
     _, po, uo = OF.fluid_step(u.astype(np.float64), f.astype(np.float64), RHO, MU, DT, g.h)
     assert rel_l2(np_(un), uo) <= 1e-5
     assert rel_l2(np_(p), po) <= 2e-5
+
+
+@pytest.mark.parametrize("n", [(32, 32, 32), (64, 64, 64), (32, 16, 48), (96, 96, 96)])
+def test_cycles_at_the_default_counts(n):
+    """V-cycles asked for on lattices that have the direct solve, at the
+    tolerances that test_gpu_fluid states for them."""
+    import torch
+    from paper_2503_22695_gb300 import ibfe
+    g, u, f = _fields(n, 100 + n[0] + n[2])
+    ud, fd = torch.from_numpy(u).cuda(), torch.from_numpy(f).cuda()
+    fl = ibfe.Fluid(g.n, g.h, RHO, MU, DT)
+    d, pd, _ = ibfe.ib_fluid_step(fl, ud, fd)
+    fl.set_solver(ibfe.IB_SOLVER_CYCLES)
+    assert fl.solver() == ibfe.IB_SOLVER_CYCLES and fl.cycles() == [2, 6]
+    un, p, res = ibfe.ib_fluid_step(fl, ud, fd, residuals=True)
+    _, po, uo = OF.fluid_step(u.astype(np.float64), f.astype(np.float64), RHO, MU, DT, g.h)
+    assert rel_l2(np_(un), uo) <= 1e-5 and rel_l2(np_(p), po) <= 2e-5
+    assert max(res) <= 1e-5
+    assert not torch.equal(p, pd)
+    fl.set_solver(ibfe.IB_SOLVER_DIRECT)
+    e, pe, _ = ibfe.ib_fluid_step(fl, ud, fd)
+    assert fl.solver() == ibfe.IB_SOLVER_DIRECT and torch.equal(e, d) and torch.equal(pe, pd)
+
+
+def test_solver_choice_is_checked():
+    from paper_2503_22695_gb300 import ibfe
+    for n, prec in (((56, 8, 8), ibfe.IB_FP32_SPLIT), ((16, 16, 16), ibfe.IB_FP64)):
+        fl = ibfe.Fluid(n, 1.0 / n[0], RHO, MU, DT, precision=prec)
+        fl.set_solver(ibfe.IB_SOLVER_CYCLES)
+        with pytest.raises(ibfe.IBError) as e:
+            fl.set_solver(ibfe.IB_SOLVER_DIRECT)
+        assert e.value.code == ibfe.IB_ERR_UNSUPPORTED
+        with pytest.raises(ibfe.IBError) as e:
+            fl.set_solver(2)
+        assert e.value.code == ibfe.IB_ERR_INVALID_ARG
