@@ -114,3 +114,65 @@ def test_solver_choice_is_checked():
         with pytest.raises(ibfe.IBError) as e:
             fl.set_solver(2)
         assert e.value.code == ibfe.IB_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("n", [(56, 8, 8), (8, 22, 8), (56, 56, 56), (28, 56, 56), (104, 104, 104)])
+def test_fp32_cycles_match_the_same_cycles_in_fp64(n):
+    """Lattices that only the V-cycles take, at the default counts: the iterate
+    that FP64 gives at the same counts, to the FP32 rounding floor of
+    test_gpu_fluid's tolerances (the cycles contract errors of the iterate)."""
+    import torch
+    from paper_2503_22695_gb300 import ibfe
+    g, u, f = _fields(n, sum(n))
+    ud, fd = torch.from_numpy(u).cuda(), torch.from_numpy(f).cuda()
+    fl = ibfe.Fluid(g.n, g.h, RHO, MU, DT)
+    assert fl.solver() == ibfe.IB_SOLVER_CYCLES and fl.cycles() == [2, 6]
+    un, p, _ = ibfe.ib_fluid_step(fl, ud, fd)
+    fl64 = ibfe.Fluid(g.n, g.h, RHO, MU, DT, precision=ibfe.IB_FP64)
+    fl64.set_cycles(2, 6)
+    u64, p64, _ = ibfe.ib_fluid_step(fl64, ud.double(), fd.double())
+    assert rel_l2(np_(un), np_(u64)) <= 1e-5
+    assert rel_l2(np_(p), np_(p64)) <= 2e-5
+
+
+@pytest.mark.parametrize("n", [(56, 56, 56), (64, 32, 32)])
+def test_cycles_replayed_and_launched_directly(n):
+    """A step's V-cycles as a graph replay, recaptured for other arrays, in place
+    and as direct launches (with residuals): the same bits."""
+    import torch
+    from paper_2503_22695_gb300 import ibfe
+    g, u, f = _fields(n, 5)
+    ud, fd = torch.from_numpy(u).cuda(), torch.from_numpy(f).cuda()
+    fl = ibfe.Fluid(g.n, g.h, RHO, MU, DT)
+    fl.set_solver(ibfe.IB_SOLVER_CYCLES)
+    a, pa = torch.empty_like(ud), torch.empty_like(ud[0])
+    ibfe.ib_fluid_step(fl, ud, fd, a, pa)
+    ref, pref = a.clone(), pa.clone()
+    a.fill_(float("nan"))
+    pa.fill_(float("nan"))
+    ibfe.ib_fluid_step(fl, ud, fd, a, pa)                    # the graph again
+    assert torch.equal(a, ref) and torch.equal(pa, pref)
+    b, pb, _ = ibfe.ib_fluid_step(fl, ud.clone(), fd.clone())  # other arrays
+    assert torch.equal(b, ref) and torch.equal(pb, pref)
+    uin = ud.clone()
+    c, pc, _ = ibfe.ib_fluid_step(fl, uin, fd, u_next=uin)
+    assert torch.equal(c, ref) and torch.equal(pc, pref)
+    d, pd, res = ibfe.ib_fluid_step(fl, ud, fd, residuals=True)
+    assert torch.equal(d, ref) and torch.equal(pd, pref) and np.isfinite(res).all()
+
+
+@pytest.mark.parametrize("n", [(8, 6, 12), (48, 24, 40), (30, 128, 16), (64, 64, 64)])
+def test_direct_solve_without_viscosity(n):
+    """mu = 0: the stencils' own branch, within the direct solve's bounds."""
+    import torch
+    from paper_2503_22695_gb300 import ibfe
+    import test_gpu_spectral as S
+    g, u, f = S._fields(n, sum(n))
+    fl = ibfe.Fluid(g.n, g.h, S.RHO, 0.0, S.DT)
+    assert fl.solver() == ibfe.IB_SOLVER_DIRECT
+    ud, fd = torch.from_numpy(u).cuda(), torch.from_numpy(f).cuda()
+    us, po, uo = OF.fluid_step(u, f, S.RHO, 0.0, S.DT, g.h)
+    tu, tp = S._bounds(u, us, uo, g.h)
+    un, p, _ = ibfe.ib_fluid_step(fl, ud, fd)
+    assert S._rms(np_(un) - uo) <= tu
+    assert S._rms(np_(p) - po) <= tp
