@@ -555,19 +555,28 @@ bool use_direct(const ib_fluid* fl) {
   return fl->direct && !fl->cycles && fl->cyc_h == kCycH32 && fl->cyc_p == kCycP32;
 }
 
-// With residuals, u is kept aside (u_next may alias it) and the increment is
-// left in the solver's workspace for the residual pass (synchronises s).
+// With residuals, the increment is left in the solver's workspace for the
+// residual pass (synchronises s), which reads u and f as well: the one that
+// u_next overwrites (u in place; the V-cycles also let it be f's array) is kept
+// aside.
 ib_status step_spectral(ib_fluid* fl, const float* u, const float* f, float* un, float* p,
                         double* residuals, cudaStream_t s) {
-  float* u0 = static_cast<float*>(fl->rhs0);
-  const size_t bytes = 3 * sizeof(float) * (size_t)fl->n[0] * fl->n[1] * fl->n[2];
-  if (residuals && !ok(cudaMemcpyAsync(u0, u, bytes, cudaMemcpyDeviceToDevice, s)))
-    return IB_ERR_CUDA;
+  const float *u0 = u, *f0 = f;
+  if (residuals) {
+    const size_t n = 3 * (size_t)fl->n[0] * fl->n[1] * fl->n[2];
+    auto over = [&](const float* a) { return a && a < un + n && un < a + n; };
+    const float* lost = over(u) ? u : (over(f) ? f : nullptr);
+    float* kept = static_cast<float*>(fl->rhs0);
+    if (lost && !ok(cudaMemcpyAsync(kept, lost, sizeof(float) * n, cudaMemcpyDeviceToDevice, s)))
+      return IB_ERR_CUDA;
+    if (lost == u) u0 = kept;
+    if (lost && lost == f) f0 = kept;
+  }
   const ib_status st = spectral_step(&fl->spec, u, f, un, p, residuals != nullptr, s);
   if (st != IB_OK || !residuals) return st;
   constexpr int kCtas = kFluidRedCTAs / 4;
   double* out = fl->red + 4 * kCtas;
-  launch_spectral_resid(&fl->spec, u0, f, p, fl->rho / fl->dt, fl->mu / (fl->h * fl->h),
+  launch_spectral_resid(&fl->spec, u0, f0, p, fl->rho / fl->dt, fl->mu / (fl->h * fl->h),
                         fl->dt / fl->h, fl->red, kCtas, s);
   k_sums_l2<<<1, 256, 0, s>>>(fl->red, kCtas, 4, out, 1.0);
   double r[4] = {0.0, 0.0, 0.0, 0.0};

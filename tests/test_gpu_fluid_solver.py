@@ -176,3 +176,26 @@ def test_direct_solve_without_viscosity(n):
     un, p, _ = ibfe.ib_fluid_step(fl, ud, fd)
     assert S._rms(np_(un) - uo) <= tu
     assert S._rms(np_(p) - po) <= tp
+
+
+@pytest.mark.parametrize("n", [(16, 18, 20), (64, 32, 32)])
+def test_residuals_when_the_step_overwrites_an_input(n):
+    """u_next in u's array, in f's and in its own: the same fields and residuals,
+    by either solver."""
+    import torch
+    from paper_2503_22695_gb300 import ibfe
+    g, u, f = _fields(n, 7)
+    ud, fd = torch.from_numpy(u).cuda(), torch.from_numpy(f).cuda()
+    fl = ibfe.Fluid(g.n, g.h, RHO, MU, DT)
+    for solver in (ibfe.IB_SOLVER_DIRECT, ibfe.IB_SOLVER_CYCLES):
+        fl.set_solver(solver)
+        ref, pref, res = ibfe.ib_fluid_step(fl, ud, fd, residuals=True)
+        assert res[0] <= 1e-5 and res[1] <= 1e-5
+        for name in ("u", "f", "both"):
+            a, b = ud.clone(), fd.clone()
+            if name == "both":
+                b = a
+                ref, pref, res = ibfe.ib_fluid_step(fl, ud, ud, residuals=True)
+            un, p, r = ibfe.ib_fluid_step(fl, a, b, u_next=a if name == "u" else b, residuals=True)
+            assert torch.equal(un, ref) and torch.equal(p, pref), (solver, name)
+            assert list(r) == list(res), (solver, name)
