@@ -440,13 +440,17 @@ __device__ __forceinline__ void fx_stage(float4* rec, int part, bool store, cons
 // source tiles (each tile's blocks summed into its first block by the
 // accumulation kernel) in the fixed order (oz, oy, ox), aligned to the
 // destination tile's exponent k_ref (in units of 2^-(k+11)), and is rounded
-// once.  With k'_s = k_s + 11 and m_s = ceil(n_s / 512) for source s (n_s
-// points: m_s bounds its work items under any tuning, whose items hold 512
-// to 1024 points),
+// once.  With k'_s = k_s + 11 and m_s = ceil(n_s / 512) for source s of n_s
+// points,
 //   k_ref = min(max_s k'_s, min_s (k'_s + 17 - ceil_log2(m_s))),
 // so a source sum (below m_s 2^42) shifted left by k_ref - k'_s stays below
 // 2^59 and eight of them below 2^62; a source with k'_s > k_ref is shifted
-// right (floor).  k_ref, like k_s, does not depend on the tuning.  The conversion splits |S| into two 32-bit halves,
+// right (floor).  The bound on a source sum follows from its tile's points
+// alone, however they are cut into work items: a contribution is at most
+// 2^(30 - L), L = ceil_log2(min(n_s, 1024)), in units of 2^-k, so that n_s of
+// them add up to at most ceil(n_s / 1024) 2^30, in units of 2^-(k+11) with
+// each one's rounding to ceil(n_s / 1024) 2^41 + n_s / 2.  k_ref, like k_s, does
+// not depend on the tuning.  The conversion splits |S| into two 32-bit halves,
 // each converted exactly rounded, joined by one fma: within one unit in the
 // last place, the same bits for the same integers.
 __device__ __forceinline__ float fx_to_float(long long S, float out_scale) {
@@ -523,7 +527,7 @@ __global__ void __launch_bounds__(kFxThreads, 1024 / kFxThreads)  // 64 register
     const int tile = it.tile;
     const TileGeo geo = tile_geo<kPacked>(A.g, A.inst, A.tile_inst, tile);
     const int s = it.begin, e = s + it.n;
-    // warp w takes the groups starting at s + kFxGroup (w + 8 j)
+    // warp w takes the groups starting at s + kFxGroup (w + kFxWarps j)
     FxRaw raw = {0, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
     int g0 = s + warp * kFxGroup;
     if (stager && g0 + pt < e) fx_fetch(A, g0 + pt, raw);
@@ -640,8 +644,8 @@ __global__ void __launch_bounds__(kMT, 4) k_spread_merge_fx(SpreadArgs<float> A)
     const TileGeo geo = tile_geo<kPacked>(A.g, A.inst, A.tile_inst, tile);
     int tx, ty, tz;
     tile_coords(geo, tile, tx, ty, tz);
-    // (first block slot or -1, exponent k + 11, bound on the work items under
-    // any tuning, items) of each source
+    // (first block slot or -1, exponent k + 11, m_s, 1 if it holds points) of
+    // each source
     int4 r = make_int4(-1, 0, 0, 0);
     if (lane < 27) {
       const int t = tile_of(tx + lane % 3 - 1, ty + (lane / 3) % 3 - 1, tz + lane / 9 - 1, geo);
