@@ -503,7 +503,8 @@ __device__ __forceinline__ void prefetch_rows(const void* g, int bytes) {
 // The lines a warp of a CTA of `threads` threads takes are first_line(warp),
 // and from there every (threads / 32)-th.  CTAs are multiples of 16 threads (a
 // column each per place): the half warp that some end in takes no line, as the
-// full warps take them all.
+// full warps take them all.  (The threads are read from the launch: with the
+// compile-time number in the kernels' line loops 256^3 610 -> 624 us.)
 __host__ __device__ constexpr int first_line(int warp, int threads) {
   return warp < threads / 32 ? warp : kXL;
 }
@@ -633,7 +634,7 @@ __global__ void __launch_bounds__(cta_threads<N, 0>(), ctas_at_48(cta_threads<N,
   //   2 a_k = z_k + conj z_{n-k},  2 b_k = -i (z_k - conj z_{n-k})
   // (the factor 2 is in inv_n)
   const int nx = n0 / 2 + 1;
-  const int lane = threadIdx.x & 31, threads = N > 0 ? cta_threads<N, 0>() : (int)blockDim.x;
+  const int lane = threadIdx.x & 31, threads = (int)blockDim.x;
   for (int l = first_line(threadIdx.x >> 5, threads); l < 4 * np; l += threads / 32) {
     float2* o = A.spec + ((int64_t)((l & 3) * n2 + k) * n1 + 2 * (jp0 + (l >> 2))) * A.pitch;
     const float2* zl = z + l;
@@ -800,7 +801,7 @@ __global__ void __launch_bounds__(cta_threads<N, 0>(), ctas_at_48(cta_threads<N,
   if (threadIdx.x < 3)
     prefetch_rows(u + threadIdx.x * cells + (k * n1 + 2 * jp0) * n0, sizeof(float) * 2 * np * n0);
   // a warp takes a line, four groups of 32 modes of both rows in flight
-  const int lane = threadIdx.x & 31, threads = N > 0 ? cta_threads<N, 0>() : (int)blockDim.x;
+  const int lane = threadIdx.x & 31, threads = (int)blockDim.x;
   for (int l = first_line(threadIdx.x >> 5, threads); l < kXL; l += threads / 32) {
     const bool on = l < 4 * np;
     const float2* g =
