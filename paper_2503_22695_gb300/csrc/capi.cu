@@ -71,9 +71,10 @@ cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 // elements to the nodes, which fails with everything before it queued;
 // "modes" for the allocation of the direct fluid solve's workspace;
 // "earlier_error" leaves an error with the runtime ahead of every call.  Read
-// on every call; no device is touched.
+// once per call (enter); no device is touched.
+static thread_local const char* fault_spec;
 ib_status ibfe::injected(const char* entry) {
-  const char* spec = std::getenv("IBFE_FAULT");
+  const char* spec = fault_spec;
   if (!spec) return IB_OK;
   const char* colon = std::strchr(spec, ':');
   const size_t n = colon ? (size_t)(colon - spec) : std::strlen(spec);
@@ -139,11 +140,11 @@ void prof_flush(ib_plan* p) {
 // refused allocation, a failed capture): that is not this call's error, and
 // taking it for one would end the call half-way.
 ib_status ibfe::enter(const char* entry) {
-  if (const char* spec = std::getenv("IBFE_FAULT"))
-    if (!std::strcmp(spec, "earlier_error")) {  // an error of the host API, refused as an argument
-      int v;
-      cudaDeviceGetAttribute(&v, cudaDevAttrWarpSize, -1);
-    }
+  fault_spec = std::getenv("IBFE_FAULT");
+  if (fault_spec && !std::strcmp(fault_spec, "earlier_error")) {
+    int v;  // an error of the host API: an argument it refuses
+    cudaDeviceGetAttribute(&v, cudaDevAttrWarpSize, -1);
+  }
   cudaGetLastError();
   return injected(entry);
 }
