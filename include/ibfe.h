@@ -380,7 +380,8 @@ ib_status ib_batch_destroy(ib_batch* batch);
  * FP32, lattices whose lengths are even, at most 1024 and have no prime
  * factor above 5 (n2 at most 900), at the default cycle counts: both solves
  * directly, by one discrete Fourier transform of the increment
- * u^{n+1} - u^n (five launches).  Otherwise: geometric multigrid V-cycles
+ * u^{n+1} - u^n (five launches; the sums over the lattice of f + mu Lap_h u and
+ * h div_h u must be FP32 numbers, which holds below 3e38 / (n0 n1 n2)).  Otherwise: geometric multigrid V-cycles
  * (red-black Gauss-Seidel, 2 pre- and 2
  * post-sweeps; levels halve every dimension while all are even, none is
  * below 4 and the largest exceeds 8; the coarsest is solved in one CTA's
@@ -400,7 +401,7 @@ typedef struct ib_fluid ib_fluid;
  * odd size or a coarsest level above 8192 cells, IB_ERR_CAPACITY for
  * 3 n0 n1 n2 >= 2^31) with density rho > 0,
  * viscosity mu >= 0 and time step dt > 0.  Allocates its multigrid hierarchy
- * (about 1.6 field volumes) and, where the direct solve applies, its modes
+ * (about 2 field volumes) and, where the direct solve applies, its modes
  * (1.4 field volumes) on the current device; without room for the modes every
  * step runs V-cycles. */
 ib_status ib_fluid_create(const ib_grid* grid, int32_t precision, double rho, double mu,

@@ -38,11 +38,11 @@
 // (171 -> 163), the y transforms' lines one wave of CTAs ahead (106 -> 91).  A wave ahead for k_spec_rhs (171 -> 204), the solve (158 -> 168)
 // and k_spec_out's modes (140 -> 159) costs more than it hides.
 //
-// Measured on GB300 (us; V-cycles of fluid.cu before, this after): 32^3 step
-// 632 -> 30, 192^3 3416 -> 285, 256^3 6550 -> 640.  At 256^3 the five kernels
-// take 162, 90, 153, 97 and 137 us for 0.67, 0.54, 0.54, 0.54 and 0.74 GB:
-// 4.1, 6.0, 3.5, 5.6 and 5.4 TB/s; k_spec_rhs and the solve issue on 56 and
-// 58% of their cycles beside their loads' latency (bank conflicts and L1
+// Measured on GB300 (us; V-cycles of fluid.cu before, this after, steps back to
+// back): 32^3 632 -> 22, 192^3 3416 -> 284, 256^3 6550 -> 610.  At 256^3 the five
+// kernels take 164, 83, 151, 83 and 133 us (ncu) for 0.64, 0.50, 0.50, 0.50 and
+// 0.69 GB: 3.9, 6.0, 3.3, 6.0 and 5.2 TB/s; k_spec_rhs and the solve issue on 56
+// and 58% of their cycles beside their loads' latency (bank conflicts and L1
 // requests taken out of k_spec_rhs change nothing).  Choices measured before
 // the lengths were compiled in: x lines use radices up to 8 (48 registers, 5
 // CTAs per SM: 184 against 250 us with radix 16 for k_spec_out); y lines up to
